@@ -17,6 +17,10 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libnanodisk.so")
 SOURCES = ["nd_fused_f32.cu", "nd_fused_f64.cu", "nd_glob_f32.cu", "nd_glob_f64.cu", "nd_dispatch.cu", "nd_aux.cu", "nd_api.cu", "nd_noalloc.cu", "nd_spectra.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
+# The stepping, relaxation and field kernels write their fused multiply-adds
+# out (fm in nd_common.cuh): without contraction by the compiler every
+# schedule of a step rounds alike, whichever kernel it is inlined into.
+NO_CONTRACT = {"nd_fused_f32.cu", "nd_fused_f64.cu", "nd_glob_f32.cu", "nd_glob_f64.cu", "nd_noalloc.cu"}
 
 
 def nvcc() -> str:
@@ -52,7 +56,8 @@ def build(force: bool = False, verbose_ptxas: bool = False, jobs: int | None = N
 
     def one(src):
         obj = os.path.join(BUILD, src.replace(".cu", ".o"))
-        cmd = [cc] + _flags(verbose_ptxas) + ["-c", os.path.join(CSRC, src), "-o", obj]
+        exact = ["-fmad=false"] if src in NO_CONTRACT else []
+        cmd = [cc] + _flags(verbose_ptxas) + exact + ["-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed on {src}:\n{r.stderr}")

@@ -74,12 +74,17 @@ struct SizeClass {
     bool fused_fp64 = false;   // fused kernel in FP64 (energy)
     size_t smem_main = 0, smem_fp64 = 0;
     size_t smem_wbuf = 0;      // fused Heun with the normals kept in shared memory (0: does not fit)
-    int plan[2] = {-1, -1};    // stepping plan for RK4 / Heun: -1 default, 0..2 fused variant, kPlanGlobal, kPlanCluster
+    int plan[2] = {-1, -1};    // stepping plan for RK4 / Heun: -1 default (default_plan), 0..2 fused variant, kPlanGlobal, kPlanCluster
     // time-sliced schedule, cached per (mode, n_steps)
     SegmentHost *segs_d = nullptr;
     int *seg_off_d = nullptr;
     int seg_mode = -1, seg_ncta = 0;
     long long seg_nsteps = -1;
+    int *cflags_d = nullptr;   // cluster schedules: hand-over flags of the replicas, then the ticket counter
+    // resident clusters per (RK4 / Heun, 8 / 16 CTAs) and the plan the default
+    // stands for per method: -1 not yet looked up
+    mutable int max_clusters[2][2] = {{-1, -1}, {-1, -1}};
+    mutable int default_plan[2] = {-1, -1};
 };
 
 constexpr int kPlanGlobal = 100;
@@ -271,13 +276,110 @@ static void build_segments(int Bc, long long n, int ncta, std::vector<SegmentHos
     off[ncta] = (int)segs.size();
 }
 
-// Whether a cluster plan of nc CTAs per replica exists for the class: the
-// size has one, its shared memory fits, and the GPU can hold such a cluster.
+static int ensure_alloc(void **p, size_t bytes)
+{
+    if (*p) return ND_OK;
+    ND_CUDA(cudaMalloc(p, bytes));
+    return ND_OK;
+}
+
+// Clusters of nc CTAs of the class that can be resident at once: 0 where the
+// size has no such plan, its shared memory does not fit, or the GPU cannot hold
+// such a cluster.
+static int cluster_slots(const nd_handle *h, const SizeClass &c, int prec, bool heun, int nc)
+{
+    int &n = c.max_clusters[heun ? 1 : 0][nc == 16 ? 1 : 0];
+    if (n < 0) {
+        const size_t sm = cluster_smem(c.P, prec, c.maxD, c.maxDpad, heun, nc);
+        n = (sm == (size_t)-1 || sm + 1024 > h->max_smem) ? 0
+                                                          : cluster_max_active(c.P, prec, c.maxD, c.maxDpad, heun, nc);
+    }
+    return n;
+}
 static bool cluster_plan_fits(const nd_handle *h, const SizeClass &c, int prec, bool heun, int nc)
 {
-    const size_t sm = cluster_smem(c.P, prec, c.maxD, c.maxDpad, heun, nc);
-    if (sm == (size_t)-1 || sm + 1024 > h->max_smem) return false;
-    return cluster_max_active(c.P, prec, c.maxD, c.maxDpad, heun, nc) > 0;
+    return cluster_slots(h, c, prec, heun, nc) > 0;
+}
+
+// Microseconds of one field evaluation with its epilogue (Heun, one replica
+// per CTA or cluster): the one-CTA kernel (P >= 192, and FP64 above 64: the
+// global path with up to 16 replicas), a cluster of 8 and of 16 CTAs.
+// Measured at D = 7, 14, 30, 50 (FP64 the same), 81 and 100; 0: no such plan.
+struct EvalTime { int P; float one, c8, c16; };
+static const EvalTime kEval32[] = {{16, 3.6f, 0, 0},        {32, 5.1f, 4.6f, 4.4f}, {64, 7.0f, 4.0f, 4.0f},
+                                   {128, 20.5f, 6.1f, 5.3f}, {192, 30.f, 0, 10.2f},  {256, 28.f, 0, 11.5f}};
+static const EvalTime kEval64[] = {{16, 23.8f, 16.9f, 0}, {32, 50.f, 36.f, 33.f}, {64, 130.f, 36.f, 36.f},
+                                   {128, 282.f, 94.f, 70.f}};
+
+// The plan that the default (-1) stands for.  Few replicas leave most SMs
+// idle with one CTA each, so they take a cluster plan while its rounds, with
+// the replicas time-sliced over the clusters the GPU holds (about 15 of 8
+// CTAs, 7 of 16; 8% for the hand-overs), cost less than one round of the
+// one-CTA kernel: up to 7 replicas 16 CTAs at P = 128 (5.3 against 20.5 us
+// per evaluation), up to 47 eight (6.1 us per 15 replicas); at P = 64 up to
+// 24 (4.0 against 7.0 us).  Every plan of a size rounds alike (at P = 128 all
+// but the global path), so the choice changes no trajectory.  The classes of
+// one handle step side by side: they take clusters only if all of them fit
+// on the GPU together.
+static int default_plan(const nd_handle *h, const SizeClass &c0, int mode)
+{
+    const int slot = mode == M_RK4 ? 0 : 1;
+    if (c0.default_plan[slot] >= 0) return c0.default_plan[slot];
+    const int prec = h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32;
+    std::vector<int> pick;
+    int sms = 0;
+    for (const auto &c : h->classes) {
+        const int plain = c.fused_main ? 0 : kPlanGlobal, B = (int)c.reps.size();
+        const EvalTime *e = nullptr;
+        if (prec == ND_PREC_FP64) { for (const auto &t : kEval64) if (t.P == c.P) e = &t; }
+        else                      { for (const auto &t : kEval32) if (t.P == c.P) e = &t; }
+        int best = plain, best_nc = 0;
+        float t = e ? e->one : 0.f;
+        for (int nc : {8, 16}) {
+            const float per = !e ? 0.f : nc == 8 ? e->c8 : e->c16;
+            if (per == 0.f || per >= t) continue;
+            if (B > 64) continue;   // (never the faster one; spares the query)
+            const int slots = cluster_slots(h, c, prec, mode == M_HEUN, nc);
+            if (slots < 1) continue;
+            const float rounds = B <= slots ? 1.f : 1.08f * (float)B / (float)slots;
+            if (per * rounds < t) {
+                t = per * rounds;
+                best = nc == 8 ? kPlanCluster : kPlanCluster16;
+                best_nc = nc * std::min(B, slots);
+            }
+        }
+        pick.push_back(best);
+        sms += best_nc ? best_nc : plain == 0 ? B : h->n_sm;
+    }
+    const bool together = h->classes.size() == 1 || sms <= h->n_sm;
+    for (size_t k = 0; k < h->classes.size(); ++k) {
+        const auto &c = h->classes[k];
+        c.default_plan[slot] = together ? pick[k] : c.fused_main ? 0 : kPlanGlobal;
+    }
+    return c0.default_plan[slot];
+}
+
+// The time-sliced schedule of a class's replicas over nslots CTAs or clusters,
+// cached per (mode, n_steps, slots).
+static int class_segments(SizeClass &c, int mode, long long nsteps, int nslots)
+{
+    if (c.seg_mode == mode && c.seg_nsteps == nsteps && c.seg_ncta == nslots) return ND_OK;
+    std::vector<SegmentHost> segs;
+    std::vector<int> off;
+    build_segments((int)c.reps.size(), nsteps, nslots, segs, off);
+    for (auto &g : segs) g.rep = c.reps[g.rep];   // segments refer to positions in c.reps
+    cudaFree(c.segs_d);
+    cudaFree(c.seg_off_d);
+    c.segs_d = nullptr;
+    c.seg_off_d = nullptr;
+    ND_CUDA(cudaMalloc(&c.segs_d, sizeof(SegmentHost) * segs.size()));
+    ND_CUDA(cudaMalloc(&c.seg_off_d, sizeof(int) * off.size()));
+    ND_CUDA(cudaMemcpy(c.segs_d, segs.data(), sizeof(SegmentHost) * segs.size(), cudaMemcpyHostToDevice));
+    ND_CUDA(cudaMemcpy(c.seg_off_d, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice));
+    c.seg_mode = mode;
+    c.seg_nsteps = nsteps;
+    c.seg_ncta = nslots;
+    return ND_OK;
 }
 
 // Run one mode over all replicas.  fp64 selects the FP64 kernels (with y a
@@ -324,7 +426,8 @@ static int run_mode(nd_handle *h, int mode, bool fp64, void *y, void *out, long 
         int variant = 0;
         int cluster_nc = 0;
         if (stepping) {
-            const int pl = c.plan[mode == M_RK4 ? 0 : 1];
+            int pl = c.plan[mode == M_RK4 ? 0 : 1];
+            if (pl == -1) pl = default_plan(h, c, mode);
             if (pl == kPlanGlobal) fused = false;
             else if (plan_cluster_nc(pl)) cluster_nc = plan_cluster_nc(pl);
             else if (pl > 0) variant = pl;
@@ -333,6 +436,20 @@ static int run_mode(nd_handle *h, int mode, bool fp64, void *y, void *out, long 
         if (cluster_nc) {
             a.use_wbuf = mode == M_HEUN ? 1 : 0;
             a.status = h->status_d;
+            const int slots = cluster_slots(h, c, prec, mode == M_HEUN, cluster_nc);
+            const int Bc = (int)c.reps.size(), B = (int)h->rep_disk.size();
+            if (Bc > slots && nsteps >= 2) {
+                // more replicas than resident clusters: every cluster steps for
+                // the same time instead of in waves of whole replicas
+                if (int rc = class_segments(c, mode, nsteps, slots)) return rc;
+                if (int rc = ensure_alloc((void **)&c.cflags_d, sizeof(int) * (B + 1))) return rc;
+                ND_CUDA(cudaMemsetAsync(c.cflags_d, 0, sizeof(int) * (B + 1), st));
+                a.segs = c.segs_d;
+                a.seg_off = c.seg_off_d;
+                a.flags = c.cflags_d;
+                a.n_rep = B;
+                a.ncta = slots;
+            }
             ND_CUDA(launch_cluster(c.P, prec, a, c.maxD, c.maxDpad, cluster_nc));
         } else if (fused) {
             a.smem = fp64 ? c.smem_fp64 : c.smem_main;
@@ -347,28 +464,11 @@ static int run_mode(nd_handle *h, int mode, bool fp64, void *y, void *out, long 
                 }
             }
             if ((mode == M_HEUN || mode == M_RK4) && !fp64 && nsteps >= 2) {
-                // localise the replicas' indices to the class: segments refer to positions in c.reps
                 const int per_sm = fused_blocks_per_sm(c.P, prec, mode, a.smem, variant);
                 const int ncta = per_sm * h->n_sm;
                 const int Bc = (int)c.reps.size();
                 if (per_sm > 0 && Bc > ncta) {
-                    if (c.seg_mode != mode || c.seg_nsteps != nsteps || c.seg_ncta != ncta) {
-                        std::vector<SegmentHost> segs;
-                        std::vector<int> off;
-                        build_segments(Bc, nsteps, ncta, segs, off);
-                        for (auto &g : segs) g.rep = c.reps[g.rep];
-                        cudaFree(c.segs_d);
-                        cudaFree(c.seg_off_d);
-                        c.segs_d = nullptr;
-                        c.seg_off_d = nullptr;
-                        ND_CUDA(cudaMalloc(&c.segs_d, sizeof(SegmentHost) * segs.size()));
-                        ND_CUDA(cudaMalloc(&c.seg_off_d, sizeof(int) * off.size()));
-                        ND_CUDA(cudaMemcpy(c.segs_d, segs.data(), sizeof(SegmentHost) * segs.size(), cudaMemcpyHostToDevice));
-                        ND_CUDA(cudaMemcpy(c.seg_off_d, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice));
-                        c.seg_mode = mode;
-                        c.seg_nsteps = nsteps;
-                        c.seg_ncta = ncta;
-                    }
+                    if (int rc = class_segments(c, mode, nsteps, ncta)) return rc;
                     ND_CUDA(cudaMemsetAsync(h->flags_d, 0, sizeof(int) * h->rep_disk.size(), st));
                     a.segs = c.segs_d;
                     a.seg_off = c.seg_off_d;
@@ -390,13 +490,6 @@ static int run_mode(nd_handle *h, int mode, bool fp64, void *y, void *out, long 
     }
     if (concurrent)
         for (size_t k = 0; k < h->side.size(); ++k) ND_CUDA(cudaStreamWaitEvent(st0, h->join_ev[k], 0));
-    return ND_OK;
-}
-
-static int ensure_alloc(void **p, size_t bytes)
-{
-    if (*p) return ND_OK;
-    ND_CUDA(cudaMalloc(p, bytes));
     return ND_OK;
 }
 
@@ -635,7 +728,7 @@ void nd_destroy(nd_handle *h)
     for (auto st2 : h->side) { cudaStreamSynchronize(st2); cudaStreamDestroy(st2); }
     for (auto e2 : h->join_ev) cudaEventDestroy(e2);
     if (h->fork_ev) cudaEventDestroy(h->fork_ev);
-    for (auto &c : h->classes) { cudaFree(c.work_d); cudaFree(c.segs_d); cudaFree(c.seg_off_d); }
+    for (auto &c : h->classes) { cudaFree(c.work_d); cudaFree(c.segs_d); cudaFree(c.seg_off_d); cudaFree(c.cflags_d); }
     cudaFree(h->flags_d);
     cudaFree(h->status_d);
     for (auto &kv : h->tw64) cudaFree(kv.second);
@@ -1479,7 +1572,7 @@ static int tune_items(std::vector<TuneItem> &items, double dt, long long n_steps
             // descent between near-equal plans
             std::vector<int> cands = plan_candidates(it.h, c, it.mode);
             int cur = c.plan[it.slot];
-            if (cur == -1) cur = c.fused_main ? 0 : kPlanGlobal;   // what the default runs
+            if (cur == -1) cur = default_plan(it.h, c, it.mode);   // what the default runs
             const auto pos = std::find(cands.begin(), cands.end(), cur);
             if (pos != cands.end()) std::rotate(cands.begin(), pos, pos + 1);
             float best_ms = 1e30f;
@@ -1607,18 +1700,19 @@ int nd_plan_info(const nd_handle *h, int cls, int *P, int *n_replicas, int *plan
     if (int rc = check_handle(h)) return rc;
     if (cls < 0 || cls >= (int)h->classes.size()) return fail(ND_ERR_ARG, "no such size class");
     const SizeClass &c = h->classes[cls];
-    auto threads = [&](int pl) {
+    auto threads = [&](int pl, int mode) {
+        if (pl == -1) pl = default_plan(h, c, mode);
         if (pl == kPlanGlobal) return 0;
         if (plan_cluster_nc(pl)) return cluster_cta_threads(c.P) * plan_cluster_nc(pl);   // threads of the cluster
         if (!c.fused_main) return 0;
-        return fused_variant_threads(c.P, pl < 0 ? 0 : pl);
+        return fused_variant_threads(c.P, pl);
     };
     if (P) *P = c.P;
     if (n_replicas) *n_replicas = (int)c.reps.size();
     if (plan_rk4) *plan_rk4 = c.plan[0];
     if (plan_heun) *plan_heun = c.plan[1];
-    if (threads_rk4) *threads_rk4 = threads(c.plan[0]);
-    if (threads_heun) *threads_heun = threads(c.plan[1]);
+    if (threads_rk4) *threads_rk4 = threads(c.plan[0], M_RK4);
+    if (threads_heun) *threads_heun = threads(c.plan[1], M_HEUN);
     return ND_OK;
 }
 

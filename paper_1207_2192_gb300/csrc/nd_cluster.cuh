@@ -94,9 +94,8 @@ __device__ __forceinline__ void cluster_packed_scale(cplx<T> *v, const T *s0t, c
         const T h = T(0.5);
         cplx<T> F0 = {h * (v[o].x + w.x), h * (v[o].y - w.y)};
         cplx<T> F1 = {h * (v[o].y + w.y), -h * (v[o].x - w.x)};
-        F0 = cscale(F0, s0t[kyr]);
-        F1 = cscale(F1, s1t[kyr]);
-        v[o] = {F0.x - F1.y, F0.y + F1.x};
+        const T s0 = s0t[kyr], s1 = s1t[kyr];
+        v[o] = {fm(F0.x, s0, -(F1.y * s1)), fm(F0.y, s0, F1.x * s1)};   // s0 F0 + i s1 F1
     }
     __syncwarp(gmask);
 }
@@ -155,11 +154,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity)
     return false;
 }
 
-template <int P, typename T, int MODE, int NC>
+// Without SEG, one replica per cluster for the whole launch (compiled apart:
+// the schedule's loop around the steps cost 5-10% of each step).  With SEG
+// (more replicas than clusters fit on the GPU), a time-sliced schedule: the cluster
+// with ticket i (tickets count the clusters in the order they start, so every
+// cluster that another one waits for is already running) runs the segments
+// segs[seg_off[i] .. seg_off[i+1]), passing replicas on through flags.
+template <int P, typename T, int MODE, int NC, bool SEG>
 __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     k_cluster(const Replica *__restrict__ reps, const int *__restrict__ work, T *__restrict__ ybase,
-              const cplx<T> *__restrict__ twP, long long nsteps, unsigned long long step_base, int use_wbuf,
-              unsigned *__restrict__ status)
+              const cplx<T> *__restrict__ twP, long long nsteps_all, unsigned long long step_base, int use_wbuf,
+              unsigned *__restrict__ status, const Segment *__restrict__ segs, const int *__restrict__ seg_off,
+              int *__restrict__ flags, int *__restrict__ ticket)
 {
     using Gm = FFTGeom<P>;
     using CG = ClusterGeom<P, T, NC>;
@@ -171,16 +177,40 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     extern __shared__ __align__(16) unsigned char smem[];
     const int tid = threadIdx.x;
     GroupId<P> gid(tid);
-    const int ridx = work[blockIdx.x / NC];
-    const Replica &r = reps[ridx];
+    unsigned long long *mbars = reinterpret_cast<unsigned long long *>(smem);   // [0] columns, [1] rows
+    const uint32_t mb_col = smem_addr(mbars), mb_row = smem_addr(mbars + 1);
+    cplx<T> *tw = reinterpret_cast<cplx<T> *>(smem + 16);
+    __shared__ int bcast;   // rank 0's: the cluster's ticket, then whether a hand-over arrived
+    load_twiddles<P>(tw, twP, tid, NT);
+    if (tid == 0) {
+        mbar_init(mb_col, 1);
+        mbar_init(mb_row, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if (SEG && rank == 0) bcast = atomicAdd(ticket, 1);
+    }
+    cluster.sync();   // every CTA runs, with its barriers initialised, before the first remote store
+    const int slot = SEG ? *cluster.map_shared_rank(&bcast, 0) : 0;
+    uint32_t phase = 0;
+    bool bailed = false;   // this thread's wait ran out once: it skips every later wait
+    const int sg_begin = SEG ? seg_off[slot] : 0, sg_end = SEG ? seg_off[slot + 1] : 1;
+    for (int sg = sg_begin; sg < sg_end; ++sg) {
+    const Segment seg = SEG ? segs[sg] : Segment{work[blockIdx.x / NC], 0, 0, 0, 0, nsteps_all};
+    const long long nsteps = seg.nsteps;
+    const Replica &r = reps[seg.rep];
+    if (SEG) {   // (the same for every CTA of the cluster)
+        cluster.sync();   // the ticket is read; the previous segment's rows and columns are no longer used
+        if (rank == 0 && tid == 0) {
+            bcast = seg.wait ? (int)wait_flag(flags + seg.rep) : 1;
+            if (!bcast) atomicOr(status, ND_DEV_TIMEOUT);
+        }
+        cluster.sync();
+        if (!*cluster.map_shared_rank(&bcast, 0)) break;
+    }
     const int D = r.D, Dpad = r.Dpad, rpc = cluster_rows(D, NC);
     const int ylo = rank * rpc, nloc = max(0, min(D, ylo + rpc) - ylo);   // this CTA's rows [ylo, ylo + nloc)
     const long long lcs = (long long)rpc * RS;                            // local spectrum component stride
     const long long lms = (long long)rpc * Dpad;                          // local state component stride
     const long long ms_s = (long long)D * Dpad;                           // global state component stride
-    unsigned long long *mbars = reinterpret_cast<unsigned long long *>(smem);   // [0] columns, [1] rows
-    const uint32_t mb_col = smem_addr(mbars), mb_row = smem_addr(mbars + 1);
-    cplx<T> *tw = reinterpret_cast<cplx<T> *>(smem + 16);
     cplx<T> *colbuf = tw + R1 * G;                                        // [3][P/2][SW]
     cplx<T> *spec = colbuf + 3 * (P / 2) * SW;                            // [3][rpc][RS]
     cplx<T> *scratch = spec + 3 * lcs;
@@ -190,7 +220,6 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     T *wl = use_wbuf ? accl + 3 * lms : nullptr;
     int *crange = reinterpret_cast<int *>((use_wbuf ? wl : accl) + 3 * lms);
     cplx<T> *scr = scratch + gid.group * Gm::SCRATCH;
-    load_twiddles<P>(tw, twP, tid, NT);
     const V3Ptr<T> ms{msl, lms}, wb{wl, lms}, ynv{ynl, lms}, accv{accl, lms}, none{nullptr, 0};
     const V3Ptr<T> yg{ybase + r.state_off, ms_s};
     // the state of the CTA's rows (zero outside the disk)
@@ -232,12 +261,6 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     const bool ctask = gid.group < 3 * SPC;   // groups beyond 3 SPC idle in the column pass
     const int kslot = rank * SPC + cj;
     const bool packed = ctask && kslot == 0;
-    if (tid == 0) {
-        mbar_init(mb_col, 1);
-        mbar_init(mb_row, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    bool bailed = false;   // this thread's wait ran out once: it skips every later wait
     // bytes each CTA receives from the other CTAs per stage (what it sends to
     // itself goes by plain stores, made visible by a CTA barrier): its SPC
     // column slots of every other CTA's rows, and the P/2 + 1 spectrum entries
@@ -245,12 +268,11 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     // packed pair: SPC + 1 entries of its own)
     const uint32_t bytes_col = (uint32_t)(3 * (D - nloc) * SPC * sizeof(cplx<T>));
     const uint32_t bytes_row = (uint32_t)(3 * nloc * (P / 2 + 1 - SPC - (rank == 0 ? 1 : 0)) * sizeof(cplx<T>));
-    uint32_t phase = 0;
-    cluster.sync();   // every CTA runs, with its barriers initialised, before the first remote store
+    __syncthreads();   // the state, the kernel's entries and the cell range are in place
     const int c0 = crange[0], c1 = crange[1];
 
     for (long long n = 0; n < nsteps; ++n) {
-        const unsigned long long step = step_base + r.step0 + (unsigned long long)n;
+        const unsigned long long step = step_base + r.step0 + (unsigned long long)(seg.step_begin + n);
         for (int stage = 0; stage < ModeStages<MODE>::n; ++stage) {
             if (tid == 0) {
                 mbar_expect(mb_col, bytes_col);
@@ -485,21 +507,30 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
         const int y = cell / D, x = cell - y * D;
         yg.st((long long)y * Dpad + x, ynv.ld((long long)(y - ylo) * Dpad + x));
     }
+    if (SEG && seg.signal) {   // every CTA's rows are written before the flag
+        __threadfence();
+        cluster.sync();
+        if (rank == 0 && tid == 0) {
+            __threadfence();
+            atomicExch(flags + seg.rep, 1);
+        }
+    }
+    }
     cluster.sync();   // no CTA leaves while another may still access its shared memory
 }
 
 // Launch configuration of one replica per cluster of NC CTAs (the cluster
 // shape is a launch attribute; NC = 16 is a non-portable size the GPU allows).
-template <int P, typename T, int MODE, int NC>
-static cudaError_t cluster_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int nwork, size_t sm,
+template <int P, typename T, int MODE, int NC, bool SEG>
+static cudaError_t cluster_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int nclusters, size_t sm,
                                   cudaStream_t st)
 {
-    auto kern = k_cluster<P, T, MODE, NC>;
+    auto kern = k_cluster<P, T, MODE, NC, SEG>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e == cudaSuccess && NC > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cfg = cudaLaunchConfig_t{};
-    cfg.gridDim = dim3(nwork * NC, 1, 1);
+    cfg.gridDim = dim3(nclusters * NC, 1, 1);
     cfg.blockDim = dim3(ClusterGeom<P, T, NC>::NT, 1, 1);
     cfg.dynamicSmemBytes = sm;
     cfg.stream = st;
@@ -512,16 +543,17 @@ static cudaError_t cluster_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *
     return cudaSuccess;
 }
 
-template <int P, typename T, int MODE, int NC>
+template <int P, typename T, int MODE, int NC, bool SEG>
 static cudaError_t launch_cluster_t(const LaunchArgs &a, int maxD, int maxDpad)
 {
     const size_t sm = cluster_smem_bytes<P, T, NC>(maxD, maxDpad, a.use_wbuf != 0);
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    cudaError_t e = cluster_config<P, T, MODE, NC>(cfg, attr, a.nwork, sm, a.stream);
+    cudaError_t e = cluster_config<P, T, MODE, NC, SEG>(cfg, attr, SEG ? a.ncta : a.nwork, sm, a.stream);
     if (e != cudaSuccess) return e;
-    return cudaLaunchKernelEx(&cfg, k_cluster<P, T, MODE, NC>, a.reps, a.work, (T *)a.y, (const cplx<T> *)a.tw,
-                              a.nsteps, a.step_base, a.use_wbuf, a.status);
+    return cudaLaunchKernelEx(&cfg, k_cluster<P, T, MODE, NC, SEG>, a.reps, a.work, (T *)a.y, (const cplx<T> *)a.tw,
+                              a.nsteps, a.step_base, a.use_wbuf, a.status, reinterpret_cast<const Segment *>(a.segs),
+                              a.seg_off, a.flags, a.flags ? a.flags + a.n_rep : nullptr);
 }
 
 // Clusters of the size class that can be resident at once (0: the cluster
@@ -532,12 +564,12 @@ static int cluster_max_active_t(int maxD, int maxDpad, bool wbuf)
     const size_t sm = cluster_smem_bytes<P, T, NC>(maxD, maxDpad, wbuf);
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    if (cluster_config<P, T, M_HEUN, NC>(cfg, attr, 1, sm, 0) != cudaSuccess) {
+    if (cluster_config<P, T, M_HEUN, NC, false>(cfg, attr, 1, sm, 0) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_cluster<P, T, M_HEUN, NC>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, k_cluster<P, T, M_HEUN, NC, false>, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -547,8 +579,12 @@ static int cluster_max_active_t(int maxD, int maxDpad, bool wbuf)
 template <int P, typename T, int NC>
 static cudaError_t launch_cluster_p(const LaunchArgs &a, int maxD, int maxDpad)
 {
-    if (a.mode == M_RK4) return launch_cluster_t<P, T, M_RK4, NC>(a, maxD, maxDpad);
-    if (a.mode == M_HEUN) return launch_cluster_t<P, T, M_HEUN, NC>(a, maxD, maxDpad);
+    if (a.mode == M_RK4)
+        return a.segs ? launch_cluster_t<P, T, M_RK4, NC, true>(a, maxD, maxDpad)
+                      : launch_cluster_t<P, T, M_RK4, NC, false>(a, maxD, maxDpad);
+    if (a.mode == M_HEUN)
+        return a.segs ? launch_cluster_t<P, T, M_HEUN, NC, true>(a, maxD, maxDpad)
+                      : launch_cluster_t<P, T, M_HEUN, NC, false>(a, maxD, maxDpad);
     return cudaErrorInvalidValue;
 }
 

@@ -7,6 +7,14 @@
 
 namespace nd {
 
+// The kernels that step, relax and evaluate fields are compiled with
+// -fmad=false and name every fused multiply-add themselves, so that the
+// rounding of an expression does not depend on the function it is inlined
+// into: the one-CTA kernel, the cluster kernel and the global path round each
+// cell alike, and the default plan may take whichever is faster.
+__device__ __forceinline__ float fm(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fm(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 template <typename T> struct cplx { T x, y; };
 template <typename T> struct vec3 { T x, y, z; };
 
@@ -14,11 +22,11 @@ template <typename T> __device__ __forceinline__ cplx<T> cadd(cplx<T> a, cplx<T>
 template <typename T> __device__ __forceinline__ cplx<T> csub(cplx<T> a, cplx<T> b) { return {a.x - b.x, a.y - b.y}; }
 template <typename T> __device__ __forceinline__ cplx<T> cmul(cplx<T> a, cplx<T> b)
 {
-    return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
+    return {fm(a.x, b.x, -(a.y * b.y)), fm(a.x, b.y, a.y * b.x)};
 }
 template <typename T> __device__ __forceinline__ cplx<T> cmulc(cplx<T> a, cplx<T> b)  // a * conj(b)
 {
-    return {a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y};
+    return {fm(a.x, b.x, a.y * b.y), fm(a.y, b.x, -(a.x * b.y))};
 }
 template <typename T> __device__ __forceinline__ cplx<T> cconj(cplx<T> a) { return {a.x, -a.y}; }
 template <typename T> __device__ __forceinline__ cplx<T> cscale(cplx<T> a, T s) { return {a.x * s, a.y * s}; }

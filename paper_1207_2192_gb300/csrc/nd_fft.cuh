@@ -128,6 +128,18 @@ __device__ __forceinline__ cplx<T> twid(cplx<T> b, int k, int N)
     return DIR < 0 ? cmul(b, w) : cmulc(b, w);
 }
 
+// a + w^k b for the N-th root w = exp(DIR 2 pi i / N), N | 32: where one
+// output is wanted, two multiply-adds per part instead of a product and an
+// addition.
+template <int DIR, typename T>
+__device__ __forceinline__ cplx<T> axwb(cplx<T> a, cplx<T> b, int k, int N)
+{
+    if (k == 0 || 4 * k == N || 2 * k == N || 4 * k == 3 * N) return cadd(a, twid<DIR>(b, k, N));
+    const cplx<T> w = w32<T>(k * (32 / N));
+    const T s = DIR < 0 ? w.y : -w.y;
+    return {fm(b.x, w.x, fm(-b.y, s, a.x)), fm(b.x, s, fm(b.y, w.x, a.y))};
+}
+
 // In-register N-point DFT, natural order in and out:
 // v[k] <- sum_n v[n] exp(DIR 2 pi i n k / N), for N a power of two up to 32
 // (radix 2), or three or five times one (one radix-3 stage on top, N | 24, or
@@ -180,10 +192,10 @@ __device__ __forceinline__ void dft_reg(cplx<T> *v)
             const cplx<T> b0 = a[0][k], b1 = twid<DIR>(a[1][k], k, N), b2 = twid<DIR>(a[2][k], 2 * k, N),
                           b3 = twid<DIR>(a[3][k], 3 * k, N), b4 = twid<DIR>(a[4][k], 4 * k, N);
             const cplx<T> t1 = cadd(b1, b4), t2 = cadd(b2, b3), t3 = csub(b1, b4), t4 = csub(b2, b3);
-            const cplx<T> p1 = {b0.x + c1 * t1.x + c2 * t2.x, b0.y + c1 * t1.y + c2 * t2.y};
-            const cplx<T> p2 = {b0.x + c2 * t1.x + c1 * t2.x, b0.y + c2 * t1.y + c1 * t2.y};
-            const cplx<T> q1 = {s1 * t3.x + s2 * t4.x, s1 * t3.y + s2 * t4.y};
-            const cplx<T> q2 = {s2 * t3.x - s1 * t4.x, s2 * t3.y - s1 * t4.y};
+            const cplx<T> p1 = {fm(c2, t2.x, fm(c1, t1.x, b0.x)), fm(c2, t2.y, fm(c1, t1.y, b0.y))};
+            const cplx<T> p2 = {fm(c1, t2.x, fm(c2, t1.x, b0.x)), fm(c1, t2.y, fm(c2, t1.y, b0.y))};
+            const cplx<T> q1 = {fm(s1, t3.x, s2 * t4.x), fm(s1, t3.y, s2 * t4.y)};
+            const cplx<T> q2 = {fm(s2, t3.x, -(s1 * t4.x)), fm(s2, t3.y, -(s1 * t4.y))};
             // DIR i q = DIR (-q.y, q.x)
             const cplx<T> e1 = DIR < 0 ? cplx<T>{q1.y, -q1.x} : cplx<T>{-q1.y, q1.x};
             const cplx<T> e2 = DIR < 0 ? cplx<T>{q2.y, -q2.x} : cplx<T>{-q2.y, q2.x};
@@ -213,12 +225,12 @@ __device__ __forceinline__ void dft_reg(cplx<T> *v)
         for (int k = 0; k < M; ++k) {
             const cplx<T> bk = twid<DIR>(b[k], k, N), ck = twid<DIR>(c[k], 2 * k, N);
             const cplx<T> s = cadd(bk, ck), d = csub(bk, ck);
-            const cplx<T> t = {a[k].x - T(0.5) * s.x, a[k].y - T(0.5) * s.y};
+            const cplx<T> t = {fm(T(-0.5), s.x, a[k].x), fm(T(-0.5), s.y, a[k].y)};
             // exp(DIR 2 pi i/3) = -1/2 + DIR i sin(pi/3): X[k + M] = t + DIR i h3 d, X[k + 2M] = t - DIR i h3 d
-            const cplx<T> e = DIR < 0 ? cplx<T>{h3 * d.y, -h3 * d.x} : cplx<T>{-h3 * d.y, h3 * d.x};
+            const T h = DIR < 0 ? h3 : -h3;
             v[k] = cadd(a[k], s);
-            v[k + M] = cadd(t, e);
-            v[k + 2 * M] = csub(t, e);
+            v[k + M] = {fm(h, d.y, t.x), fm(-h, d.x, t.y)};
+            v[k + 2 * M] = {fm(-h, d.y, t.x), fm(h, d.x, t.y)};
         }
     }
 }
@@ -257,7 +269,10 @@ __device__ __forceinline__ void dft_reg_halfout(cplx<T> *v)
     dft_reg<N / 2, DIR>(a);
     dft_reg<N / 2, DIR>(b);
 #pragma unroll
-    for (int k = 0; k < N / 2; ++k) v[k] = cadd(a[k], twid<DIR>(b[k], k, N));
+    for (int k = 0; k < N / 2; ++k) {
+        if constexpr (32 % N == 0) v[k] = axwb<DIR>(a[k], b[k], k, N);
+        else v[k] = cadd(a[k], twid<DIR>(b[k], k, N));
+    }
 }
 
 enum : int { FFT_FULL = 0, FFT_HALF_IN = 1, FFT_HALF_OUT = 2 };

@@ -24,28 +24,32 @@ namespace nd {
 template <typename T> __device__ __forceinline__ vec3<T> v3(T x, T y, T z) { return {x, y, z}; }
 template <typename T> __device__ __forceinline__ vec3<T> cross3(vec3<T> a, vec3<T> b)
 {
-    return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
+    return {fm(a.y, b.z, -(a.z * b.y)), fm(a.z, b.x, -(a.x * b.z)), fm(a.x, b.y, -(a.y * b.x))};
 }
 template <typename T> __device__ __forceinline__ vec3<T> axpy3(T s, vec3<T> a, vec3<T> b)
 {
-    return {b.x + s * a.x, b.y + s * a.y, b.z + s * a.z};
+    return {fm(s, a.x, b.x), fm(s, a.y, b.y), fm(s, a.z, b.z)};
+}
+template <typename T> __device__ __forceinline__ T dot3(vec3<T> a, vec3<T> b)
+{
+    return fm(a.z, b.z, fm(a.y, b.y, a.x * b.x));
 }
 template <typename T> __device__ __forceinline__ vec3<T> normalize3(vec3<T> v)
 {
-    T r = drsqrt<T>(v.x * v.x + v.y * v.y + v.z * v.z);
+    T r = drsqrt<T>(dot3(v, v));
     return {v.x * r, v.y * r, v.z * r};
 }
 // Landau-Lifshitz right-hand side m x b - alpha m x (m x b) (Section III.A).
 template <typename T> __device__ __forceinline__ vec3<T> llg_rhs(vec3<T> m, vec3<T> b, T alpha)
 {
     vec3<T> p = cross3(m, b), q = cross3(m, p);
-    return {p.x - alpha * q.x, p.y - alpha * q.y, p.z - alpha * q.z};
+    return axpy3(-alpha, q, p);
 }
 // One Heun stage change m x [g - alpha m x g], g = b dtau + sigma w (Section III.C).
 template <typename T> __device__ __forceinline__ vec3<T> heun_dm(vec3<T> m, vec3<T> g, T alpha)
 {
     vec3<T> p = cross3(m, g);
-    return cross3(m, vec3<T>{g.x - alpha * p.x, g.y - alpha * p.y, g.z - alpha * p.z});
+    return cross3(m, axpy3(-alpha, p, g));
 }
 
 // Programmatic dependent launch: the global path's kernels are launched so
@@ -102,15 +106,14 @@ __device__ __forceinline__ StageOut<T> stage_update(const StepParams<T> &sp, boo
         }
     } else {   // M_HEUN
         vec3<T> g = {b.x * dt, b.y * dt, b.z * dt};
-        if (noise) { g.x += sp.sigma * w.x; g.y += sp.sigma * w.y; g.z += sp.sigma * w.z; }
+        if (noise) g = axpy3(sp.sigma, w, g);
         vec3<T> d = heun_dm(m, g, alpha);
         if (stage == 0) {
             o.acc = d;
             o.nm = normalize3(vec3<T>{m.x + d.x, m.y + d.y, m.z + d.z});
             o.w_acc = true; o.w_yn = false;
         } else {
-            o.nm = normalize3(vec3<T>{y.x + T(0.5) * (a.x + d.x), y.y + T(0.5) * (a.y + d.y),
-                                      y.z + T(0.5) * (a.z + d.z)});
+            o.nm = normalize3(axpy3(T(0.5), vec3<T>{a.x + d.x, a.y + d.y, a.z + d.z}, y));
             o.w_acc = false; o.w_yn = true;
         }
     }
@@ -138,8 +141,8 @@ __device__ __forceinline__ double epilogue_cell(const Replica &r, int cell, long
     } else if (MODE == M_ENERGY) {
         // E/J = -sum_i m_i . (b'_i / 2 + c h_ext), b' = b - c h_ext  (Eq. Hmm)
         double bx = (double)b.x - r.chext[0], by = (double)b.y - r.chext[1], bz = (double)b.z - r.chext[2];
-        return -((double)m.x * (0.5 * bx + r.chext[0]) + (double)m.y * (0.5 * by + r.chext[1]) +
-                 (double)m.z * (0.5 * bz + r.chext[2]));
+        return -fm((double)m.x, fm(0.5, bx, r.chext[0]),
+                   fm((double)m.y, fm(0.5, by, r.chext[1]), (double)m.z * fm(0.5, bz, r.chext[2])));
     } else if (MODE == M_RK4 || MODE == M_HEUN) {
         const StepParams<T> sp = step_params<T>(r);
         const vec3<T> zero = {T(0), T(0), T(0)};
@@ -245,24 +248,25 @@ __device__ __forceinline__ vec3<T> relax_cell(vec3<T> m, vec3<T> b, bool inW, T 
                                               RelaxAcc<T> &acc)
 {
     vec3<T> e = b;
-    if (inW) e.z += l0 * T(2) * m.z * dx + l1 * T(2) * m.z * dy;
-    const T en = dsqrt<T>(e.x * e.x + e.y * e.y + e.z * e.z);
+    if (inW) e.z = fm(l0 * T(2) * m.z, dx, fm(l1 * T(2) * m.z, dy, e.z));
+    const T en = dsqrt<T>(dot3(e, e));
     const vec3<T> u = {e.x / en, e.y / en, e.z / en};
     const vec3<T> tq = cross3(m, u);
-    acc.res = max(acc.res, dsqrt<T>(tq.x * tq.x + tq.y * tq.y + tq.z * tq.z));
-    const vec3<T> v = {(T(1) - eta) * m.x + eta * u.x, (T(1) - eta) * m.y + eta * u.y, (T(1) - eta) * m.z + eta * u.z};
-    const T vn = dsqrt<T>(v.x * v.x + v.y * v.y + v.z * v.z);
+    acc.res = max(acc.res, dsqrt<T>(dot3(tq, tq)));
+    const T om = T(1) - eta;
+    const vec3<T> v = {fm(eta, u.x, om * m.x), fm(eta, u.y, om * m.y), fm(eta, u.z, om * m.z)};
+    const T vn = dsqrt<T>(dot3(v, v));
     const vec3<T> mp = {v.x / vn, v.y / vn, v.z / vn};
     if (inW) {
-        const vec3<T> q = {-u.x * u.z / en, -u.y * u.z / en, (T(1) - u.z * u.z) / en};
-        const T mq = mp.x * q.x + mp.y * q.y + mp.z * q.z;
-        const T kap = eta * (q.z - mp.z * mq) / vn;
+        const vec3<T> q = {-u.x * u.z / en, -u.y * u.z / en, fm(-u.z, u.z, T(1)) / en};
+        const T mq = dot3(mp, q);
+        const T kap = eta * fm(-mp.z, mq, q.z) / vn;
         const T w = T(4) * mp.z * m.z * kap;
-        acc.C0 += mp.z * mp.z * dx;
-        acc.C1 += mp.z * mp.z * dy;
-        acc.J00 += w * dx * dx;
-        acc.J01 += w * dx * dy;
-        acc.J11 += w * dy * dy;
+        acc.C0 = fm(mp.z * mp.z, dx, acc.C0);
+        acc.C1 = fm(mp.z * mp.z, dy, acc.C1);
+        acc.J00 = fm(w * dx, dx, acc.J00);
+        acc.J01 = fm(w * dx, dy, acc.J01);
+        acc.J11 = fm(w * dy, dy, acc.J11);
     }
     return mp;
 }
@@ -358,7 +362,7 @@ __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
         // row tasks: one real row each (half-length transforms) at P = 128,
         // else a complex row pair each
         constexpr bool HR = HalfRows<P>::on;
-        const int nrow = HR ? 3 * D : row_tasks(D);
+        const int nrow = row_pass_tasks<P>(D);
         double esum = 0.0;
         T relX = 0, relY = 0;
         if (MODE == M_RELAX) {
@@ -417,7 +421,7 @@ __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
                         const long long si = (long long)y * Dpad + x, hi = (long long)y * (2 * RS) + x;
                         vec3<T> b = {hr[hi] + sp.chext[0], hr[2 * cs + hi] + sp.chext[1], hr[4 * cs + hi] + sp.chext[2]};
                         const T dx = (T)x - T(0.5) * (T)(D - 1) - relX, dy = (T)y - T(0.5) * (T)(D - 1) - relY;
-                        relax_cell<T>(ms.ld(si), b, dx * dx + dy * dy < rc2, dx, dy, l0, l1, eta, a);
+                        relax_cell<T>(ms.ld(si), b, fm(dx, dx, dy * dy) < rc2, dx, dy, l0, l1, eta, a);
                     }
                     a.C0 = warp_sum_t(a.C0); a.C1 = warp_sum_t(a.C1); a.J00 = warp_sum_t(a.J00);
                     a.J01 = warp_sum_t(a.J01); a.J11 = warp_sum_t(a.J11); a.res = warp_max_t(a.res);
@@ -450,7 +454,7 @@ __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
                         vec3<T> b = {hr[hi] + sp.chext[0], hr[2 * cs + hi] + sp.chext[1], hr[4 * cs + hi] + sp.chext[2]};
                         const T dx = (T)x - T(0.5) * (T)(D - 1) - relX, dy = (T)y - T(0.5) * (T)(D - 1) - relY;
                         RelaxAcc<T> dummy = {T(0), T(0), T(0), T(0), T(0), T(0)};
-                        ms.st(si, relax_cell<T>(ms.ld(si), b, dx * dx + dy * dy < rc2, dx, dy, m0, m1, eta, dummy));
+                        ms.st(si, relax_cell<T>(ms.ld(si), b, fm(dx, dx, dy * dy) < rc2, dx, dy, m0, m1, eta, dummy));
                     }
                     __syncthreads();
                     continue;
@@ -556,14 +560,23 @@ __global__ void __launch_bounds__(NT, RowsMinB<P, T>::v)
     __syncthreads();
     GroupId<P> gid(tid);
     const int q = blockIdx.x * NGRP + gid.group;
-    const int nrow = row_tasks(D);
+    const int nrow = row_pass_tasks<P>(D);
     if (blockIdx.x * NGRP >= nrow) return;   // CTA-uniform
     if (!gid.valid) return;                  // lanes past the warp's last group
     const long long cs = (long long)D * RS;
     cplx<T> *spec = specbase + r.spec_off;
     cplx<T> *scr = scratch + gid.group * Gm::SCRATCH;
-    if (!inverse) {
-        const long long ms_s = (long long)D * r.Dpad;
+    const long long ms_s = (long long)D * r.Dpad;
+    if constexpr (HalfRows<P>::on) {
+        const bool act = q < nrow;
+        const int c = act ? q / D : 0, y = act ? q - c * D : 0;
+        cplx<T> *row = spec + c * cs + (long long)y * RS;
+        if (!inverse)
+            row_fwd_half<P, T>(act, msbase + r.state_off + c * ms_s + (long long)y * r.Dpad, D, row, gid.t, scr, tw,
+                               gid.gmask);
+        else
+            row_inv_half<P, T>(act, row, D, reinterpret_cast<T *>(row), gid.t, scr, tw, gid.gmask);
+    } else if (!inverse) {
         row_fwd_task<P, T>(q, q < nrow, D, msbase + r.state_off, r.Dpad, ms_s, spec, cs, gid.t, gid.lane, scr, tw,
                            gid.gmask);
     } else {
@@ -961,7 +974,7 @@ __global__ void __launch_bounds__(256)
         const long long si = (long long)y * r.Dpad + x, hi = (long long)y * (2 * RS) + x;
         const vec3<T> b = {hr[hi] + sp.chext[0], hr[2 * cs + hi] + sp.chext[1], hr[4 * cs + hi] + sp.chext[2]};
         const T dx = (T)x - T(0.5) * (T)(D - 1) - relX, dy = (T)y - T(0.5) * (T)(D - 1) - relY;
-        relax_cell<T>(ms.ld(si), b, dx * dx + dy * dy < rc2, dx, dy, l0, l1, eta, a);
+        relax_cell<T>(ms.ld(si), b, fm(dx, dx, dy * dy) < rc2, dx, dy, l0, l1, eta, a);
     }
     a.C0 = warp_sum_t(a.C0); a.C1 = warp_sum_t(a.C1); a.J00 = warp_sum_t(a.J00);
     a.J01 = warp_sum_t(a.J01); a.J11 = warp_sum_t(a.J11); a.res = warp_max_t(a.res);
@@ -1027,7 +1040,7 @@ __global__ void __launch_bounds__(256)
     const vec3<T> b = {hr[hi] + sp.chext[0], hr[2 * cs + hi] + sp.chext[1], hr[4 * cs + hi] + sp.chext[2]};
     const T dx = (T)x - T(0.5) * (T)(D - 1) - relX, dy = (T)y - T(0.5) * (T)(D - 1) - relY;
     RelaxAcc<T> dummy = {T(0), T(0), T(0), T(0), T(0), T(0)};
-    ms.st(si, relax_cell<T>(ms.ld(si), b, dx * dx + dy * dy < (T)rc2_d, dx, dy, m0, m1, (T)eta_d, dummy));
+    ms.st(si, relax_cell<T>(ms.ld(si), b, fm(dx, dx, dy * dy) < (T)rc2_d, dx, dy, m0, m1, (T)eta_d, dummy));
 }
 
 // The same sweep driven by an externally computed energy gradient: the field
@@ -1056,7 +1069,7 @@ __global__ void __launch_bounds__(256)
         const long long si = (long long)y * r.Dpad + x;
         const vec3<T> g = gr.ld(si), b = {sc * g.x, sc * g.y, sc * g.z};
         const T dx = (T)x - T(0.5) * (T)(D - 1) - relX, dy = (T)y - T(0.5) * (T)(D - 1) - relY;
-        relax_cell<T>(ms.ld(si), b, dx * dx + dy * dy < rc2, dx, dy, l0, l1, eta, a);
+        relax_cell<T>(ms.ld(si), b, fm(dx, dx, dy * dy) < rc2, dx, dy, l0, l1, eta, a);
     }
     a.C0 = warp_sum_t(a.C0); a.C1 = warp_sum_t(a.C1); a.J00 = warp_sum_t(a.J00);
     a.J01 = warp_sum_t(a.J01); a.J11 = warp_sum_t(a.J11); a.res = warp_max_t(a.res);
@@ -1095,7 +1108,7 @@ __global__ void __launch_bounds__(256)
     const vec3<T> g = gr.ld(si), b = {sc * g.x, sc * g.y, sc * g.z};
     const T dx = (T)x - T(0.5) * (T)(D - 1) - relX, dy = (T)y - T(0.5) * (T)(D - 1) - relY;
     RelaxAcc<T> dummy = {T(0), T(0), T(0), T(0), T(0), T(0)};
-    ms.st(si, relax_cell<T>(ms.ld(si), b, dx * dx + dy * dy < (T)rc2_d, dx, dy, m0, m1, (T)eta_d, dummy));
+    ms.st(si, relax_cell<T>(ms.ld(si), b, fm(dx, dx, dy * dy) < (T)rc2_d, dx, dy, m0, m1, (T)eta_d, dummy));
 }
 
 // One gradient-driven sweep over the replicas of one size class.
@@ -1298,7 +1311,7 @@ template <int P, typename T>
 static void glob_rows(const LaunchArgs &a, int maxD, int inverse)
 {
     constexpr int NT = GlobNT<P>::v, NGRP = groups_per_block<P, NT>();
-    const int nrow = row_tasks(maxD);
+    const int nrow = row_pass_tasks<P>(maxD);
     dim3 gr((nrow + NGRP - 1) / NGRP, a.nwork);
     launch_pdl(k_g_rows<P, T, NT>, gr, dim3(NT), glob_smem_bytes<P, T, NT>(), a.stream, a.reps, a.work,
                (const T *)a.ms, (cplx<T> *)a.spec, (const cplx<T> *)a.tw, inverse);
@@ -1355,8 +1368,10 @@ static cudaError_t launch_global_p(const LaunchArgs &a, int maxD)
     constexpr int NT = GlobNT<P>::v;
     const int sm = (int)glob_smem_bytes<P, T, NT>();
     cudaError_t e0 = cudaFuncSetAttribute(k_g_rows<P, T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    if (e0 == cudaSuccess) e0 = cudaFuncSetAttribute(k_g_cols<P, T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    if constexpr (GlobTiled<P>::v) {
+    if constexpr (!GlobTiled<P>::v) {
+        if (e0 == cudaSuccess)
+            e0 = cudaFuncSetAttribute(k_g_cols<P, T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    } else {
         if (e0 == cudaSuccess)
             e0 = cudaFuncSetAttribute(k_g_cols_tile<P, T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)glob_smem_bytes<P, T, ColTile<P, T, true>::NT>());

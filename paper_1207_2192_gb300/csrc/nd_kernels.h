@@ -42,8 +42,9 @@ struct LaunchArgs {
     // segs[seg_off[b] .. seg_off[b+1]) and hand replicas over through flags
     const void *segs = nullptr;
     const int *seg_off = nullptr;
-    int *flags = nullptr;
-    int ncta = 0;
+    int *flags = nullptr;            // cluster plans: n_rep flags, then the ticket counter
+    int n_rep = 0;
+    int ncta = 0;                    // CTAs (cluster plans: clusters) of the schedule
     unsigned *status = nullptr;      // device status word (ND_DEV_* bits)
     int use_wbuf = 0;                // keep the Heun predictor's normals in shared memory
     int smem_optin = 0;              // per-block shared-memory limit of the device

@@ -138,7 +138,7 @@ __device__ __forceinline__ void row_fwd_task(int q, bool active, int D, const T 
 template <typename T>
 __device__ __forceinline__ cplx<T> tensor_row(T g0, cplx<T> a, T g1, cplx<T> b)
 {
-    return {g0 * a.x + g1 * b.x, g0 * a.y + g1 * b.y};
+    return {fm(g1, b.x, g0 * a.x), fm(g1, b.y, g0 * a.y)};
 }
 
 template <int P, typename T>
@@ -168,8 +168,8 @@ __device__ __forceinline__ void col_multiply_z(cplx<T> *vz, const T *Ghat, int k
     for (int o = 0; o < R1; ++o) {
         const int ky = t + G * o;
         const int kyr = ky <= P / 2 ? ky : P - ky;
-        GhatVal<T> g = load_ghat<T>(Ghat, kx * KH + kyr);
-        vz[o] = cscale(vz[o], g.zz);
+        // from the component-major copy: a quarter of the bytes of the interleaved entries
+        vz[o] = cscale(vz[o], __ldg(Ghat + 7 * KH * KH + kx * KH + kyr));
     }
 }
 
@@ -248,9 +248,7 @@ __device__ __forceinline__ void packed_col_scale(cplx<T> *v, int c, const T *Gha
         const T h = T(0.5);
         cplx<T> F0 = {h * (v[o].x + w.x), h * (v[o].y - w.y)};
         cplx<T> F1 = {h * (v[o].y + w.y), -h * (v[o].x - w.x)};
-        F0 = cscale(F0, s0);
-        F1 = cscale(F1, s1);
-        v[o] = {F0.x - F1.y, F0.y + F1.x};
+        v[o] = {fm(F0.x, s0, -(F1.y * s1)), fm(F0.y, s0, F1.x * s1)};   // s0 F0 + i s1 F1
     }
     __syncwarp(gmask);
 }
@@ -469,6 +467,12 @@ __device__ __forceinline__ void row_inv_task(int q, bool active, int D, cplx<T> 
 template <int P> struct HalfRows { static constexpr bool on = false; };
 template <> struct HalfRows<128> { static constexpr bool on = FFTGeom<64>::G == FFTGeom<128>::G; };
 
+// Tasks of a row pass over D rows: one per component and row, or pairs.
+template <int P> __host__ __device__ __forceinline__ int row_pass_tasks(int D)
+{
+    return HalfRows<P>::on ? 3 * D : row_tasks(D);
+}
+
 // Forward: the real row x (x[i], i < D; zero beyond) to its half spectrum:
 // X[k] for k = t + G o (k < M) left in v[o], X[M] (real) in xm on lane t = 0.
 template <int P, typename T>
@@ -483,23 +487,24 @@ __device__ __forceinline__ void row_fwd_half_spectrum(bool active, const T *x, i
         const int n = t + G * o;
         if (active) {
             const T a = 2 * n < D ? x[2 * n] : T(0), b = 2 * n + 1 < D ? x[2 * n + 1] : T(0);
-            v[o] = {a, b};
+            // halved here, where half of the registers are zero, instead of in
+            // the split below (a power of two: the rounding is the same)
+            v[o] = {T(0.5) * a, T(0.5) * b};
         }
     }
     fft_group<M, -1, FFT_HALF_IN, 2 * G>(v, t, scr, twP, gmask);
     mirror_put<M>(v, scr, t);
     __syncwarp(gmask);
     const cplx<T> w1 = twP[G + t];   // W^t
-    const T h = T(0.5);
-    xm = v[0].x - v[0].y;            // X[M] = Re Z[0] - Im Z[0] (used on lane 0)
+    xm = T(2) * (v[0].x - v[0].y);   // X[M] = Re Z[0] - Im Z[0] (used on lane 0)
 #pragma unroll
     for (int o = 0; o < R1; ++o) {
         const int k = t + G * o;
         const cplx<T> z = v[o], zm = mirror_get<M>(scr, k);
-        const cplx<T> e = {h * (z.x + zm.x), h * (z.y - zm.y)};   // (Z[k] + conj Z[M-k]) / 2
-        const cplx<T> d = {h * (z.x - zm.x), h * (z.y + zm.y)};   // (Z[k] - conj Z[M-k]) / 2
-        const cplx<T> wd = cmul(twid<-1>(w1, o, P / G), d);        // W^k d, W^k = W^t W^(G o)
-        v[o] = {e.x + wd.y, e.y - wd.x};                            // e - i W^k d
+        const cplx<T> e = {z.x + zm.x, z.y - zm.y};   // (Z[k] + conj Z[M-k]) / 2
+        const cplx<T> d = {z.x - zm.x, z.y + zm.y};   // (Z[k] - conj Z[M-k]) / 2
+        const cplx<T> w = twid<-1>(w1, o, P / G);     // W^k = W^t W^(G o)
+        v[o] = {fm(d.x, w.y, fm(d.y, w.x, e.x)), fm(-d.x, w.x, fm(d.y, w.y, e.y))};   // e - i W^k d
     }
     __syncwarp(gmask);
 }
@@ -540,8 +545,7 @@ __device__ __forceinline__ void row_inv_half(bool active, const cplx<T> *src, in
         const cplx<T> s = {a.x + b.x, a.y - b.y};                     // X[k] + conj X[M-k]
         const cplx<T> d = {a.x - b.x, a.y + b.y};                     // X[k] - conj X[M-k]
         const cplx<T> wk = twid<-1>(w1, o, P / G);                    // W^k
-        const cplx<T> wd = {wk.x * d.x + wk.y * d.y, wk.x * d.y - wk.y * d.x};   // W^-k d
-        v[o] = {s.x - wd.y, s.y + wd.x};                                // s + i W^-k d
+        v[o] = {fm(-d.y, wk.x, fm(d.x, wk.y, s.x)), fm(d.x, wk.x, fm(d.y, wk.y, s.y))};   // s + i W^-k d
     }
     fft_group<M, +1, FFT_HALF_OUT, 2 * G>(v, t, scr, twP, gmask);
     if (active) {

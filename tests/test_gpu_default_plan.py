@@ -1,0 +1,48 @@
+"""The default stepping plan: few replicas step on thread-block clusters, more
+than the resident clusters time-sliced over them, many on the one-CTA kernel
+or the global path.  Every plan of a size rounds alike, so a replica ends bit
+for bit where the plain plan puts it, whatever shares its handle."""
+import numpy as np
+import pytest
+import torch
+
+import paper_1207_2192_gb300 as nd
+from paper_1207_2192_gb300 import Disk, Nanodisk
+
+pytestmark = pytest.mark.gpu
+
+
+def states(disks, reps, prec, plan, method, steps=5):
+    h = Nanodisk(disks, reps, prec)
+    if plan is not None:
+        nd.nd_set_plan(h.h, 0, method, plan)
+    X0 = np.stack([np.linspace(-3e-9, 3e-9, h.B), np.full(h.B, 0.5e-9)], 1)
+    m = h.empty_device()
+    h.init_vortex(m, X0)
+    if method == nd.ND_METHOD_HEUN:
+        h.heun(m, steps, 1e-14, np.linspace(0.0, 300.0, h.B), np.arange(h.B, dtype=np.uint64) + 7, step0=3)
+    else:
+        h.rk4(m, steps, 1e-14)
+    torch.cuda.synchronize()
+    assert nd.nd_check_status(h.h) == nd.ND_OK
+    return m
+
+
+@pytest.mark.parametrize("method", [nd.ND_METHOD_HEUN, nd.ND_METHOD_RK4])
+@pytest.mark.parametrize("R,prec,B,plain", [
+    (7e-9, nd.ND_FP32, 3, 0), (16e-9, nd.ND_FP32, 9, 0), (32e-9, nd.ND_FP32, 17, 0), (33e-9, nd.ND_FP32, 1, 0),
+    (50e-9, nd.ND_FP32, 33, 0), (64e-9, nd.ND_FP32, 8, 0), (65e-9, nd.ND_FP32, 9, 100), (128e-9, nd.ND_FP32, 2, 100),
+    (9e-9, nd.ND_FP64, 16, 0), (31e-9, nd.ND_FP64, 18, 0), (34e-9, nd.ND_FP64, 2, 100), (64e-9, nd.ND_FP64, 17, 100)])
+def test_default_plan_gives_the_plain_plans_trajectory(R, prec, B, plain, method):
+    disks = [Disk(R, 0.2 * R, alpha=0.02, hext=(0.0, 5e3, 0.0))]
+    assert torch.equal(states(disks, [B], prec, None, method), states(disks, [B], prec, plain, method))
+
+
+@pytest.mark.parametrize("method", [nd.ND_METHOD_HEUN, nd.ND_METHOD_RK4])
+def test_time_sliced_clusters_with_disks_of_different_sizes(method):
+    """One class (P = 128) of disks with different rows per CTA, more replicas
+    than clusters: the clusters pass replicas of every size on."""
+    disks = [Disk(r * 1e-9, 8e-9, alpha=0.02) for r in (33, 41, 50, 57, 64)]
+    reps = [4, 3, 5, 4, 3]
+    assert torch.equal(states(disks, reps, nd.ND_FP32, 200, method), states(disks, reps, nd.ND_FP32, 0, method))
+    assert torch.equal(states(disks, reps, nd.ND_FP32, 201, method), states(disks, reps, nd.ND_FP32, 0, method))
