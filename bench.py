@@ -77,7 +77,7 @@ def device_sms(device=0):
 # unit and the device headers it includes (nd_kernels.h holds only host
 # declarations and is left out).
 KERNEL_SOURCES = {
-    "batched_heun": ["nd_fused_f32.cu", "nd_cluster.cuh", "nd_field_impl.cuh", "nd_phases.cuh", "nd_fft.cuh",
+    "batched_heun": ["nd_fused_f32.cu", "nd_cluster_f32.cu", "nd_cluster.cuh", "nd_field_impl.cuh", "nd_phases.cuh", "nd_fft.cuh",
                      "nd_common.cuh"],
     "large_disk": ["nd_glob_f32.cu", "nd_field_impl.cuh", "nd_phases.cuh", "nd_fft.cuh", "nd_common.cuh"],
 }

@@ -80,16 +80,22 @@ struct SizeClass {
     int *seg_off_d = nullptr;
     int seg_mode = -1, seg_ncta = 0;
     long long seg_nsteps = -1;
-    int *cflags_d = nullptr;   // cluster schedules: hand-over flags of the replicas, then the ticket counter
+    int *cflags_d = nullptr;   // cluster schedules: hand-over flags of the replicas, the ticket counter, the count of finished ones
     // resident clusters per (RK4 / Heun, 8 / 16 CTAs) and the plan the default
     // stands for per method: -1 not yet looked up
     mutable int max_clusters[2][2] = {{-1, -1}, {-1, -1}};
     mutable int default_plan[2] = {-1, -1};
+    mutable int alone_plan[2] = {-1, -1};   // the same for the class without the others of its handle
 };
 
 constexpr int kPlanGlobal = 100;
 constexpr int kPlanCluster = 200;     // one replica per thread-block cluster of 8 CTAs (P <= 128)
 constexpr int kPlanCluster16 = 201;   // one replica per cluster of 16 CTAs (32 <= P <= 128)
+// Sweeps of one turn of a replica when more relax than clusters fit: with 16
+// replicas on 15 clusters a turn of 128 sweeps (about 1 ms at P = 128) makes
+// the hand-over (a state and a kernel table, some 5 us) small and still evens
+// out replicas that need different numbers of sweeps.
+constexpr int kRelaxTurn = 128;
 static int plan_cluster_nc(int pl) { return pl == kPlanCluster ? 8 : pl == kPlanCluster16 ? 16 : 0; }
 
 int next_pow2_at_least(int n)
@@ -227,6 +233,7 @@ static void fill_reps(nd_handle *h, bool fp64_kernel, double dt_seconds, const d
         R.state_off = h->rep_off[r];
         R.spec_off = h->rep_spec_off[r];
         R.Ghat = table == TAB_DL ? (const void *)d.ghatL : (fp64_kernel ? (const void *)d.ghat64 : (const void *)d.ghat32);
+        R.Ghat64 = d.ghat64;
         R.mask = d.mask_d;
         R.cells = d.cells_d;
         R.ncells = d.C;
@@ -355,8 +362,18 @@ static int default_plan(const nd_handle *h, const SizeClass &c0, int mode)
     for (size_t k = 0; k < h->classes.size(); ++k) {
         const auto &c = h->classes[k];
         c.default_plan[slot] = together ? pick[k] : c.fused_main ? 0 : kPlanGlobal;
+        c.alone_plan[slot] = pick[k];
     }
     return c0.default_plan[slot];
+}
+
+// CTAs per replica of the class's relaxation: 0 without clusters.  The grid-wide
+// passes of a class on the global path leave the GPU mostly idle for the few
+// replicas that take clusters, so here the classes choose one by one.
+static int relax_cluster_nc(const nd_handle *h, const SizeClass &c)
+{
+    default_plan(h, c, M_HEUN);   // (the relaxation's shared memory is that of a Heun step)
+    return plan_cluster_nc(c.alone_plan[1]);
 }
 
 // The time-sliced schedule of a class's replicas over nslots CTAs or clusters,
@@ -442,8 +459,8 @@ static int run_mode(nd_handle *h, int mode, bool fp64, void *y, void *out, long 
                 // more replicas than resident clusters: every cluster steps for
                 // the same time instead of in waves of whole replicas
                 if (int rc = class_segments(c, mode, nsteps, slots)) return rc;
-                if (int rc = ensure_alloc((void **)&c.cflags_d, sizeof(int) * (B + 1))) return rc;
-                ND_CUDA(cudaMemsetAsync(c.cflags_d, 0, sizeof(int) * (B + 1), st));
+                if (int rc = ensure_alloc((void **)&c.cflags_d, sizeof(int) * (B + 2))) return rc;
+                ND_CUDA(cudaMemsetAsync(c.cflags_d, 0, sizeof(int) * (B + 2), st));
                 a.segs = c.segs_d;
                 a.seg_off = c.seg_off_d;
                 a.flags = c.cflags_d;
@@ -1000,7 +1017,26 @@ int nd_relax_constrained(nd_handle *h, void *m, const double *X, double tol, int
     fill_reps(h, h->prec == ND_FP64, 0.0, nullptr, nullptr, 0);
     upload_reps(h, st);
     const int prec = h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32;
-    for (auto &c : h->classes) {
+    // The classes are independent: the ones that relax in one launch go to side
+    // streams, and those on the global path, whose host loop waits for each 32
+    // sweeps, follow one by one on the caller's.
+    const bool side = h->side.size() + 1 == h->classes.size() && !h->side.empty();
+    if (side) ND_CUDA(cudaEventRecord(h->fork_ev, st));
+    auto on_chip = [&](const SizeClass &c) { return c.fused_main || relax_cluster_nc(h, c); };
+    std::vector<int> order;
+    for (int pass = 0; pass < 2; ++pass)
+        for (int ci = 0; ci < (int)h->classes.size(); ++ci)
+            if (on_chip(h->classes[ci]) == (pass == 0)) order.push_back(ci);
+    size_t nside = 0;
+    std::vector<cudaEvent_t> joined;
+    const cudaStream_t st0 = st;
+    for (int ci : order) {
+        auto &c = h->classes[ci];
+        cudaStream_t st = st0;
+        if (side && nside < h->side.size() && on_chip(c)) {
+            st = h->side[nside++];
+            ND_CUDA(cudaStreamWaitEvent(st, h->fork_ev, 0));
+        }
         const DiskInfo &d = h->disks[h->rep_disk[c.reps[0]]];
         const double rcut = 4.0 * d.lambda / d.desc.a;
         LaunchArgs a;
@@ -1018,7 +1054,22 @@ int nd_relax_constrained(nd_handle *h, void *m, const double *X, double tol, int
         a.tol = tol;
         a.rc2 = rcut * rcut;
         a.max_iter = max_iter;
-        if (c.fused_main) {
+        // few replicas relax on clusters where the default would step them on
+        // clusters (a sweep is a field evaluation and two passes over the cells)
+        const int nc = relax_cluster_nc(h, c);
+        if (nc) {
+            const int slots = cluster_slots(h, c, prec, true, nc), Bc = a.nwork;
+            if (int rc = ensure_alloc((void **)&c.cflags_d, sizeof(int) * (B + 2))) return rc;
+            ND_CUDA(cudaMemsetAsync(c.cflags_d, 0, sizeof(int) * (B + 2), st));
+            a.status = h->status_d;
+            a.flags = c.cflags_d;
+            a.n_rep = B;
+            a.ncta = std::min(Bc, slots);
+            a.tw64 = h->tw64[c.P];
+            a.use_wbuf = 1;   // (the halos take the normals' place)
+            a.quantum = Bc > slots ? kRelaxTurn : std::max(max_iter, 1);
+            ND_CUDA(launch_cluster(c.P, prec, a, c.maxD, c.maxDpad, nc));
+        } else if (c.fused_main) {
             ND_CUDA(launch_fused(c.P, prec, a));
         } else {
             a.ms = h->ms;
@@ -1030,7 +1081,12 @@ int nd_relax_constrained(nd_handle *h, void *m, const double *X, double tol, int
             a.n_sm = h->n_sm;
             ND_CUDA(launch_global(c.P, prec, a, c.maxD));
         }
+        if (st != st0) {
+            ND_CUDA(cudaEventRecord(h->join_ev[nside - 1], st));
+            joined.push_back(h->join_ev[nside - 1]);
+        }
     }
+    for (cudaEvent_t e : joined) ND_CUDA(cudaStreamWaitEvent(st0, e, 0));
     ND_CUDA(cudaMemcpyAsync(h->rio_h, h->rio_d, sizeof(RelaxIO) * B, cudaMemcpyDeviceToHost, st));
     ND_CUDA(cudaStreamSynchronize(st));
     int rc = ND_OK;

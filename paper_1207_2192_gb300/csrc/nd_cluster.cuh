@@ -70,7 +70,7 @@ __host__ __device__ __forceinline__ size_t cluster_smem_bytes(int D, int Dpad, b
     b += sizeof(T) * (size_t)4 * CG::NTAB * CG::KH;                                     // kernel table
     b += sizeof(T) * (size_t)3 * rpc * Dpad * (wbuf ? 4 : 3);   // stage state, y_n, accumulator (+ normals)
     b += 2 * sizeof(int);                                                               // own cell range
-    b += 16;                                                                            // two mbarriers
+    b += 32;                                                                            // mbarriers
     return b;
 }
 
@@ -122,6 +122,16 @@ __device__ __forceinline__ void st_async(uint32_t a, cplx<double> v, uint32_t mb
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];"
                  :: "r"(a), "d"(v.x), "d"(v.y), "r"(mbar) : "memory");
 }
+__device__ __forceinline__ void st_async(uint32_t a, float v, uint32_t mbar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];"
+                 :: "r"(a), "f"(v), "r"(mbar) : "memory");
+}
+__device__ __forceinline__ void st_async(uint32_t a, double v, uint32_t mbar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f64 [%0], %1, [%2];"
+                 :: "r"(a), "d"(v), "r"(mbar) : "memory");
+}
 __device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(mbar), "r"(count) : "memory");
@@ -154,6 +164,29 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity)
     return false;
 }
 
+// The constrained relaxation (MODE == M_RELAX): the sweep of k_fused.  Its
+// schedule is a queue of turns: ticket k takes turn k / nwork of replica
+// work[k % nwork] -- at most `quantum` sweeps -- once the replica's turn
+// before that is over (flags[rep] counts them; that turn's ticket is lower, so
+// its cluster is running).  Converged replicas are passed over, and the
+// clusters leave when all have converged or used up their sweeps.  With no
+// more replicas than clusters a turn is the whole relaxation.
+//
+// The torque m x e is what the sweep drives to zero, so it is evaluated from
+// small terms: the exchange as sum_j (m_j - m_i) over the neighbours inside
+// the disk, straight from the state (the edge rows of the neighbouring CTAs
+// arrive as halos), and the demagnetisation alone through the FFT.  With the
+// exchange folded into the FFT, whose rounding is relative to |b| ~ 4, the
+// residual of an FP32 sweep carried noise of ~5e-7 and replicas stopped up to
+// ten sweeps from where FP64 arithmetic stops.
+struct ClusterRelax {
+    RelaxIO *rio;
+    const double *twP64;   // exp(-2 pi i k / P), FP64
+    double eta, tol, rc2;
+    int max_iter, quantum, nwork;
+    int *ndone;   // replicas finished
+};
+
 // Without SEG, one replica per cluster for the whole launch (compiled apart:
 // the schedule's loop around the steps cost 5-10% of each step).  With SEG
 // (more replicas than clusters fit on the GPU), a time-sliced schedule: the cluster
@@ -165,39 +198,84 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     k_cluster(const Replica *__restrict__ reps, const int *__restrict__ work, T *__restrict__ ybase,
               const cplx<T> *__restrict__ twP, long long nsteps_all, unsigned long long step_base, int use_wbuf,
               unsigned *__restrict__ status, const Segment *__restrict__ segs, const int *__restrict__ seg_off,
-              int *__restrict__ flags, int *__restrict__ ticket)
+              int *__restrict__ flags, int *__restrict__ ticket, const ClusterRelax rx)
 {
     using Gm = FFTGeom<P>;
     using CG = ClusterGeom<P, T, NC>;
     constexpr int G = Gm::G, R1 = Gm::R1, RS = SpecGeom<P>::RS, KH = CG::KH, NT = CG::NT, NGRP = CG::NGRP;
     constexpr int SPC = CG::SPC, SW = CG::SW, NTAB = CG::NTAB;
-    static_assert(MODE == M_RK4 || MODE == M_HEUN, "stepping modes");
+    static_assert(MODE == M_RK4 || MODE == M_HEUN || (MODE == M_RELAX && SEG), "stepping and relaxation modes");
+    constexpr bool RELAX = MODE == M_RELAX;
     cgc::cluster_group cluster = cgc::this_cluster();
     const int rank = (int)cluster.block_rank();
     extern __shared__ __align__(16) unsigned char smem[];
     const int tid = threadIdx.x;
     GroupId<P> gid(tid);
-    unsigned long long *mbars = reinterpret_cast<unsigned long long *>(smem);   // [0] columns, [1] rows
-    const uint32_t mb_col = smem_addr(mbars), mb_row = smem_addr(mbars + 1);
-    cplx<T> *tw = reinterpret_cast<cplx<T> *>(smem + 16);
+    unsigned long long *mbars = reinterpret_cast<unsigned long long *>(smem);   // [0] columns, [1] rows, [2] sums, [3] halos
+    const uint32_t mb_col = smem_addr(mbars), mb_row = smem_addr(mbars + 1), mb_red = smem_addr(mbars + 2);
+    const uint32_t mb_halo = smem_addr(mbars + 3);
+    cplx<T> *tw = reinterpret_cast<cplx<T> *>(smem + 32);
+    __shared__ RelaxAcc<T> racc[RELAX ? NT / 32 : 1];   // per warp
+    __shared__ T rpart[RELAX ? NC : 1][6];              // per CTA of the cluster
+    __shared__ T lam_s[2];
+    __shared__ int conv_s;
     __shared__ int bcast;   // rank 0's: the cluster's ticket, then whether a hand-over arrived
     load_twiddles<P>(tw, twP, tid, NT);
     if (tid == 0) {
         mbar_init(mb_col, 1);
         mbar_init(mb_row, 1);
+        mbar_init(mb_red, 1);
+        mbar_init(mb_halo, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        if (SEG && rank == 0) bcast = atomicAdd(ticket, 1);
+        if (SEG && !RELAX && rank == 0) bcast = atomicAdd(ticket, 1);
     }
     cluster.sync();   // every CTA runs, with its barriers initialised, before the first remote store
-    const int slot = SEG ? *cluster.map_shared_rank(&bcast, 0) : 0;
-    uint32_t phase = 0;
+    const int slot = SEG && !RELAX ? *cluster.map_shared_rank(&bcast, 0) : 0;
+    uint32_t phase = 0, hphase = 0;
     bool bailed = false;   // this thread's wait ran out once: it skips every later wait
-    const int sg_begin = SEG ? seg_off[slot] : 0, sg_end = SEG ? seg_off[slot + 1] : 1;
+    const int sg_begin = SEG && !RELAX ? seg_off[slot] : 0;
+    const int sg_end = RELAX ? 0x7fffffff : SEG ? seg_off[slot + 1] : 1;
     for (int sg = sg_begin; sg < sg_end; ++sg) {
-    const Segment seg = SEG ? segs[sg] : Segment{work[blockIdx.x / NC], 0, 0, 0, 0, nsteps_all};
+    Segment seg;
+    if constexpr (RELAX) {
+        // rank 0 takes the next turn of a replica that has not finished: -1 none left, -2 a wait expired
+        cluster.sync();
+        if (rank == 0 && tid == 0) {
+            int got = -1;
+            while (atomicAdd(rx.ndone, 0) < rx.nwork) {
+                const int k = atomicAdd(ticket, 1), rep = work[k % rx.nwork], turn = k / rx.nwork;
+                if ((long long)turn * rx.quantum >= rx.max_iter) break;
+                bool ok = false;
+                for (int it = 0; it < (1 << 22) && !ok; ++it) {
+                    ok = atomicAdd(flags + rep, 0) >= turn;
+                    if (!ok) __nanosleep(256);
+                }
+                if (!ok) {
+                    atomicOr(status, ND_DEV_TIMEOUT);
+                    got = -2;
+                    break;
+                }
+                __threadfence();
+                if (__ldcg(&rx.rio[rep].status) != 0) {
+                    got = rep;
+                    break;
+                }
+                atomicExch(flags + rep, 0x7fffffff);   // finished: its later turns wait for nothing
+            }
+            bcast = got;
+        }
+        cluster.sync();
+        seg = Segment{*cluster.map_shared_rank(&bcast, 0), 0, 1, 0, 0, 0};
+        if (seg.rep < 0) break;   // (the same for every CTA of the cluster)
+        seg.nsteps = min(rx.quantum, rx.max_iter - __ldcg(&rx.rio[seg.rep].iters));
+    } else if constexpr (SEG) {
+        seg = segs[sg];
+    } else {
+        seg = Segment{work[blockIdx.x / NC], 0, 0, 0, 0, nsteps_all};
+    }
     const long long nsteps = seg.nsteps;
     const Replica &r = reps[seg.rep];
-    if (SEG) {   // (the same for every CTA of the cluster)
+    if (SEG && !RELAX) {   // (the same for every CTA of the cluster)
         cluster.sync();   // the ticket is read; the previous segment's rows and columns are no longer used
         if (rank == 0 && tid == 0) {
             bcast = seg.wait ? (int)wait_flag(flags + seg.rep) : 1;
@@ -238,7 +316,23 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
         for (int i = tid; i < 4 * NTAB * KH; i += NT) {
             const int c = i / (NTAB * KH), rem = i - c * (NTAB * KH), j = rem / KH, ky = rem - j * KH;
             const int kx = j < SPC ? rank * SPC + j : P / 2;
-            gtab[i] = __ldg(Gc + (long long)c * KK + kx * KH + ky);
+            if constexpr (RELAX) {   // without the exchange
+                const double g = __ldg(r.Ghat64 + (long long)(4 + c) * KK + kx * KH + ky);
+                const double ex = c == 2 ? 0.0 : 2.0 * (__ldg(rx.twP64 + 2 * kx) + __ldg(rx.twP64 + 2 * ky));
+                gtab[i] = (T)fm(-ex, 1.0 / ((double)P * P), g);
+            } else {
+                gtab[i] = __ldg(Gc + (long long)c * KK + kx * KH + ky);
+            }
+        }
+    }
+    // relaxation: the rows of the neighbouring CTAs above and below, zero where there are none
+    T *const halo = wl;   // [2][3][Dpad]
+    const bool up = RELAX && rank > 0 && nloc > 0, down = RELAX && nloc > 0 && ylo + nloc < D;
+    if constexpr (RELAX) {
+        for (int i = tid; i < 2 * Dpad; i += NT) {
+            const int h = i / Dpad, x = i - h * Dpad, y = h ? ylo + nloc : ylo - 1;
+            const bool in = (h ? down : up) && x < D && r.mask[y * D + x];
+            V3Ptr<T>{halo + h * 3 * Dpad, Dpad}.st(x, in ? yg.ldcg((long long)y * Dpad + x) : vec3<T>{T(0), T(0), T(0)});
         }
     }
     // the CTA's cells: a contiguous range of the ascending cell list
@@ -268,15 +362,30 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     // packed pair: SPC + 1 entries of its own)
     const uint32_t bytes_col = (uint32_t)(3 * (D - nloc) * SPC * sizeof(cplx<T>));
     const uint32_t bytes_row = (uint32_t)(3 * nloc * (P / 2 + 1 - SPC - (rank == 0 ? 1 : 0)) * sizeof(cplx<T>));
+    T relX = T(0), relY = T(0);
+    if constexpr (RELAX) {
+        const RelaxIO *io = rx.rio + seg.rep;
+        relX = (T)io->X[0];
+        relY = (T)io->X[1];
+        if (tid == 0) {
+            lam_s[0] = (T)__ldcg(&io->lam[0]);
+            lam_s[1] = (T)__ldcg(&io->lam[1]);
+            conv_s = 0;
+        }
+    }
     __syncthreads();   // the state, the kernel's entries and the cell range are in place
     const int c0 = crange[0], c1 = crange[1];
+    T *const zl = reinterpret_cast<T *>(scratch);   // relaxation: neighbour counts (the FFT scratch is idle then)
+    T res_last = T(0);   // thread 0: the last sweep's residual
+    long long n = 0;
 
-    for (long long n = 0; n < nsteps; ++n) {
+    for (n = 0; n < nsteps; ++n) {
         const unsigned long long step = step_base + r.step0 + (unsigned long long)(seg.step_begin + n);
         for (int stage = 0; stage < ModeStages<MODE>::n; ++stage) {
             if (tid == 0) {
                 mbar_expect(mb_col, bytes_col);
                 mbar_expect(mb_row, bytes_row);
+                if (RELAX) mbar_expect(mb_red, (uint32_t)((NC - 1) * 6 * sizeof(T)));
             }
             // 1. forward rows of the CTA's own rows, sent to the column owners
             if constexpr (HR) {
@@ -486,10 +595,120 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
                 }
             }
             __syncthreads();
+            if constexpr (RELAX) {
+                // the sweep of k_fused's relaxation mode: trial alignment with the
+                // current multipliers (kept in the accumulator for the cells that
+                // they do not touch), sums over the cluster, one Newton step by
+                // every CTA alike, then the update
+                const StepParams<T> sp = step_params<T>(r);
+                const T *hr = reinterpret_cast<const T *>(spec);
+                const T eta = (T)rx.eta, rc2 = (T)rx.rc2, half = T(0.5) * (T)(D - 1);
+                const T l0 = lam_s[0], l1 = lam_s[1];
+                if (n > 0) {   // (the first sweep's halos were read from the caller's state)
+                    if (!bailed && !mbar_wait(mb_halo, hphase & 1)) {
+                        bailed = true;
+                        atomicOr(status, ND_DEV_TIMEOUT);
+                    }
+                    ++hphase;
+                }
+                RelaxAcc<T> a = {T(0), T(0), T(0), T(0), T(0), T(0)};
+                const vec3<T> zero3 = {T(0), T(0), T(0)};
+                for (int k = c0 + tid; k < c1; k += NT) {
+                    const int cell = __ldg(r.cells + k), y = cell / D, x = cell - y * D, lr = y - ylo;
+                    const long long mi = (long long)lr * Dpad + x, hi = (long long)lr * (2 * RS) + x;
+                    const vec3<T> m = ms.ld(mi);
+                    vec3<T> e = {hr[hi] + sp.chext[0], hr[2 * lcs + hi] + sp.chext[1], hr[4 * lcs + hi] + sp.chext[2]};
+                    T z = T(0);   // neighbours inside the disk (cells outside hold zero)
+                    auto add = [&](vec3<T> q) {
+                        const bool in = q.x != T(0) || q.y != T(0) || q.z != T(0);
+                        z += in ? T(1) : T(0);
+                        e.x += in ? q.x - m.x : T(0);
+                        e.y += in ? q.y - m.y : T(0);
+                        e.z += in ? q.z - m.z : T(0);
+                    };
+                    add(x > 0 ? ms.ld(mi - 1) : zero3);
+                    add(x + 1 < D ? ms.ld(mi + 1) : zero3);
+                    add(lr > 0 ? ms.ld(mi - Dpad) : V3Ptr<T>{halo, Dpad}.ld(x));
+                    add(lr + 1 < nloc ? ms.ld(mi + Dpad) : V3Ptr<T>{halo + 3 * Dpad, Dpad}.ld(x));
+                    const T dx = (T)x - half - relX, dy = (T)y - half - relY;
+                    // (y_n's place keeps e for the second alignment, the normals' the halos)
+                    ynv.st(mi, e);
+                    accv.st(mi, relax_cell<T>(m, e, fm(dx, dx, dy * dy) < rc2, dx, dy, l0, l1, eta, a, z));
+                    zl[mi] = z;
+                }
+                a.C0 = warp_sum_t(a.C0); a.C1 = warp_sum_t(a.C1); a.J00 = warp_sum_t(a.J00);
+                a.J01 = warp_sum_t(a.J01); a.J11 = warp_sum_t(a.J11); a.res = warp_max_t(a.res);
+                if ((tid & 31) == 0) racc[tid >> 5] = a;
+                __syncthreads();
+                if (tid < 6 * NC) {   // value v of this CTA to CTA q
+                    const int q = tid / 6, v = tid - 6 * q;
+                    T t = (&racc[0].C0)[v];
+                    for (int w = 1; w < NT / 32; ++w) {
+                        const T u = (&racc[w].C0)[v];
+                        t = v == 5 ? max(t, u) : t + u;
+                    }
+                    if (q == rank) rpart[q][v] = t;
+                    else st_async(cluster_addr(smem_addr(&rpart[rank][v]), q), t, cluster_addr(mb_red, q));
+                }
+                __syncthreads();
+                if (tid < 32) {
+                    if (!bailed && !mbar_wait(mb_red, (phase - 1) & 1)) {
+                        bailed = true;
+                        atomicOr(status, ND_DEV_TIMEOUT);
+                    }
+                    const int v = min(tid, 5);
+                    T t = rpart[0][v];
+                    for (int q = 1; q < NC; ++q) t = v == 5 ? max(t, rpart[q][v]) : t + rpart[q][v];
+                    const T C0 = __shfl_sync(0xffffffffu, t, 0), C1 = __shfl_sync(0xffffffffu, t, 1);
+                    const T J00 = __shfl_sync(0xffffffffu, t, 2), J01 = __shfl_sync(0xffffffffu, t, 3);
+                    const T J11 = __shfl_sync(0xffffffffu, t, 4), res = __shfl_sync(0xffffffffu, t, 5);
+                    if (tid == 0) {
+                        res_last = res;
+                        if (res < (T)rx.tol) {
+                            conv_s = 1;
+                        } else {
+                            const T det = fm(J00, J11, -(J01 * J01));
+                            if (det != T(0) && isfinite(det)) {
+                                lam_s[0] += -fm(J11, C0, -(J01 * C1)) / det;
+                                lam_s[1] += -fm(J00, C1, -(J01 * C0)) / det;
+                            }
+                        }
+                    }
+                }
+                __syncthreads();
+                if (conv_s) break;   // leaves the stage loop; the sweep loop stops below
+                const T m0 = lam_s[0], m1 = lam_s[1];
+                for (int k = c0 + tid; k < c1; k += NT) {
+                    const int cell = __ldg(r.cells + k), y = cell / D, x = cell - y * D, lr = y - ylo;
+                    const long long mi = (long long)lr * Dpad + x;
+                    const T dx = (T)x - half - relX, dy = (T)y - half - relY;
+                    vec3<T> mp = accv.ld(mi);   // this thread's own store
+                    if (fm(dx, dx, dy * dy) < rc2) {
+                        RelaxAcc<T> dummy = {T(0), T(0), T(0), T(0), T(0), T(0)};
+                        mp = relax_cell<T>(ms.ld(mi), ynv.ld(mi), true, dx, dy, m0, m1, eta, dummy, zl[mi]);
+                    }
+                    ms.st(mi, mp);
+                }
+                __syncthreads();
+                if (n + 1 < nsteps) {   // the edge rows to the neighbours (which have read theirs: their sums arrived)
+                    if (tid == 0) mbar_expect(mb_halo, (uint32_t)((int)up + (int)down) * 3 * D * sizeof(T));
+                    for (int i = tid; i < 3 * D; i += NT) {
+                        const int c = i / D, x = i - c * D;
+                        if (up)   // my first row is the row below the CTA above
+                            st_async(cluster_addr(smem_addr(halo + (3 + c) * Dpad + x), rank - 1),
+                                     msl[c * lms + x], cluster_addr(mb_halo, rank - 1));
+                        if (down)
+                            st_async(cluster_addr(smem_addr(halo + c * Dpad + x), rank + 1),
+                                     msl[c * lms + (long long)(nloc - 1) * Dpad + x], cluster_addr(mb_halo, rank + 1));
+                    }
+                }
+                continue;
+            }
             // the per-cell epilogue of the CTA's cells
             const StepParams<T> sp = step_params<T>(r);
             const vec3<T> cx = step_chext<T>(r, sp, step);
             const T *hr = reinterpret_cast<const T *>(spec);
+            if constexpr (!RELAX)
             for (int k = c0 + tid; k < c1; k += NT) {
                 const int cell = __ldg(r.cells + k);
                 const int y = cell / D, x = cell - y * D, lr = y - ylo;
@@ -500,19 +719,32 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
             }
             __syncthreads();
         }
+        if (RELAX && conv_s) break;
     }
     // the final state of the CTA's cells back to the caller's buffer
     for (int k = c0 + tid; k < c1; k += NT) {
         const int cell = __ldg(r.cells + k);
         const int y = cell / D, x = cell - y * D;
-        yg.st((long long)y * Dpad + x, ynv.ld((long long)(y - ylo) * Dpad + x));
+        const long long mi = (long long)(y - ylo) * Dpad + x;
+        yg.st((long long)y * Dpad + x, RELAX ? ms.ld(mi) : ynv.ld(mi));
+    }
+    if (RELAX && rank == 0 && tid == 0) {
+        RelaxIO *io = rx.rio + seg.rep;
+        const int iters = __ldcg(&io->iters) + (int)n;
+        __stcg(&io->lam[0], (double)lam_s[0]);
+        __stcg(&io->lam[1], (double)lam_s[1]);
+        __stcg(&io->resid, (double)res_last);
+        __stcg(&io->iters, iters);
+        if (conv_s) __stcg(&io->status, 0);
+        if (conv_s || iters >= rx.max_iter) atomicAdd(rx.ndone, 1);
     }
     if (SEG && seg.signal) {   // every CTA's rows are written before the flag
         __threadfence();
         cluster.sync();
         if (rank == 0 && tid == 0) {
             __threadfence();
-            atomicExch(flags + seg.rep, 1);
+            if (RELAX) atomicAdd(flags + seg.rep, 1);
+            else atomicExch(flags + seg.rep, 1);
         }
     }
     }
@@ -551,9 +783,11 @@ static cudaError_t launch_cluster_t(const LaunchArgs &a, int maxD, int maxDpad)
     cudaLaunchAttribute attr[1];
     cudaError_t e = cluster_config<P, T, MODE, NC, SEG>(cfg, attr, SEG ? a.ncta : a.nwork, sm, a.stream);
     if (e != cudaSuccess) return e;
+    const ClusterRelax rx = {a.rio, (const double *)a.tw64, a.eta, a.tol, a.rc2, a.max_iter, a.quantum, a.nwork,
+                             a.flags ? a.flags + a.n_rep + 1 : nullptr};
     return cudaLaunchKernelEx(&cfg, k_cluster<P, T, MODE, NC, SEG>, a.reps, a.work, (T *)a.y, (const cplx<T> *)a.tw,
                               a.nsteps, a.step_base, a.use_wbuf, a.status, reinterpret_cast<const Segment *>(a.segs),
-                              a.seg_off, a.flags, a.flags ? a.flags + a.n_rep : nullptr);
+                              a.seg_off, a.flags, a.flags ? a.flags + a.n_rep : nullptr, rx);
 }
 
 // Clusters of the size class that can be resident at once (0: the cluster
@@ -585,6 +819,7 @@ static cudaError_t launch_cluster_p(const LaunchArgs &a, int maxD, int maxDpad)
     if (a.mode == M_HEUN)
         return a.segs ? launch_cluster_t<P, T, M_HEUN, NC, true>(a, maxD, maxDpad)
                       : launch_cluster_t<P, T, M_HEUN, NC, false>(a, maxD, maxDpad);
+    if (a.mode == M_RELAX) return launch_cluster_t<P, T, M_RELAX, NC, true>(a, maxD, maxDpad);
     return cudaErrorInvalidValue;
 }
 

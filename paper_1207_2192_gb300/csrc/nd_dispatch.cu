@@ -5,6 +5,8 @@ namespace nd {
 
 cudaError_t upload_tw_fused_f32(const double *, const double *);
 cudaError_t upload_tw_fused_f64(const double *, const double *);
+cudaError_t upload_tw_cluster_f32(const double *, const double *);
+cudaError_t upload_tw_cluster_f64(const double *, const double *);
 cudaError_t upload_tw_glob_f32(const double *, const double *);
 cudaError_t upload_tw_glob_f64(const double *, const double *);
 cudaError_t upload_tw_spectra(const double *, const double *);
@@ -31,6 +33,8 @@ cudaError_t upload_twiddle_constants(const double *re, const double *im)
     cudaError_t e;
     if ((e = upload_tw_fused_f32(re, im)) != cudaSuccess) return e;
     if ((e = upload_tw_fused_f64(re, im)) != cudaSuccess) return e;
+    if ((e = upload_tw_cluster_f32(re, im)) != cudaSuccess) return e;
+    if ((e = upload_tw_cluster_f64(re, im)) != cudaSuccess) return e;
     if ((e = upload_tw_glob_f32(re, im)) != cudaSuccess) return e;
     if ((e = upload_tw_spectra(re, im)) != cudaSuccess) return e;
     return upload_tw_glob_f64(re, im);

@@ -243,16 +243,19 @@ template <typename T> __device__ __forceinline__ T warp_max_t(T v)
 // and the exact 2x2 Jacobian of C(m'(lambda)) for cells of the window.
 template <typename T> struct RelaxAcc { T C0, C1, J00, J01, J11, res; };
 
+// The field is b + z m; z, a multiple of m that turns nothing, is left out of
+// the torque (0 where the caller's b holds all of the field).
 template <typename T>
 __device__ __forceinline__ vec3<T> relax_cell(vec3<T> m, vec3<T> b, bool inW, T dx, T dy, T l0, T l1, T eta,
-                                              RelaxAcc<T> &acc)
+                                              RelaxAcc<T> &acc, T z = T(0))
 {
-    vec3<T> e = b;
-    if (inW) e.z = fm(l0 * T(2) * m.z, dx, fm(l1 * T(2) * m.z, dy, e.z));
+    vec3<T> f = b;
+    if (inW) f.z = fm(l0 * T(2) * m.z, dx, fm(l1 * T(2) * m.z, dy, f.z));
+    const vec3<T> e = axpy3(z, m, f);
     const T en = dsqrt<T>(dot3(e, e));
     const vec3<T> u = {e.x / en, e.y / en, e.z / en};
-    const vec3<T> tq = cross3(m, u);
-    acc.res = max(acc.res, dsqrt<T>(dot3(tq, tq)));
+    const vec3<T> tq = cross3(m, f);
+    acc.res = max(acc.res, dsqrt<T>(dot3(tq, tq)) / en);
     const T om = T(1) - eta;
     const vec3<T> v = {fm(eta, u.x, om * m.x), fm(eta, u.y, om * m.y), fm(eta, u.z, om * m.z)};
     const T vn = dsqrt<T>(dot3(v, v));

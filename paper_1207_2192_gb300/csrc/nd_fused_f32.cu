@@ -1,5 +1,5 @@
 // nd_fused_f32.cu -- instantiations of the fused on-chip kernel in FP32.
-#include "nd_cluster.cuh"
+#include "nd_field_impl.cuh"
 
 namespace nd {
 
@@ -52,36 +52,6 @@ cudaError_t launch_fused_f32(int P, const LaunchArgs &a)
     case 128: return launch_fused_p<128, float>(a);
     default: return cudaErrorInvalidValue;
     }
-}
-
-// Cluster plans: NC = 8 CTAs for every on-chip size, NC = 16 for P >= 32
-// (where the P/2 column slots split over 16 CTAs), and P = 192 and 256 on 16
-// CTAs (spectra too large for one CTA's shared memory).
-#define ND_CLUSTER_CASES(X)      \
-    X(16, 8) X(32, 8) X(64, 8) X(128, 8) X(32, 16) X(64, 16) X(128, 16) X(192, 16) X(256, 16)
-
-size_t cluster_smem_f32(int P, int D, int Dpad, bool wbuf, int nc)
-{
-#define X(p, n) if (P == p && nc == n) return cluster_smem_bytes<p, float, n>(D, Dpad, wbuf);
-    ND_CLUSTER_CASES(X)
-#undef X
-    return (size_t)-1;
-}
-
-int cluster_max_active_f32(int P, int D, int Dpad, bool wbuf, int nc)
-{
-#define X(p, n) if (P == p && nc == n) return cluster_max_active_t<p, float, n>(D, Dpad, wbuf);
-    ND_CLUSTER_CASES(X)
-#undef X
-    return 0;
-}
-
-cudaError_t launch_cluster_f32(int P, const LaunchArgs &a, int maxD, int maxDpad, int nc)
-{
-#define X(p, n) if (P == p && nc == n) return launch_cluster_p<p, float, n>(a, maxD, maxDpad);
-    ND_CLUSTER_CASES(X)
-#undef X
-    return cudaErrorInvalidValue;
 }
 
 }  // namespace nd

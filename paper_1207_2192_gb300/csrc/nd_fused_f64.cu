@@ -1,5 +1,5 @@
 // nd_fused_f64.cu -- instantiations of the fused on-chip kernel in FP64.
-#include "nd_cluster.cuh"
+#include "nd_field_impl.cuh"
 
 namespace nd {
 
@@ -15,7 +15,6 @@ size_t fused_smem_f64(int P, int D, int Dpad, bool wbuf, int variant)
     case 16: return fused_smem_bytes<16, double>(D, Dpad, nt, wbuf);
     case 32: return fused_smem_bytes<32, double>(D, Dpad, nt, wbuf);
     case 64: return fused_smem_bytes<64, double>(D, Dpad, nt, wbuf);
-    case 128: return fused_smem_bytes<128, double>(D, Dpad, nt, wbuf);
     default: return (size_t)-1;
     }
 }
@@ -36,7 +35,6 @@ int fused_blocks_per_sm_f64(int P, int mode, size_t smem, int variant)
     case 16: return occ_p<16>(mode, smem, variant);
     case 32: return occ_p<32>(mode, smem, variant);
     case 64: return occ_p<64>(mode, smem, variant);
-    case 128: return occ_p<128>(mode, smem, variant);
     default: return 0;
     }
 }
@@ -49,38 +47,8 @@ cudaError_t launch_fused_f64(int P, const LaunchArgs &a)
     case 16: return launch_fused_p<16, double>(a);
     case 32: return launch_fused_p<32, double>(a);
     case 64: return launch_fused_p<64, double>(a);
-    case 128: return launch_fused_p<128, double>(a);
     default: return cudaErrorInvalidValue;
     }
-}
-
-// Cluster plans: NC = 8 CTAs for every on-chip size, NC = 16 for P >= 32
-// (where the P/2 column slots split over 16 CTAs).
-#define ND_CLUSTER_CASES(X)      \
-    X(16, 8) X(32, 8) X(64, 8) X(128, 8) X(32, 16) X(64, 16) X(128, 16)
-
-size_t cluster_smem_f64(int P, int D, int Dpad, bool wbuf, int nc)
-{
-#define X(p, n) if (P == p && nc == n) return cluster_smem_bytes<p, double, n>(D, Dpad, wbuf);
-    ND_CLUSTER_CASES(X)
-#undef X
-    return (size_t)-1;
-}
-
-int cluster_max_active_f64(int P, int D, int Dpad, bool wbuf, int nc)
-{
-#define X(p, n) if (P == p && nc == n) return cluster_max_active_t<p, double, n>(D, Dpad, wbuf);
-    ND_CLUSTER_CASES(X)
-#undef X
-    return 0;
-}
-
-cudaError_t launch_cluster_f64(int P, const LaunchArgs &a, int maxD, int maxDpad, int nc)
-{
-#define X(p, n) if (P == p && nc == n) return launch_cluster_p<p, double, n>(a, maxD, maxDpad);
-    ND_CLUSTER_CASES(X)
-#undef X
-    return cudaErrorInvalidValue;
 }
 
 }  // namespace nd

@@ -26,6 +26,7 @@ struct LaunchArgs {
     void *spec = nullptr;            // global-path spectrum scratch
     double *red = nullptr;           // per-replica reduction output (energy), indexed by replica
     const void *tw = nullptr;        // length-P twiddle table exp(-2 pi i k/P) of the precision
+    const void *tw64 = nullptr;      // the same table in FP64 (cluster relaxation)
     long long nsteps = 1;
     unsigned long long step_base = 0;
     size_t smem = 0;
@@ -38,6 +39,7 @@ struct LaunchArgs {
     double *part = nullptr;          // global-path relaxation partial sums: [replicas][kRelaxBlocks][6]
     double eta = 0.5, tol = 1e-6, rc2 = 0.0;
     int max_iter = 0;
+    int quantum = 0;                 // cluster plans: sweeps of one turn of a replica
     // time-sliced schedule (fused steppers): ncta CTAs run the segments
     // segs[seg_off[b] .. seg_off[b+1]) and hand replicas over through flags
     const void *segs = nullptr;

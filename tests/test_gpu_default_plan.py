@@ -46,3 +46,30 @@ def test_time_sliced_clusters_with_disks_of_different_sizes(method):
     reps = [4, 3, 5, 4, 3]
     assert torch.equal(states(disks, reps, nd.ND_FP32, 200, method), states(disks, reps, nd.ND_FP32, 0, method))
     assert torch.equal(states(disks, reps, nd.ND_FP32, 201, method), states(disks, reps, nd.ND_FP32, 0, method))
+
+
+@pytest.mark.parametrize("prec", [nd.ND_FP32, nd.ND_FP64])
+@pytest.mark.parametrize("tol,max_iter", [(1e-12, 300), (2e-3, 5000)])
+def test_replicas_relaxing_in_turns_end_where_they_do_alone(prec, tol, max_iter):
+    """More replicas than clusters relax in turns of some sweeps: each ends
+    with the state, multipliers and sweep count it has in a small handle,
+    whether its sweeps run out or it converges."""
+    disk = Disk(30e-9, 6e-9)
+    B = 20
+    X = np.stack([np.linspace(0.0, 12e-9, B), np.linspace(-2e-9, 2e-9, B)], 1)
+
+    def relax(sel):
+        h = Nanodisk([disk], [len(sel)], prec)
+        m = h.empty_device()
+        h.init_vortex(m, np.zeros((len(sel), 2)))
+        rc, U, lam, it = h.relax(m, X[sel], tol=tol, max_iter=max_iter)
+        assert nd.nd_check_status(h.h) == nd.ND_OK
+        assert rc == (nd.ND_ERR_NOT_CONVERGED if (it == max_iter).any() else nd.ND_OK)
+        return m, U, lam, it
+
+    m, U, lam, it = relax(np.arange(B))
+    assert (it == max_iter).all() if tol < 1e-9 else len(set(it)) > 1
+    parts = [relax(np.arange(k, k + 5)) for k in range(0, B, 5)]
+    assert torch.equal(m, torch.cat([p[0] for p in parts]))
+    assert np.array_equal(lam, np.concatenate([p[2] for p in parts]))
+    assert np.array_equal(it, np.concatenate([p[3] for p in parts]))
