@@ -167,9 +167,9 @@ int nd_set_field_schedule(nd_handle *h, int d, long long n_steps, const double *
  * b has the state layout; cells outside the disks are written as zero. */
 int nd_effective_field(nd_handle *h, const void *m, void *b, void *stream);
 
-/* Energy of Eq. Hmm for every replica, in units of J = 2AL, evaluated with a
- * double-precision field and double-precision sums whatever the handle's
- * precision: E_out[r] = -{ sum_pairs m_i . m_j + (a^2/lambda^2) sum_i
+/* Energy of Eq. Hmm for every replica, in units of J = 2AL, evaluated with
+ * double-precision transforms and sums (in the spectral domain) whatever the
+ * handle's precision: E_out[r] = -{ sum_pairs m_i . m_j + (a^2/lambda^2) sum_i
  * (h_ext + h^M_i / 2) . m_i }.  If dEdL_out is not NULL it receives, per
  * replica, the derivative of the energy in joules, E = J E_out, with respect
  * to the thickness L at fixed m (J/m): dE/dL = 2A E_out + J d(E/J)/dL, the

@@ -16,7 +16,8 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libnanodisk.so")
 SOURCES = ["nd_fused_f32.cu", "nd_fused_f64.cu", "nd_cluster_f32.cu", "nd_cluster_f64.cu", "nd_glob_f32.cu", "nd_glob_f64.cu",
-           "nd_dispatch.cu", "nd_aux.cu", "nd_api.cu", "nd_noalloc.cu", "nd_spectra.cu"]
+           "nd_dispatch.cu", "nd_aux.cu", "nd_api.cu", "nd_noalloc.cu", "nd_spectra.cu",
+           "nd_energy.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # The stepping, relaxation and field kernels write their fused multiply-adds
 # out (fm in nd_common.cuh): without contraction by the compiler every

@@ -71,8 +71,7 @@ struct SizeClass {
     std::vector<int> reps;     // replica indices
     int *work_d = nullptr;     // device copy of reps
     bool fused_main = false;   // fused kernel in the handle precision
-    bool fused_fp64 = false;   // fused kernel in FP64 (energy)
-    size_t smem_main = 0, smem_fp64 = 0;
+    size_t smem_main = 0;
     size_t smem_wbuf = 0;      // fused Heun with the normals kept in shared memory (0: does not fit)
     int plan[2] = {-1, -1};    // stepping plan for RK4 / Heun: -1 default (default_plan), 0..2 fused variant, kPlanGlobal, kPlanCluster
     // time-sliced schedule, cached per (mode, n_steps)
@@ -155,8 +154,9 @@ struct nd_handle {
     void *ms = nullptr;                   // handle-precision stage state (global path)
     void *spec = nullptr;                 // spectrum scratch (global path), sized for FP64
     void *stage_in = nullptr, *stage_out = nullptr;   // staging of host buffers
-    double *y64 = nullptr, *ms64 = nullptr;           // FP64 copies (energy of FP32 handles)
-    double *red_d = nullptr;              // [B] reductions
+    double *red_d = nullptr;              // [B][2] energies and their thickness derivatives
+    double *energy_part = nullptr;        // [B][P/2][2] partial sums of the energies (largest P)
+    unsigned *energy_done = nullptr;      // [B] counters of finished partial sums
     double *red_h = nullptr;              // pinned [B * 4]
     double *aux_d = nullptr;              // [B * 4] small per-replica inputs/outputs
     int *aux_i = nullptr;                 // [B * 2]
@@ -196,8 +196,6 @@ static int setup_class_paths(nd_handle *h)
         // 1 KiB of the per-block limit is left for the kernels' static shared variables
         c.smem_main = fused_smem(c.P, h->prec, c.maxD, c.maxDpad);
         c.fused_main = c.smem_main != (size_t)-1 && c.smem_main + 1024 <= h->max_smem;
-        c.smem_fp64 = fused_smem(c.P, ND_PREC_FP64, c.maxD, c.maxDpad);
-        c.fused_fp64 = c.smem_fp64 != (size_t)-1 && c.smem_fp64 + 1024 <= h->max_smem;
     }
     return ND_OK;
 }
@@ -217,10 +215,8 @@ static void upload_reps(nd_handle *h, cudaStream_t st)
     cudaEventRecord(h->slot_ev[h->slot], st);
 }
 
-enum { TAB_MAIN = 0, TAB_DL = 1 };
-
 static void fill_reps(nd_handle *h, bool fp64_kernel, double dt_seconds, const double *Tk,
-                      const unsigned long long *seed, unsigned long long step0, int table = TAB_MAIN)
+                      const unsigned long long *seed, unsigned long long step0)
 {
     const int B = (int)h->rep_disk.size();
     next_slot(h);
@@ -232,12 +228,13 @@ static void fill_reps(nd_handle *h, bool fp64_kernel, double dt_seconds, const d
         R.disk = h->rep_disk[r];
         R.state_off = h->rep_off[r];
         R.spec_off = h->rep_spec_off[r];
-        R.Ghat = table == TAB_DL ? (const void *)d.ghatL : (fp64_kernel ? (const void *)d.ghat64 : (const void *)d.ghat32);
+        R.Ghat = fp64_kernel ? (const void *)d.ghat64 : (const void *)d.ghat32;
         R.Ghat64 = d.ghat64;
+        R.GhatL = d.ghatL;
         R.mask = d.mask_d;
         R.cells = d.cells_d;
         R.ncells = d.C;
-        for (int k = 0; k < 3; ++k) R.chext[k] = table == TAB_DL ? 0.0 : d.cfac * d.h[k];
+        for (int k = 0; k < 3; ++k) R.chext[k] = d.cfac * d.h[k];
         R.alpha = h->alpha[r];
         R.dtau = d.desc.gamma * d.B0 * dt_seconds;
         double Ts = Tk ? kBoltzmann * Tk[r] / d.J : 0.0;
@@ -249,9 +246,9 @@ static void fill_reps(nd_handle *h, bool fp64_kernel, double dt_seconds, const d
         R.falpha = (float)R.alpha;
         R.fdtau = (float)R.dtau;
         R.fsigma = (float)R.sigma;
-        R.fsched = table == TAB_DL ? nullptr : d.sched32;
-        R.dsched = table == TAB_DL ? nullptr : d.sched64;
-        R.nsched = table == TAB_DL ? 0 : d.nsched;
+        R.fsched = d.sched32;
+        R.dsched = d.sched64;
+        R.nsched = d.nsched;
     }
 }
 
@@ -399,12 +396,11 @@ static int class_segments(SizeClass &c, int mode, long long nsteps, int nslots)
     return ND_OK;
 }
 
-// Run one mode over all replicas.  fp64 selects the FP64 kernels (with y a
-// double buffer of the state layout), otherwise the handle precision.
-static int run_mode(nd_handle *h, int mode, bool fp64, void *y, void *out, long long nsteps, cudaStream_t st,
+// Run one mode over all replicas in the handle's precision.
+static int run_mode(nd_handle *h, int mode, void *y, void *out, long long nsteps, cudaStream_t st,
                     const Replica *reps = nullptr, int only_class = -1)
 {
-    const int prec = fp64 ? ND_PREC_FP64 : (h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32);
+    const int prec = h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32;
     // The stepping kernels of the size classes are independent (each touches
     // only its replicas' state and scratch), so they run side by side on
     // forked streams: a class fills only the SMs of its replicas.  Not when a
@@ -431,15 +427,14 @@ static int run_mode(nd_handle *h, int mode, bool fp64, void *y, void *out, long 
         a.nwork = (int)c.reps.size();
         a.y = y;
         a.out = out;
-        a.red = h->red_d;
         a.nsteps = nsteps;
         a.step_base = 0;
         a.stream = st;
         a.tw = (prec == ND_PREC_FP64) ? h->tw64[c.P] : h->tw32[c.P];
         a.smem_optin = (int)h->max_smem;
         a.n_sm = h->n_sm;
-        bool fused = fp64 ? c.fused_fp64 : c.fused_main;
-        const bool stepping = (mode == M_HEUN || mode == M_RK4) && !fp64;
+        bool fused = c.fused_main;
+        const bool stepping = mode == M_HEUN || mode == M_RK4;
         int variant = 0;
         int cluster_nc = 0;
         if (stepping) {
@@ -469,18 +464,18 @@ static int run_mode(nd_handle *h, int mode, bool fp64, void *y, void *out, long 
             }
             ND_CUDA(launch_cluster(c.P, prec, a, c.maxD, c.maxDpad, cluster_nc));
         } else if (fused) {
-            a.smem = fp64 ? c.smem_fp64 : c.smem_main;
+            a.smem = c.smem_main;
             a.status = h->status_d;
             a.variant = variant;
             if (variant != 0) a.smem = fused_smem(c.P, prec, c.maxD, c.maxDpad, false, variant);
-            if (mode == M_HEUN && !fp64) {
+            if (mode == M_HEUN) {
                 const size_t w = variant == 0 ? c.smem_wbuf : fused_smem(c.P, prec, c.maxD, c.maxDpad, true, variant);
                 if (w && w != (size_t)-1 && w + 1024 <= h->max_smem) {
                     a.smem = w;
                     a.use_wbuf = 1;
                 }
             }
-            if ((mode == M_HEUN || mode == M_RK4) && !fp64 && nsteps >= 2) {
+            if (stepping && nsteps >= 2) {
                 const int per_sm = fused_blocks_per_sm(c.P, prec, mode, a.smem, variant);
                 const int ncta = per_sm * h->n_sm;
                 const int Bc = (int)c.reps.size();
@@ -495,7 +490,7 @@ static int run_mode(nd_handle *h, int mode, bool fp64, void *y, void *out, long 
             }
             ND_CUDA(launch_fused(c.P, prec, a));
         } else {
-            a.ms = fp64 ? (void *)h->ms64 : h->ms;
+            a.ms = h->ms;
             a.spec = h->spec;
             if (!a.ms || !a.spec) return fail(ND_ERR_ARG, "global-path buffers are not allocated");
             ND_CUDA(launch_global(c.P, prec, a, c.maxD));
@@ -688,7 +683,7 @@ int nd_create_disk(const nd_disk_desc *disks, int n_disks, const int *replicas_p
         if ((e = cudaEventCreateWithFlags(&h->slot_ev[k], cudaEventDisableTiming)) != cudaSuccess)
             return cuda_fail(e, "cudaEventCreate");
     if ((e = cudaMalloc(&h->reps_d, sizeof(Replica) * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
-    if ((e = cudaMalloc(&h->red_d, sizeof(double) * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
+    if ((e = cudaMalloc(&h->red_d, sizeof(double) * 2 * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = cudaMallocHost(&h->red_h, sizeof(double) * 4 * B)) != cudaSuccess) return cuda_fail(e, "cudaMallocHost");
     if ((e = cudaMalloc(&h->aux_d, sizeof(double) * 4 * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = cudaMalloc(&h->aux_i, sizeof(int) * 2 * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
@@ -706,16 +701,11 @@ int nd_create_disk(const nd_disk_desc *disks, int n_disks, const int *replicas_p
         for (int r = 0; r < B; ++r) av[r] = h->disks[h->rep_disk[r]].desc.a;
         cudaMemcpy(h->a_rep, av.data(), sizeof(double) * B, cudaMemcpyHostToDevice);
     }
-    bool any_global = false, any_global64 = false;
-    for (auto &c : h->classes) { any_global |= !c.fused_main; any_global64 |= !c.fused_fp64; }
-    if (any_global || any_global64) {
-        if ((e = cudaMalloc(&h->spec, sizeof(double) * 2 * h->spec_words)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
-    }
+    bool any_global = false;
+    for (auto &c : h->classes) any_global |= !c.fused_main;
+    if (any_global && (e = cudaMalloc(&h->spec, sizeof(double) * 2 * h->spec_words)) != cudaSuccess)
+        return cuda_fail(e, "cudaMalloc");
     if (any_global && (e = cudaMalloc(&h->ms, h->elt * h->state_elems)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
-    if (h->prec == ND_FP32 && (e = cudaMalloc((void **)&h->y64, sizeof(double) * h->state_elems)) != cudaSuccess)
-        return cuda_fail(e, "cudaMalloc");
-    if (any_global64 && (e = cudaMalloc((void **)&h->ms64, sizeof(double) * h->state_elems)) != cudaSuccess)
-        return cuda_fail(e, "cudaMalloc");
     for (int d = 0; d < n_disks; ++d) {
         DiskInfo &di = h->disks[d];
         const size_t kh = ghat_table_entries(di.P);
@@ -775,8 +765,8 @@ void nd_destroy(nd_handle *h)
     cudaFree(h->spec);
     cudaFree(h->stage_in);
     cudaFree(h->stage_out);
-    cudaFree(h->y64);
-    cudaFree(h->ms64);
+    cudaFree(h->energy_part);
+    cudaFree(h->energy_done);
     delete h;
 }
 
@@ -907,7 +897,7 @@ int nd_effective_field(nd_handle *h, const void *m, void *b, void *stream)
     ND_CUDA(cudaMemsetAsync(bd, 0, (size_t)h->state_elems * h->elt, st));
     fill_reps(h, h->prec == ND_FP64, 0.0, nullptr, nullptr, 0);
     upload_reps(h, st);
-    if (int rc = run_mode(h, M_FIELD, false, md, bd, 1, st)) return rc;
+    if (int rc = run_mode(h, M_FIELD, md, bd, 1, st)) return rc;
     return stage_out(h, b, bd, st);
 }
 
@@ -919,31 +909,39 @@ int nd_energy(nd_handle *h, const void *m, double *E_out, double *dEdL_out, void
     void *md = nullptr;
     if (int rc = stage_in(h, m, &md, true, st, &h->stage_in)) return rc;
     const int B = (int)h->rep_disk.size();
-    void *y64 = md;
-    if (h->prec == ND_FP32) {
-        ND_CUDA(launch_convert(ND_PREC_FP64, md, h->y64, (size_t)h->state_elems, st));
-        y64 = h->y64;
+    if (int rc = ensure_alloc(&h->spec, sizeof(double) * 2 * h->spec_words)) return rc;
+    if (!h->energy_part) {
+        int maxP = 0;
+        for (auto &c : h->classes) maxP = std::max(maxP, c.P);
+        if (int rc = ensure_alloc((void **)&h->energy_done, sizeof(unsigned) * B)) return rc;
+        ND_CUDA(cudaMemsetAsync(h->energy_done, 0, sizeof(unsigned) * B, st));
+        if (int rc = ensure_alloc((void **)&h->energy_part, sizeof(double) * (size_t)maxP * B)) return rc;
     }
     fill_reps(h, true, 0.0, nullptr, nullptr, 0);
     upload_reps(h, st);
-    ND_CUDA(cudaMemsetAsync(h->red_d, 0, sizeof(double) * B, st));
-    if (int rc = run_mode(h, M_ENERGY, true, y64, nullptr, 1, st)) return rc;
-    ND_CUDA(cudaMemcpyAsync(h->red_h, h->red_d, sizeof(double) * B, cudaMemcpyDeviceToHost, st));
+    for (auto &c : h->classes) {
+        EnergyArgs a;
+        a.reps = h->reps_d;
+        a.work = c.work_d;
+        a.nwork = (int)c.reps.size();
+        a.maxD = c.maxD;
+        a.with_dl = dEdL_out ? 1 : 0;
+        a.m = md;
+        a.spec = h->spec;
+        a.tw = h->tw64[c.P];
+        a.part = h->energy_part;
+        a.done = h->energy_done;
+        a.out = h->red_d;
+        a.stream = st;
+        ND_CUDA(launch_energy(c.P, h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32, a));
+    }
+    ND_CUDA(cudaMemcpyAsync(h->red_h, h->red_d, sizeof(double) * 2 * B, cudaMemcpyDeviceToHost, st));
     ND_CUDA(cudaStreamSynchronize(st));
-    for (int r = 0; r < B; ++r) E_out[r] = h->red_h[r];
-    if (dEdL_out) {
-        // -1/2 sum_i m_i . (c dh^M/dl)_i with the derivative kernel = d(E/J)/dl at fixed m;
-        // then dE/dL = 2A E/J + J d(E/J)/dl / a  (E = J E/J, J = 2AL)
-        fill_reps(h, true, 0.0, nullptr, nullptr, 0, TAB_DL);
-        upload_reps(h, st);
-        ND_CUDA(cudaMemsetAsync(h->red_d, 0, sizeof(double) * B, st));
-        if (int rc = run_mode(h, M_ENERGY, true, y64, nullptr, 1, st)) return rc;
-        ND_CUDA(cudaMemcpyAsync(h->red_h, h->red_d, sizeof(double) * B, cudaMemcpyDeviceToHost, st));
-        ND_CUDA(cudaStreamSynchronize(st));
-        for (int r = 0; r < B; ++r) {
-            const DiskInfo &d = h->disks[h->rep_disk[r]];
-            dEdL_out[r] = 2.0 * d.desc.A * E_out[r] + d.J * h->red_h[r] / d.desc.a;
-        }
+    for (int r = 0; r < B; ++r) {
+        const DiskInfo &d = h->disks[h->rep_disk[r]];
+        E_out[r] = h->red_h[2 * r];
+        // dE/dL = 2A E/J + J d(E/J)/dl / a  (E = J E/J, J = 2AL, l = L/a)
+        if (dEdL_out) dEdL_out[r] = 2.0 * d.desc.A * E_out[r] + d.J * h->red_h[2 * r + 1] / d.desc.a;
     }
     return ND_OK;
 }
@@ -959,7 +957,7 @@ int nd_step_rk4(nd_handle *h, void *m, long long n_steps, double dt_seconds, voi
     if (n_steps > 0) {
         fill_reps(h, h->prec == ND_FP64, dt_seconds, nullptr, nullptr, h->rk4_step);
         upload_reps(h, st);
-        if (int rc = run_mode(h, M_RK4, false, md, nullptr, n_steps, st)) return rc;
+        if (int rc = run_mode(h, M_RK4, md, nullptr, n_steps, st)) return rc;
         h->rk4_step += (unsigned long long)n_steps;
     }
     return stage_out(h, m, md, st);
@@ -980,7 +978,7 @@ int nd_step_heun(nd_handle *h, void *m, long long n_steps, double dt_seconds, co
     if (n_steps > 0) {
         fill_reps(h, h->prec == ND_FP64, dt_seconds, T_kelvin, seed, step0);
         upload_reps(h, st);
-        if (int rc = run_mode(h, M_HEUN, false, md, nullptr, n_steps, st)) return rc;
+        if (int rc = run_mode(h, M_HEUN, md, nullptr, n_steps, st)) return rc;
     }
     return stage_out(h, m, md, st);
 }
@@ -1045,7 +1043,6 @@ int nd_relax_constrained(nd_handle *h, void *m, const double *X, double tol, int
         a.work = c.work_d;
         a.nwork = (int)c.reps.size();
         a.y = md;
-        a.red = h->red_d;
         a.tw = (prec == ND_PREC_FP64) ? h->tw64[c.P] : h->tw32[c.P];
         a.smem = c.smem_main;
         a.stream = st;
@@ -1592,7 +1589,7 @@ static int tune_run(std::vector<TuneItem> &items, double dt, long long n_steps, 
         const bool heun = it.mode == M_HEUN;
         fill_reps(it.h, it.h->prec == ND_FP64, dt, heun ? it.T.data() : nullptr, heun ? it.sd.data() : nullptr, 0);
         upload_reps(it.h, s);
-        if (int rc = run_mode(it.h, it.mode, false, it.tmp, nullptr, n_steps, s, nullptr, only_class)) return rc;
+        if (int rc = run_mode(it.h, it.mode, it.tmp, nullptr, n_steps, s, nullptr, only_class)) return rc;
         if (many) {
             ND_CUDA(cudaEventRecord(joins[k], s));
             ND_CUDA(cudaStreamWaitEvent(st0, joins[k], 0));
@@ -1849,7 +1846,7 @@ int nd_graph_create(nd_handle *h, void *m, int method, long long n_steps, double
         Replica *r2 = nullptr;
         cudaMalloc(&r2, sizeof(Replica) * B);
         cudaMemcpy(r2, g->reps, sizeof(Replica) * B, cudaMemcpyDeviceToDevice);
-        int rc = run_mode(h, mode, false, tmp, nullptr, n_steps, 0, r2);
+        int rc = run_mode(h, mode, tmp, nullptr, n_steps, 0, r2);
         cudaDeviceSynchronize();
         cudaFree(tmp);
         cudaFree(r2);
@@ -1859,7 +1856,7 @@ int nd_graph_create(nd_handle *h, void *m, int method, long long n_steps, double
         return bail(ND_ERR_CUDA, std::string("cudaStreamCreate: ") + cudaGetErrorString(e));
     if ((e = cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
         return bail(ND_ERR_CUDA, std::string("cudaStreamBeginCapture: ") + cudaGetErrorString(e));
-    int rc = run_mode(h, mode, false, m, nullptr, n_steps, g->cap, g->reps);
+    int rc = run_mode(h, mode, m, nullptr, n_steps, g->cap, g->reps);
     if (rc == ND_OK && (stats_sample & ND_GRAPH_STATS)) rc = stats_launches(h, m, n_steps * dt_seconds, g->cap, g->reps);
     if (rc == ND_OK && (stats_sample & ND_GRAPH_SERIES)) rc = series_launches(h, m, g->cap, g->reps);
     if (rc == ND_OK && launch_advance_steps(g->reps, B, n_steps, g->cap) != cudaSuccess) rc = ND_ERR_CUDA;

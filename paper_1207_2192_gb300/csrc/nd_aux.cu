@@ -1,6 +1,6 @@
 // nd_aux.cu -- once-per-geometry spectral kernel build and the small
 // per-replica kernels: analytic vortex profile, vortex-core estimator, <m>,
-// precision conversion and finiteness check.
+// finiteness check.
 #include <math.h>
 
 #include "nd_common.cuh"
@@ -471,23 +471,7 @@ cudaError_t launch_mean_m(int prec, const Replica *reps, const int *work, int nw
     return cudaGetLastError();
 }
 
-// ---------------------------------------------------- conversion, checks
-
-template <typename S, typename D_>
-__global__ void k_convert(const S *src, D_ *dst, size_t n)
-{
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        dst[i] = (D_)src[i];
-}
-
-cudaError_t launch_convert(int to_prec, const void *src, void *dst, size_t n, cudaStream_t st)
-{
-    const int blocks = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-    if (n == 0) return cudaSuccess;
-    if (to_prec == ND_PREC_FP64) k_convert<float, double><<<blocks, 256, 0, st>>>((const float *)src, (double *)dst, n);
-    else k_convert<double, float><<<blocks, 256, 0, st>>>((const double *)src, (float *)dst, n);
-    return cudaGetLastError();
-}
+// ---------------------------------------------------------------- checks
 
 // Sets ND_DEV_NAN in *flag if any component of a cell inside a disk is not
 // finite (cells outside the disks and padding columns are ignored).

@@ -104,6 +104,7 @@ struct Replica {
     const void *Ghat;            // [P/2+1 (kx)][P/2+1 (ky)][4] spectral kernel, incl. exchange and 1/P^2,
                                  // then the same values as [4][P/2+1][P/2+1]
     const double *Ghat64;        // the same in FP64 (null where no kernel reads it)
+    const double *GhatL;         // its thickness derivative (the energy kernels)
     const unsigned char *mask;   // [D][D]
     const int *cells;            // the cells inside the disk, j*D+i in increasing order (ncells of them)
     int ncells, pad_cells;

@@ -124,25 +124,18 @@ __device__ __forceinline__ StageOut<T> stage_update(const StepParams<T> &sp, boo
 //   ms  : stage magnetisation (read; overwritten with the next stage's input)
 //   yn  : state y_n (user buffer), acc : stage accumulator (scratch)
 //   b   : the full dimensionless induction b_i at this cell
-// Returns the cell's contribution to the reduced quantity (energy mode).
 // For Heun, wbuf (when not null) keeps the predictor's normals for the
 // corrector, which then reads them instead of regenerating them.
 // ynl, accl: where y_n and the accumulator are read from (the same arrays, or
 // copies of them staged in shared memory); writes always go to yn and acc.
 template <typename T, int MODE>
-__device__ __forceinline__ double epilogue_cell(const Replica &r, int cell, long long si, long long mi, vec3<T> b,
+__device__ __forceinline__ void epilogue_cell(const Replica &r, int cell, long long si, long long mi, vec3<T> b,
                                                 V3Ptr<T> ms, V3Ptr<T> yn, V3Ptr<T> acc, V3Ptr<T> out, int stage,
                                                 unsigned long long step, V3Ptr<T> wbuf, V3Ptr<T> ynl, V3Ptr<T> accl)
 {
     vec3<T> m = ms.ld(mi);
     if (MODE == M_FIELD) {
         out.st(si, b);
-        return 0.0;
-    } else if (MODE == M_ENERGY) {
-        // E/J = -sum_i m_i . (b'_i / 2 + c h_ext), b' = b - c h_ext  (Eq. Hmm)
-        double bx = (double)b.x - r.chext[0], by = (double)b.y - r.chext[1], bz = (double)b.z - r.chext[2];
-        return -fm((double)m.x, fm(0.5, bx, r.chext[0]),
-                   fm((double)m.y, fm(0.5, by, r.chext[1]), (double)m.z * fm(0.5, bz, r.chext[2])));
     } else if (MODE == M_RK4 || MODE == M_HEUN) {
         const StepParams<T> sp = step_params<T>(r);
         const vec3<T> zero = {T(0), T(0), T(0)};
@@ -161,29 +154,20 @@ __device__ __forceinline__ double epilogue_cell(const Replica &r, int cell, long
         if (o.w_acc) acc.st(si, o.acc);
         if (o.w_yn) yn.st(si, o.nm);
         ms.st(mi, o.nm);
-        return 0.0;
     }
-    return 0.0;
 }
 
 template <typename T, int MODE>
-__device__ __forceinline__ double epilogue_cell(const Replica &r, int cell, long long si, long long mi, vec3<T> b,
+__device__ __forceinline__ void epilogue_cell(const Replica &r, int cell, long long si, long long mi, vec3<T> b,
                                                 V3Ptr<T> ms, V3Ptr<T> yn, V3Ptr<T> acc, V3Ptr<T> out, int stage,
                                                 unsigned long long step, V3Ptr<T> wbuf = V3Ptr<T>{nullptr, 0})
 {
-    return epilogue_cell<T, MODE>(r, cell, si, mi, b, ms, yn, acc, out, stage, step, wbuf, yn, acc);
+    epilogue_cell<T, MODE>(r, cell, si, mi, b, ms, yn, acc, out, stage, step, wbuf, yn, acc);
 }
 
 template <int MODE> struct ModeStages { static constexpr int n = 1; };
 template <> struct ModeStages<M_RK4> { static constexpr int n = 4; };
 template <> struct ModeStages<M_HEUN> { static constexpr int n = 2; };
-
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
 
 // ------------------------------------------------------------ fused path
 
@@ -195,9 +179,8 @@ __host__ __device__ __forceinline__ size_t fused_smem_bytes(int D, int Dpad, int
     size_t spec = sizeof(cplx<T>) * 3 * (size_t)D * SpecGeom<P>::RS;
     size_t scr = sizeof(cplx<T>) * (size_t)(nthreads / Gm::G) * Gm::SCRATCH;
     size_t ms = sizeof(T) * 3 * (size_t)D * Dpad;
-    size_t red = sizeof(double) * 32;
     size_t w = wbuf ? sizeof(T) * 3 * (size_t)D * Dpad : 0;
-    return tw + spec + scr + ms + red + w;
+    return tw + spec + scr + ms + w;
 }
 
 // A piece of one replica's trajectory run by one CTA (time-sliced schedule).
@@ -299,8 +282,7 @@ template <int P, int NT> struct FusedMinBlocks {
 template <int P, typename T, int MODE, int NT>
 __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
     k_fused(const Replica *__restrict__ reps, const int *__restrict__ work, T *__restrict__ ybase,
-            T *__restrict__ accbase, T *__restrict__ outbase, double *__restrict__ red_out,
-            const cplx<T> *__restrict__ twP, long long nsteps, unsigned long long step_base,
+            T *__restrict__ accbase, T *__restrict__ outbase, const cplx<T> *__restrict__ twP, long long nsteps, unsigned long long step_base,
             RelaxIO *__restrict__ rio, double eta_d, double tol_d, double rc2_d, int max_iter,
             const Segment *__restrict__ segs, const int *__restrict__ seg_off, int *__restrict__ flags,
             unsigned *__restrict__ status, int use_wbuf)
@@ -345,8 +327,7 @@ __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
         cplx<T> *spec = tw + R1 * G;
         cplx<T> *scratch = spec + 3 * cs;
         T *msm = reinterpret_cast<T *>(scratch + NGRP * Gm::SCRATCH);
-        double *red = reinterpret_cast<double *>(msm + 3 * ms_s);
-        T *wsm = use_wbuf ? reinterpret_cast<T *>(red + 32) : nullptr;
+        T *wsm = use_wbuf ? msm + 3 * ms_s : nullptr;
         cplx<T> *scr = scratch + gid.group * Gm::SCRATCH;
 
         V3Ptr<T> yn{ybase + r.state_off, ms_s};
@@ -366,7 +347,6 @@ __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
         // else a complex row pair each
         constexpr bool HR = HalfRows<P>::on;
         const int nrow = row_pass_tasks<P>(D);
-        double esum = 0.0;
         T relX = 0, relY = 0;
         if (MODE == M_RELAX) {
             relX = (T)rio[ridx].X[0];
@@ -374,7 +354,7 @@ __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
             if (tid == 0) { lam_s[0] = (T)rio[ridx].lam[0]; lam_s[1] = (T)rio[ridx].lam[1]; conv_s = 0; }
             __syncthreads();
         }
-        const long long nst = (MODE == M_FIELD || MODE == M_ENERGY) ? 1 : (MODE == M_RELAX ? (long long)max_iter : nseg);
+        const long long nst = MODE == M_FIELD ? 1 : (MODE == M_RELAX ? (long long)max_iter : nseg);
         long long n = 0;
         T res_last = T(0);
         for (n = 0; n < nst; ++n) {
@@ -496,10 +476,7 @@ __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
                     const long long si = (long long)y * Dpad + x;
                     const long long hi = (long long)y * (2 * RS) + x;
                     vec3<T> b = {hr[hi] + cx.x, hr[2 * cs + hi] + cx.y, hr[4 * cs + hi] + cx.z};
-                    if (MODE == M_ENERGY)
-                        esum += epilogue_cell<T, MODE>(r, cell, si, si, b, ms, yn, acc, out, stage, step);
-                    else
-                        epilogue_cell<T, MODE>(r, cell, si, si, b, ms, yn, acc, out, stage, step, wb, ynl, accl);
+                    epilogue_cell<T, MODE>(r, cell, si, si, b, ms, yn, acc, out, stage, step, wb, ynl, accl);
                 }
                 __syncthreads();
             }
@@ -519,16 +496,6 @@ __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
                 rio[ridx].resid = (double)res_last;
                 rio[ridx].iters = (int)n;
                 rio[ridx].status = conv_s ? 0 : 1;
-            }
-        }
-        if (MODE == M_ENERGY) {
-            esum = warp_sum(esum);
-            if ((tid & 31) == 0) red[warp] = esum;
-            __syncthreads();
-            if (tid == 0) {
-                double s = 0.0;
-                for (int w = 0; w < NW; ++w) s += red[w];
-                red_out[ridx] = s;
             }
         }
         __syncthreads();   // every write of this segment is done before the flag and the next segment
@@ -787,8 +754,7 @@ template <int P, typename T, int MODE>
 __global__ void __launch_bounds__(256)
     k_g_epi(const Replica *__restrict__ reps, const int *__restrict__ work, T *__restrict__ msbase,
             T *__restrict__ ybase, T *__restrict__ accbase, T *__restrict__ outbase,
-            const cplx<T> *__restrict__ specbase, double *__restrict__ red_out, int stage,
-            unsigned long long step)
+            const cplx<T> *__restrict__ specbase, int stage, unsigned long long step)
 {
     constexpr int RS = SpecGeom<P>::RS;
     const int ridx = work[blockIdx.y];
@@ -796,7 +762,6 @@ __global__ void __launch_bounds__(256)
     const int D = r.D, DD = D * D;
     const long long ms_s = (long long)D * r.Dpad, cs = (long long)D * RS;
     const int cell = blockIdx.x * 256 + threadIdx.x;
-    double e = 0.0;
     if (cell < DD && r.mask[cell]) {
         const int y = cell / D, x = cell - y * D;
         const long long si = (long long)y * r.Dpad + x;
@@ -808,18 +773,7 @@ __global__ void __launch_bounds__(256)
         vec3<T> b = {hr[hi] + cx.x, hr[2 * cs + hi] + cx.y, hr[4 * cs + hi] + cx.z};
         V3Ptr<T> ms{msbase + r.state_off, ms_s}, yn{ybase + r.state_off, ms_s};
         V3Ptr<T> acc{accbase ? accbase + r.state_off : nullptr, ms_s}, out{outbase ? outbase + r.state_off : nullptr, ms_s};
-        e = epilogue_cell<T, MODE>(r, cell, si, si, b, ms, yn, acc, out, stage, step + r.step0);
-    }
-    if (MODE == M_ENERGY) {
-        __shared__ double red[8];
-        e = warp_sum(e);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double s = 0.0;
-            for (int w = 0; w < 8; ++w) s += red[w];
-            atomicAdd(red_out + ridx, s);
-        }
+        epilogue_cell<T, MODE>(r, cell, si, si, b, ms, yn, acc, out, stage, step + r.step0);
     }
 }
 
@@ -1177,7 +1131,7 @@ static cudaError_t launch_fused_t(const LaunchArgs &a)
     if (e != cudaSuccess) return e;
     const Segment *segs = reinterpret_cast<const Segment *>(a.segs);
     if (!segs) {
-        kern<<<a.nwork, NT, a.smem, a.stream>>>(a.reps, a.work, (T *)a.y, (T *)a.acc, (T *)a.out, a.red,
+        kern<<<a.nwork, NT, a.smem, a.stream>>>(a.reps, a.work, (T *)a.y, (T *)a.acc, (T *)a.out,
                                                 (const cplx<T> *)a.tw, a.nsteps, a.step_base, a.rio, a.eta, a.tol,
                                                 a.rc2, a.max_iter, nullptr, nullptr, nullptr, a.status, a.use_wbuf);
         return cudaGetLastError();
@@ -1187,7 +1141,6 @@ static cudaError_t launch_fused_t(const LaunchArgs &a)
     const Replica *reps = a.reps;
     const int *work = a.work;
     T *y = (T *)a.y, *acc = (T *)a.acc, *out = (T *)a.out;
-    double *red = a.red;
     const cplx<T> *tw = (const cplx<T> *)a.tw;
     long long nsteps = a.nsteps;
     unsigned long long step_base = a.step_base;
@@ -1197,7 +1150,7 @@ static cudaError_t launch_fused_t(const LaunchArgs &a)
     const int *seg_off = a.seg_off;
     int *flags = a.flags;
     unsigned *status = a.status;
-    void *args[] = {(void *)&reps, (void *)&work, (void *)&y, (void *)&acc, (void *)&out, (void *)&red, (void *)&tw,
+    void *args[] = {(void *)&reps, (void *)&work, (void *)&y, (void *)&acc, (void *)&out, (void *)&tw,
                     (void *)&nsteps, (void *)&step_base, (void *)&rio, (void *)&eta, (void *)&tol, (void *)&rc2,
                     (void *)&max_iter, (void *)&segs, (void *)&seg_off, (void *)&flags, (void *)&status,
                     (void *)&use_wbuf};
@@ -1259,7 +1212,6 @@ static cudaError_t launch_fused_p(const LaunchArgs &a)
     constexpr int NT0 = FusedNT<P>::v;
     switch (a.mode) {
     case M_FIELD: return launch_fused_t<P, T, M_FIELD, NT0>(a);
-    case M_ENERGY: return launch_fused_t<P, T, M_ENERGY, NT0>(a);
     case M_RK4: return launch_stepper<P, T, M_RK4>(a);
     case M_HEUN: return launch_stepper<P, T, M_HEUN>(a);
     case M_RELAX: return launch_fused_t<P, T, M_RELAX, NT0>(a);
@@ -1271,7 +1223,7 @@ template <int P, typename T, int MODE>
 static void launch_g_epi(const LaunchArgs &a, dim3 ge, int stage, unsigned long long step)
 {
     k_g_epi<P, T, MODE><<<ge, 256, 0, a.stream>>>(a.reps, a.work, (T *)a.ms, (T *)a.y, (T *)a.acc, (T *)a.out,
-                                                   (const cplx<T> *)a.spec, a.red, stage, step);
+                                                   (const cplx<T> *)a.spec, stage, step);
 }
 
 // Launch with programmatic stream serialisation: the kernel may be scheduled
@@ -1357,7 +1309,6 @@ static cudaError_t glob_eval(const LaunchArgs &a, int maxD, int stage, int mode,
     dim3 ge((maxD * maxD + 255) / 256, a.nwork);
     switch (mode) {
     case M_FIELD: launch_g_epi<P, T, M_FIELD>(a, ge, stage, step); break;
-    case M_ENERGY: launch_g_epi<P, T, M_ENERGY>(a, ge, stage, step); break;
     case M_RK4: launch_g_epi_step<P, T, M_RK4>(a, maxD, stage, step); break;
     case M_HEUN: launch_g_epi_step<P, T, M_HEUN>(a, maxD, stage, step); break;
     default: return cudaErrorInvalidValue;
@@ -1416,7 +1367,7 @@ static cudaError_t launch_global_p(const LaunchArgs &a, int maxD)
         return cudaGetLastError();
     }
     const int nst = (a.mode == M_RK4) ? 4 : (a.mode == M_HEUN ? 2 : 1);
-    const long long nsteps = (a.mode == M_FIELD || a.mode == M_ENERGY) ? 1 : a.nsteps;
+    const long long nsteps = a.mode == M_FIELD ? 1 : a.nsteps;
     for (long long n = 0; n < nsteps; ++n)
         for (int s = 0; s < nst; ++s) {
             e = glob_eval<P, T>(a, maxD, s, a.mode, a.step_base + n);

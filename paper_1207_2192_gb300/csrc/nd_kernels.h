@@ -8,7 +8,7 @@
 namespace nd {
 
 enum { ND_PREC_FP32 = 0, ND_PREC_FP64 = 1 };
-enum { M_FIELD = 0, M_RK4 = 1, M_HEUN = 2, M_ENERGY = 3, M_RELAX = 4 };
+enum { M_FIELD = 0, M_RK4 = 1, M_HEUN = 2, M_RELAX = 4 };
 
 struct Replica;
 struct RelaxIO;
@@ -24,7 +24,6 @@ struct LaunchArgs {
     void *out = nullptr;             // field output (field mode)
     void *ms = nullptr;              // global-path stage state (same layout as y)
     void *spec = nullptr;            // global-path spectrum scratch
-    double *red = nullptr;           // per-replica reduction output (energy), indexed by replica
     const void *tw = nullptr;        // length-P twiddle table exp(-2 pi i k/P) of the precision
     const void *tw64 = nullptr;      // the same table in FP64 (cluster relaxation)
     long long nsteps = 1;
@@ -73,6 +72,21 @@ size_t cluster_smem(int P, int prec, int D, int Dpad, bool wbuf, int nc);   // (
 int cluster_max_active(int P, int prec, int D, int Dpad, bool wbuf, int nc);  // 0: does not fit
 cudaError_t launch_cluster(int P, int prec, const LaunchArgs &a, int maxD, int maxDpad, int nc);
 cudaError_t launch_global(int P, int prec, const LaunchArgs &a, int maxD);
+// Energies E/J (and, with_dl, d(E/J)/dl) of a class's replicas in FP64 from the
+// state m of the given precision (nd_energy.cu): out [replicas][2].
+struct EnergyArgs {
+    const Replica *reps = nullptr;
+    const int *work = nullptr;
+    int nwork = 0, maxD = 0, with_dl = 0;
+    const void *m = nullptr;
+    void *spec = nullptr;            // FP64 spectrum scratch (Replica::spec_off)
+    const void *tw = nullptr;        // length-P FP64 twiddle table
+    double *part = nullptr;          // [replicas][column blocks <= P/2][2] of the class's P
+    unsigned *done = nullptr;        // [replicas], zero before the first call
+    double *out = nullptr;
+    cudaStream_t stream = 0;
+};
+cudaError_t launch_energy(int P, int prec, const EnergyArgs &a);
 size_t spec_words(int P, int D);   // complex words of one replica's [3][D][RS] spectrum
 // One constrained-relaxation sweep over a size class with the field taken
 // from an energy gradient: b = gscale[r] * grad (a.y: the state, a.rio/a.part:
@@ -108,7 +122,6 @@ cudaError_t launch_stats_update(const int *work, int nwork, const double *core, 
 cudaError_t launch_advance_steps(Replica *reps, int n, long long steps, cudaStream_t s);
 cudaError_t launch_mean_m(int prec, const Replica *reps, const int *work, int nwork, const void *y,
                           double *out /*[nrep][3]*/, cudaStream_t st);
-cudaError_t launch_convert(int to_prec, const void *src, void *dst, size_t n, cudaStream_t st);
 
 // Time series of <m> and their power spectra (nd_spectra.cu).
 cudaError_t launch_series_append(int prec, const Replica *reps, const int *work, int nwork, const void *y,

@@ -473,10 +473,11 @@ template <int P> __host__ __device__ __forceinline__ int row_pass_tasks(int D)
     return HalfRows<P>::on ? 3 * D : row_tasks(D);
 }
 
-// Forward: the real row x (x[i], i < D; zero beyond) to its half spectrum:
-// X[k] for k = t + G o (k < M) left in v[o], X[M] (real) in xm on lane t = 0.
-template <int P, typename T>
-__device__ __forceinline__ void row_fwd_half_spectrum(bool active, const T *x, int D, cplx<T> *v, T &xm, int t,
+// Forward: the real row x (x[i], i < D; zero beyond; a pointer or anything that
+// is indexed like one) to its half spectrum: X[k] for k = t + G o (k < M) left
+// in v[o], X[M] (real) in xm on lane t = 0.
+template <int P, typename T, typename Row>
+__device__ __forceinline__ void row_fwd_half_spectrum(bool active, Row x, int D, cplx<T> *v, T &xm, int t,
                                                       cplx<T> *scr, const cplx<T> *twP, unsigned gmask)
 {
     constexpr int M = P / 2, G = FFTGeom<M>::G, R1 = FFTGeom<M>::R1;
@@ -510,8 +511,8 @@ __device__ __forceinline__ void row_fwd_half_spectrum(bool active, const T *x, i
 }
 
 // Forward, stored: X[0..M] of the real row to dst.
-template <int P, typename T>
-__device__ __forceinline__ void row_fwd_half(bool active, const T *x, int D, cplx<T> *dst, int t, cplx<T> *scr,
+template <int P, typename T, typename Row>
+__device__ __forceinline__ void row_fwd_half(bool active, Row x, int D, cplx<T> *dst, int t, cplx<T> *scr,
                                              const cplx<T> *twP, unsigned gmask)
 {
     constexpr int M = P / 2, G = FFTGeom<M>::G, R1 = FFTGeom<M>::R1;
