@@ -94,10 +94,12 @@ template <int P> struct FFTGeom {
     static_assert(R1 % G == 0, "R1 must be a multiple of G");
     static constexpr int R2 = R1 / G;  // G-point DFTs per thread in pass 2
     // per-group scratch: R1 rows of G+1 (padding breaks the stride-G conflicts),
-    // rounded so consecutive groups start 8 complex words apart modulo 16
+    // rounded so consecutive groups start 8 complex words apart modulo 16 (two
+    // groups of a half-warp in different banks), or, where a group fills the
+    // half-warp, 2 apart (the column tiles write eight groups' areas side by side)
     static constexpr int SROW = G + 1;
     static constexpr int SRAW = R1 * SROW;
-    static constexpr int SCRATCH = SRAW + ((8 - SRAW % 16) + 16) % 16;
+    static constexpr int SCRATCH = SRAW + (((G >= 16 ? 2 : 8) - SRAW % 16) + 16) % 16;
     static constexpr int GROUPS_PER_WARP = 32 / G;   // whole groups per warp
     static constexpr bool POW2 = (G & (G - 1)) == 0;   // groups tile the warp exactly
 };

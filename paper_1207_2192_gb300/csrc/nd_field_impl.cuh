@@ -578,27 +578,28 @@ __global__ void __launch_bounds__(NT)
                    scratch + gid.group * Gm::SCRATCH, tw, gid.gmask);
 }
 
-// Tiled column pass for the large grids.  A CTA takes a block of four
-// adjacent columns kx0..kx0+3 and one FFT group per (column, component): the
-// XY kernel the x and y components (eight groups; group 4c + j holds component
-// c of column kx0 + j, its partner for the in-plane tensor is group ^ 4), the
-// Z kernel the z component (four groups).  The block's [D][4] tiles move
-// between the spectrum and the groups' scratch areas as row-contiguous runs
-// of four complex words (one 32-byte sector per row: rows start on sectors,
-// SpecGeom::RS), so every sector the pass reads or writes is used whole.  The
-// packed real columns kx = 0, P/2 are group j = 0 of block 0.  Persistent
-// grid over (replica, column block) tasks.
-template <int P, typename T, bool XY> struct ColTile {
+// Tiled column pass for the large grids.  A CTA of eight FFT groups takes one
+// of two kinds of task: four adjacent columns of the x and y components (group
+// 4c + j holds component c of column kx0 + j, its partner for the in-plane
+// tensor is group ^ 4), or eight adjacent columns of z.  Both cost about the
+// same, and one launch runs the xy tasks of all replicas and then the z tasks:
+// as two launches (xy; z with four groups) each pass ended in a round that
+// filled part of the SMs (24 replicas of D = 121 at P = 256: 18.0 + 10.6 us, 768
+// tasks each on 608 resident CTAs; 8 of D = 500 at P = 1024: 55.8 + 27.3 us).
+// The task's tiles [D][4] x 2 or [D][8] move between the spectrum and the
+// groups' scratch areas as row-contiguous runs of four or eight complex words
+// (whole 32-byte sectors: rows start on sectors, SpecGeom::RS).  The packed
+// real columns kx = 0, P/2 are column 0 of the first block.  Persistent grid.
+template <int P, typename T> struct ColTile {
     static constexpr int G = FFTGeom<P>::G;
-    static constexpr int NCOMP = XY ? 2 : 1;
-    static constexpr int NG = 4 * NCOMP;
-    // whole warps: with ten-lane groups (P = 200, three to a warp) the XY
-    // block is three warps with one group slot and each warp's last two
-    // lanes idle, the Z block two warps with two idle slots
+    static constexpr int NG = 8;
+    // whole warps: with ten-lane groups (P = 200, three to a warp) three warps
+    // with one group slot and each warp's last two lanes idle
     static constexpr bool POW2 = FFTGeom<P>::POW2;
     static constexpr int GPW = FFTGeom<P>::GROUPS_PER_WARP;
     static constexpr int NT = POW2 ? NG * G : (NG + GPW - 1) / GPW * 32;
-    static constexpr int NCB = P / 2 / 4;
+    static constexpr int NXY = P / 2 / 4;                // xy tasks of a replica
+    static constexpr int NZ = (P / 2 + 7) / 8;           // its z tasks
     // resident CTAs per SM the kernel is compiled for: 16 warps at 128
     // registers (FP64 columns take twice the registers)
     static constexpr int MINB = sizeof(T) == 8 ? 1 : 512 / NT;
@@ -612,13 +613,13 @@ template <int P, typename T, bool XY> struct ColTile {
     static constexpr bool SHARED_PACKED = FFTGeom<P>::R1 >= 32;
 };
 
-template <int P, typename T, bool XY>
-__global__ void __launch_bounds__(ColTile<P, T, XY>::NT, ColTile<P, T, XY>::MINB)
+template <int P, typename T>
+__global__ void __launch_bounds__(ColTile<P, T>::NT, ColTile<P, T>::MINB)
     k_g_cols_tile(const Replica *__restrict__ reps, const int *__restrict__ work, int nwork,
                   cplx<T> *__restrict__ specbase, const cplx<T> *__restrict__ twP)
 {
     using Gm = FFTGeom<P>;
-    using CT = ColTile<P, T, XY>;
+    using CT = ColTile<P, T>;
     constexpr int G = Gm::G, R1 = Gm::R1, KH = SpecGeom<P>::KH, RS = SpecGeom<P>::RS, NT = CT::NT, SCR = Gm::SCRATCH;
     constexpr bool SP = CT::SHARED_PACKED;
     static_assert(RS % 4 == 0, "rows start on 32-byte sectors");
@@ -629,43 +630,45 @@ __global__ void __launch_bounds__(ColTile<P, T, XY>::NT, ColTile<P, T, XY>::MINB
     load_twiddles<P>(tw, twP, tid, NT);   // constant: before the wait
     wait_prior_grid();
     GroupId<P> gid(tid);
-    const int g = gid.group, j = g & 3, c = XY ? (g >> 2) : 2, t = gid.t;
+    const int g = gid.group, t = gid.t;
     // a group of the block (idle slots and lanes take part in the tile moves
     // and the barriers only)
     const bool gv = CT::POW2 || (gid.valid && g < CT::NG);
     cplx<T> *scr = scratch + g * SCR;
-    const cplx<T> *other = scratch + (g ^ 4) * SCR;   // XY only
-    for (int task = blockIdx.x; task < nwork * CT::NCB; task += gridDim.x) {
-        const int wi = task / CT::NCB, cb = task - wi * CT::NCB, kx0 = 4 * cb;
+    const cplx<T> *other = scratch + (g ^ 4) * SCR;   // xy tasks only
+    const int jj = tid & 7;                            // the tile moves: this thread's column of the task
+    const int nxy = nwork * CT::NXY, ntask = nxy + nwork * CT::NZ;
+    for (int task = blockIdx.x; task < ntask; task += gridDim.x) {
+        const bool xy = task < nxy;
+        const int ti = xy ? task : task - nxy, per = xy ? CT::NXY : CT::NZ;
+        const int wi = ti / per, cb = ti - wi * per, kx0 = (xy ? 4 : 8) * cb;
+        const int j = xy ? g & 3 : g, c = xy ? g >> 2 : 2;
         const Replica &r = reps[work[wi]];
         const int D = r.D;
         const long long cs = (long long)D * RS;
         cplx<T> *spec = specbase + r.spec_off;
         const T *Ghat = reinterpret_cast<const T *>(r.Ghat);
         const bool packed = (cb == 0 && j == 0);
-        const int kx = packed ? 1 : kx0 + j;   // (the packed group reads no kx column of the table)
+        const bool gon = gv && (P % 16 == 0 || kx0 + j < P / 2);   // (the last z task of P = 200 has four columns)
+        const int kx = packed || !gon ? 1 : kx0 + j;   // (the packed group reads no kx column of the table)
+        // this thread's column in the tile moves: (column 0 of block 0: the
+        // packed pair c_0 + i c_{P/2}, when it moves through the tile)
+        const int mj = xy ? jj & 3 : jj, mc = xy ? jj >> 2 : 2;
+        const bool ppair = cb == 0 && mj == 0, mon = P % 16 == 0 || kx0 + mj < P / 2;
+        cplx<T> *const tile = scratch + jj * SCR;
+        cplx<T> *const gcol = spec + mc * cs + kx0 + mj;
         __syncthreads();   // twiddles filled / the previous task's tiles stored
-        // tile load: thread -> column jj = tid & 3 of the block, rows tid/4 + k NT/4
-        // (column 0 of block 0: the packed pair c_0 + i c_{P/2}, when it moves
-        // through the tile)
-        const int cbase = XY ? 0 : 2, jj = tid & 3;
-        const bool ppair = cb == 0 && jj == 0;
-        if (SP || !ppair) {
-#pragma unroll
-            for (int ci = 0; ci < CT::NCOMP; ++ci) {
-                const cplx<T> *src = spec + (cbase + ci) * cs + kx0 + jj;
-                cplx<T> *dst = scratch + (4 * ci + jj) * SCR;
-                if (SP && ppair) {
-                    for (int y = tid >> 2; y < D; y += NT / 4)
-                        dst[y] = {src[(long long)y * RS].x, src[(long long)y * RS + P / 2].x};
-                } else {
-                    for (int y = tid >> 2; y < D; y += NT / 4) dst[y] = src[(long long)y * RS];
-                }
+        if (mon && (SP || !ppair)) {
+            if (SP && ppair) {
+                for (int y = tid >> 3; y < D; y += NT / 8)
+                    tile[y] = {gcol[(long long)y * RS].x, gcol[(long long)y * RS + P / 2].x};
+            } else {
+                for (int y = tid >> 3; y < D; y += NT / 8) tile[y] = gcol[(long long)y * RS];
             }
         }
         __syncthreads();
         cplx<T> v[R1];
-        if (!gv) {
+        if (!gon) {
         } else if (!SP && packed) {
             packed_col_fwd<P, T>(v, c, true, D, spec + c * cs, Ghat, t, gid.lane, scr, tw, gid.gmask);
         } else {
@@ -678,13 +681,13 @@ __global__ void __launch_bounds__(ColTile<P, T, XY>::NT, ColTile<P, T, XY>::MINB
             }
             __syncwarp(gid.gmask);
             fft_group<P, -1, FFT_HALF_IN>(v, t, scr, tw, gid.gmask);
-            if (XY) {
+            if (xy) {
 #pragma unroll
                 for (int o = 0; o < R1; ++o) scr[o * G + t] = v[o];
             }
         }
-        if (XY) __syncthreads();
-        if (!gv) {
+        if (xy) __syncthreads();
+        if (!gon) {
         } else if (packed) {
             // (the packed pair's partner is packed too and reads no spectrum of it)
             if (SP) packed_col_scale<P, T>(v, c, Ghat, t, scr, gid.gmask);
@@ -693,7 +696,7 @@ __global__ void __launch_bounds__(ColTile<P, T, XY>::NT, ColTile<P, T, XY>::MINB
             // entries it uses (4 or 8 bytes per point instead of 16)
             constexpr int KK = KH * KH;
             const T *Gs = Ghat + 4 * KK + kx * KH;
-            if (XY) {
+            if (xy) {
                 const T *gd = Gs + c * KK, *go = Gs + 2 * KK;   // diagonal entry (xx or yy), xy
 #pragma unroll
                 for (int o = 0; o < R1; ++o) {
@@ -715,8 +718,8 @@ __global__ void __launch_bounds__(ColTile<P, T, XY>::NT, ColTile<P, T, XY>::MINB
                 }
             }
         }
-        if (XY) __syncthreads();   // the partner's spectrum is read before the scratch is reused
-        if (gv) {
+        if (xy) __syncthreads();   // the partner's spectrum is read before the scratch is reused
+        if (gon) {
             fft_group<P, +1, FFT_HALF_OUT>(v, t, scr, tw, gid.gmask);
             __syncwarp(gid.gmask);
             if (!SP && packed) {
@@ -730,20 +733,15 @@ __global__ void __launch_bounds__(ColTile<P, T, XY>::NT, ColTile<P, T, XY>::MINB
             }
         }
         __syncthreads();
-        if (SP || !ppair) {
-#pragma unroll
-            for (int ci = 0; ci < CT::NCOMP; ++ci) {
-                cplx<T> *dst = spec + (cbase + ci) * cs + kx0 + jj;
-                const cplx<T> *src = scratch + (4 * ci + jj) * SCR;
-                if (SP && ppair) {
-                    for (int y = tid >> 2; y < D; y += NT / 4) {
-                        const cplx<T> u = src[y];
-                        dst[(long long)y * RS] = {u.x, T(0)};
-                        dst[(long long)y * RS + P / 2] = {u.y, T(0)};
-                    }
-                } else {
-                    for (int y = tid >> 2; y < D; y += NT / 4) dst[(long long)y * RS] = src[y];
+        if (mon && (SP || !ppair)) {
+            if (SP && ppair) {
+                for (int y = tid >> 3; y < D; y += NT / 8) {
+                    const cplx<T> u = tile[y];
+                    gcol[(long long)y * RS] = {u.x, T(0)};
+                    gcol[(long long)y * RS + P / 2] = {u.y, T(0)};
                 }
+            } else {
+                for (int y = tid >> 3; y < D; y += NT / 8) gcol[(long long)y * RS] = tile[y];
             }
         }
     }
@@ -948,20 +946,26 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-static __global__ void k_g_relax_newton(const int *__restrict__ work, int nwork, RelaxIO *__restrict__ rio,
+// One warp per replica (one thread's chain of 64 FP64 additions per sum took 27
+// us, half a sweep of two FP64 replicas' columns).
+static __global__ void __launch_bounds__(128) k_g_relax_newton(const int *__restrict__ work, int nwork, RelaxIO *__restrict__ rio,
                                  const double *__restrict__ part, double tol, int iter)
 {
-    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (w >= nwork) return;
     const int ridx = work[w];
     RelaxIO &R = rio[ridx];
     if (R.status == 0) return;
     double s[6] = {0, 0, 0, 0, 0, 0};
-    for (int b = 0; b < kRelaxBlocks; ++b) {
+    for (int b = lane; b < kRelaxBlocks; b += 32) {
         const double *o = part + ((size_t)ridx * kRelaxBlocks + b) * 6;
         for (int k = 0; k < 5; ++k) s[k] += o[k];
         s[5] = fmax(s[5], o[5]);
     }
+    for (int k = 0; k < 5; ++k) s[k] = warp_sum_t(s[k]);
+    s[5] = warp_max_t(s[5]);
+    __syncwarp();
+    if (lane != 0) return;
     R.resid = s[5];
     if (s[5] < tol) {
         R.status = 0;   // converged: iters keeps the number of sweeps applied
@@ -1075,7 +1079,7 @@ static cudaError_t launch_relax_grad_t(const LaunchArgs &a, int maxD, const void
     const dim3 gp(kRelaxBlocks, a.nwork), gu((maxD * maxD + 255) / 256, a.nwork);
     k_relax_grad_reduce<T><<<gp, 256, 0, a.stream>>>(a.reps, a.work, (const T *)a.y, (const T *)grad, gscale, a.rio,
                                                      a.rc2, a.eta, a.part);
-    k_g_relax_newton<<<(a.nwork + 127) / 128, 128, 0, a.stream>>>(a.work, a.nwork, a.rio, a.part, a.tol, 0);
+    k_g_relax_newton<<<(a.nwork + 3) / 4, 128, 0, a.stream>>>(a.work, a.nwork, a.rio, a.part, a.tol, 0);
     k_relax_grad_update<T><<<gu, 256, 0, a.stream>>>(a.reps, a.work, (T *)a.y, (const T *)grad, gscale, a.rio, a.rc2,
                                                      a.eta);
     return cudaGetLastError();
@@ -1277,15 +1281,11 @@ static void glob_cols(const LaunchArgs &a, int maxD)
 {
     constexpr int NT = GlobNT<P>::v, NGRP = groups_per_block<P, NT>();
     if constexpr (GlobTiled<P>::v) {
-        using CX = ColTile<P, T, true>;
-        using CZ = ColTile<P, T, false>;
-        const int ntask = a.nwork * CX::NCB;
-        const int gx = ntask < a.n_sm * CX::MINB ? ntask : a.n_sm * CX::MINB;
-        const int gz = ntask < a.n_sm * CZ::MINB ? ntask : a.n_sm * CZ::MINB;
-        launch_pdl(k_g_cols_tile<P, T, true>, dim3(gx), dim3(CX::NT), glob_smem_bytes<P, T, CX::NT>(), a.stream,
-                   a.reps, a.work, a.nwork, (cplx<T> *)a.spec, (const cplx<T> *)a.tw);
-        launch_pdl(k_g_cols_tile<P, T, false>, dim3(gz), dim3(CZ::NT), glob_smem_bytes<P, T, CZ::NT>(), a.stream,
-                   a.reps, a.work, a.nwork, (cplx<T> *)a.spec, (const cplx<T> *)a.tw);
+        using CT = ColTile<P, T>;
+        const int ntask = a.nwork * (CT::NXY + CT::NZ);
+        const int grid = ntask < a.n_sm * CT::MINB ? ntask : a.n_sm * CT::MINB;
+        launch_pdl(k_g_cols_tile<P, T>, dim3(grid), dim3(CT::NT), glob_smem_bytes<P, T, CT::NT>(), a.stream, a.reps,
+                   a.work, a.nwork, (cplx<T> *)a.spec, (const cplx<T> *)a.tw);
     } else {
         dim3 gc((P / 2 + NGRP - 1) / NGRP, a.nwork);
         launch_pdl(k_g_cols<P, T, NT>, gc, dim3(NT), glob_smem_bytes<P, T, NT>(), a.stream, a.reps, a.work,
@@ -1327,11 +1327,8 @@ static cudaError_t launch_global_p(const LaunchArgs &a, int maxD)
             e0 = cudaFuncSetAttribute(k_g_cols<P, T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     } else {
         if (e0 == cudaSuccess)
-            e0 = cudaFuncSetAttribute(k_g_cols_tile<P, T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)glob_smem_bytes<P, T, ColTile<P, T, true>::NT>());
-        if (e0 == cudaSuccess)
-            e0 = cudaFuncSetAttribute(k_g_cols_tile<P, T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)glob_smem_bytes<P, T, ColTile<P, T, false>::NT>());
+            e0 = cudaFuncSetAttribute(k_g_cols_tile<P, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)glob_smem_bytes<P, T, ColTile<P, T>::NT>());
     }
     if (e0 != cudaSuccess) return e0;
 
@@ -1347,7 +1344,7 @@ static cudaError_t launch_global_p(const LaunchArgs &a, int maxD)
             glob_field_passes<P, T>(a, maxD);
             k_g_relax_reduce<P, T><<<gp, 256, 0, a.stream>>>(a.reps, a.work, (const T *)a.ms, (const cplx<T> *)a.spec,
                                                              a.rio, a.rc2, a.eta, a.part);
-            k_g_relax_newton<<<(a.nwork + 127) / 128, 128, 0, a.stream>>>(a.work, a.nwork, a.rio, a.part, a.tol, it);
+            k_g_relax_newton<<<(a.nwork + 3) / 4, 128, 0, a.stream>>>(a.work, a.nwork, a.rio, a.part, a.tol, it);
             k_g_relax_update<P, T><<<gu, 256, 0, a.stream>>>(a.reps, a.work, (T *)a.ms, (const cplx<T> *)a.spec, a.rio,
                                                              a.rc2, a.eta);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
