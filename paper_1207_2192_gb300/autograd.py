@@ -36,15 +36,6 @@ import torch
 from ._binding import nd_effective_field, nd_energy, nd_relax_sweep_grad
 
 
-def _replica_scale(h, values, device, dtype):
-    """Per-element vector that holds values[r] on replica r's block."""
-    s = torch.empty(h.state_elems, dtype=dtype, device=device)
-    for r, L in enumerate(h.layout):
-        n = 3 * L["D"] * L["Dpad"]
-        s[L["offset"]:L["offset"] + n] = float(values[r])
-    return s
-
-
 class EnergyFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, m, L, h):
@@ -61,13 +52,15 @@ class EnergyFn(torch.autograd.Function):
     def backward(ctx, gE):
         (m,) = ctx.saved_tensors
         h = ctx.h
-        g = gE.detach().to("cpu", torch.float64).numpy()
         gm = gL = None
         if ctx.needs_input_grad[0]:
-            b = torch.zeros_like(m)
+            b = torch.empty_like(m)
             nd_effective_field(h.h, m, b)
-            gm = b * _replica_scale(h, -ctx.J * g, m.device, m.dtype)
+            # the replicas of one disk are equal blocks: one row of the product each
+            scale = (-ctx.J * gE.detach().to(m.device, torch.float64)).to(m.dtype)
+            gm = (b.view(h.B, -1) * scale[:, None]).view_as(m)
         if ctx.needs_input_grad[1]:
+            g = gE.detach().to("cpu", torch.float64).numpy()
             gL = torch.as_tensor(float(np.dot(g, ctx.dEdL)), dtype=torch.float64)
         return gm, gL, None
 

@@ -149,6 +149,10 @@ struct nd_handle {
     cudaEvent_t slot_ev[kSlots] = {};
     int slot = 0;
     Replica *reps_d = nullptr;
+    // the parameter blocks without a time step, for the calls that need no
+    // other (field, energy, relaxation, observables): uploaded once, and again
+    // when a mask changes
+    Replica *base_d = nullptr;            // (behind reps_d)
     std::map<int, void *> tw64, tw32;     // P -> length-P twiddle tables
     void *acc = nullptr;                  // handle-precision scratch (state layout)
     void *ms = nullptr;                   // handle-precision stage state (global path)
@@ -175,6 +179,7 @@ struct nd_handle {
     double r_max = 0, v_max = 0;
     double *core_d = nullptr;             // [B * 4] estimator output of the last sample
     double *core_part = nullptr;          // [B][kCoreMaxBlocks][2] plaquette-scan candidates
+    unsigned *core_done = nullptr;        // [B] counters of finished scans (behind status_d)
     double *a_rep = nullptr;              // [B] cell edge per replica
     size_t max_smem = 0;
     int n_sm = 0;
@@ -187,6 +192,14 @@ struct nd_handle {
     unsigned *status_d = nullptr;         // device status word (ND_DEV_* bits)
     unsigned long long rk4_step = 0;      // step index of the next nd_step_rk4 step (field schedules)
 };
+
+static void fill_reps(nd_handle *h, double dt_seconds, const double *Tk, const unsigned long long *seed,
+                      unsigned long long step0);
+static cudaError_t upload_base(nd_handle *h)
+{
+    fill_reps(h, 0.0, nullptr, nullptr, 0);
+    return cudaMemcpy(h->base_d, h->reps_h, sizeof(Replica) * h->rep_disk.size(), cudaMemcpyHostToDevice);
+}
 
 static int setup_class_paths(nd_handle *h)
 {
@@ -215,8 +228,8 @@ static void upload_reps(nd_handle *h, cudaStream_t st)
     cudaEventRecord(h->slot_ev[h->slot], st);
 }
 
-static void fill_reps(nd_handle *h, bool fp64_kernel, double dt_seconds, const double *Tk,
-                      const unsigned long long *seed, unsigned long long step0)
+static void fill_reps(nd_handle *h, double dt_seconds, const double *Tk, const unsigned long long *seed,
+                      unsigned long long step0)
 {
     const int B = (int)h->rep_disk.size();
     next_slot(h);
@@ -228,7 +241,7 @@ static void fill_reps(nd_handle *h, bool fp64_kernel, double dt_seconds, const d
         R.disk = h->rep_disk[r];
         R.state_off = h->rep_off[r];
         R.spec_off = h->rep_spec_off[r];
-        R.Ghat = fp64_kernel ? (const void *)d.ghat64 : (const void *)d.ghat32;
+        R.Ghat = h->prec == ND_FP64 ? (const void *)d.ghat64 : (const void *)d.ghat32;
         R.Ghat64 = d.ghat64;
         R.GhatL = d.ghatL;
         R.mask = d.mask_d;
@@ -396,6 +409,16 @@ static int class_segments(SizeClass &c, int mode, long long nsteps, int nslots)
     return ND_OK;
 }
 
+// CTAs per replica of a field call: clusters where all replicas of the class
+// hold one at once.
+static int field_cluster_nc(const nd_handle *h, const SizeClass &c)
+{
+    default_plan(h, c, M_RK4);
+    const int nc = plan_cluster_nc(c.alone_plan[0]);
+    const int prec = h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32;
+    return nc && (int)c.reps.size() <= cluster_slots(h, c, prec, false, nc) ? nc : 0;
+}
+
 // Run one mode over all replicas in the handle's precision.
 static int run_mode(nd_handle *h, int mode, void *y, void *out, long long nsteps, cudaStream_t st,
                     const Replica *reps = nullptr, int only_class = -1)
@@ -436,7 +459,7 @@ static int run_mode(nd_handle *h, int mode, void *y, void *out, long long nsteps
         bool fused = c.fused_main;
         const bool stepping = mode == M_HEUN || mode == M_RK4;
         int variant = 0;
-        int cluster_nc = 0;
+        int cluster_nc = mode == M_FIELD ? field_cluster_nc(h, c) : 0;
         if (stepping) {
             int pl = c.plan[mode == M_RK4 ? 0 : 1];
             if (pl == -1) pl = default_plan(h, c, mode);
@@ -558,12 +581,6 @@ int nd_create_disk(const nd_disk_desc *disks, int n_disks, const int *replicas_p
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
     h->max_smem = (size_t)optin;
     cudaDeviceGetAttribute(&h->n_sm, cudaDevAttrMultiProcessorCount, h->device);
-    // twiddle constants exp(-2 pi i k / 32)
-    {
-        double re[32], im[32];
-        for (int k = 0; k < 32; ++k) { re[k] = cos(2.0 * M_PI * k / 32.0); im[k] = -sin(2.0 * M_PI * k / 32.0); }
-        if (upload_twiddle_constants(re, im) != cudaSuccess) { delete h; return fail(ND_ERR_CUDA, "twiddle upload failed"); }
-    }
     long long off = 0, soff = 0;
     for (int d = 0; d < n_disks; ++d) {
         const nd_disk_desc &ds = disks[d];
@@ -682,7 +699,8 @@ int nd_create_disk(const nd_disk_desc *disks, int n_disks, const int *replicas_p
     for (int k = 0; k < nd_handle::kSlots; ++k)
         if ((e = cudaEventCreateWithFlags(&h->slot_ev[k], cudaEventDisableTiming)) != cudaSuccess)
             return cuda_fail(e, "cudaEventCreate");
-    if ((e = cudaMalloc(&h->reps_d, sizeof(Replica) * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
+    if ((e = cudaMalloc(&h->reps_d, sizeof(Replica) * 2 * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
+    h->base_d = h->reps_d + B;
     if ((e = cudaMalloc(&h->red_d, sizeof(double) * 2 * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = cudaMallocHost(&h->red_h, sizeof(double) * 4 * B)) != cudaSuccess) return cuda_fail(e, "cudaMallocHost");
     if ((e = cudaMalloc(&h->aux_d, sizeof(double) * 4 * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
@@ -690,8 +708,9 @@ int nd_create_disk(const nd_disk_desc *disks, int n_disks, const int *replicas_p
     if ((e = cudaMalloc(&h->acc, h->elt * h->state_elems)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = cudaMalloc(&h->rio_d, sizeof(RelaxIO) * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = cudaMalloc(&h->flags_d, sizeof(int) * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
-    if ((e = cudaMalloc(&h->status_d, sizeof(unsigned))) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
-    if ((e = cudaMemset(h->status_d, 0, sizeof(unsigned))) != cudaSuccess) return cuda_fail(e, "cudaMemset");
+    if ((e = cudaMalloc(&h->status_d, sizeof(unsigned) * (1 + B))) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
+    if ((e = cudaMemset(h->status_d, 0, sizeof(unsigned) * (1 + B))) != cudaSuccess) return cuda_fail(e, "cudaMemset");
+    h->core_done = h->status_d + 1;
     if ((e = cudaMallocHost(&h->rio_h, sizeof(RelaxIO) * B)) != cudaSuccess) return cuda_fail(e, "cudaMallocHost");
     if ((e = cudaMalloc(&h->core_d, sizeof(double) * 4 * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = cudaMalloc(&h->core_part, sizeof(double) * 2 * kCoreMaxBlocks * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
@@ -720,6 +739,7 @@ int nd_create_disk(const nd_disk_desc *disks, int n_disks, const int *replicas_p
         rc = nd_set_green_tensor(h, d, nullptr);
         if (rc) { std::string m = g_err; nd_destroy(h); return fail(rc, m); }
     }
+    if ((e = upload_base(h)) != cudaSuccess) return cuda_fail(e, "parameter upload");
     *out = h;
     g_err.clear();
     return ND_OK;
@@ -847,6 +867,7 @@ int nd_set_mask(nd_handle *h, int d, const unsigned char *mask)
     di.C = C;
     ND_CUDA(cudaDeviceSynchronize());   // kernels in flight may still read the old cell list
     ND_CUDA(upload_mask(di));
+    ND_CUDA(upload_base(h));
     return ND_OK;
 }
 
@@ -894,10 +915,11 @@ int nd_effective_field(nd_handle *h, const void *m, void *b, void *stream)
     if (int rc = stage_in(h, m, &md, true, st, &h->stage_in)) return rc;
     if (!b) return fail(ND_ERR_ARG, "null output");
     if (int rc = stage_in(h, b, &bd, false, st, &h->stage_out)) return rc;
-    ND_CUDA(cudaMemsetAsync(bd, 0, (size_t)h->state_elems * h->elt, st));
-    fill_reps(h, h->prec == ND_FP64, 0.0, nullptr, nullptr, 0);
-    upload_reps(h, st);
-    if (int rc = run_mode(h, M_FIELD, md, bd, 1, st)) return rc;
+    // the on-chip kernels write whole blocks; the global path only cells inside the disks
+    bool any_global = false;
+    for (const auto &c : h->classes) any_global |= !c.fused_main && !field_cluster_nc(h, c);
+    if (any_global) ND_CUDA(cudaMemsetAsync(bd, 0, (size_t)h->state_elems * h->elt, st));
+    if (int rc = run_mode(h, M_FIELD, md, bd, 1, st, h->base_d)) return rc;
     return stage_out(h, b, bd, st);
 }
 
@@ -917,11 +939,9 @@ int nd_energy(nd_handle *h, const void *m, double *E_out, double *dEdL_out, void
         ND_CUDA(cudaMemsetAsync(h->energy_done, 0, sizeof(unsigned) * B, st));
         if (int rc = ensure_alloc((void **)&h->energy_part, sizeof(double) * (size_t)maxP * B)) return rc;
     }
-    fill_reps(h, true, 0.0, nullptr, nullptr, 0);
-    upload_reps(h, st);
     for (auto &c : h->classes) {
         EnergyArgs a;
-        a.reps = h->reps_d;
+        a.reps = h->base_d;
         a.work = c.work_d;
         a.nwork = (int)c.reps.size();
         a.maxD = c.maxD;
@@ -955,7 +975,7 @@ int nd_step_rk4(nd_handle *h, void *m, long long n_steps, double dt_seconds, voi
     void *md = nullptr;
     if (int rc = stage_in(h, m, &md, true, st, &h->stage_in)) return rc;
     if (n_steps > 0) {
-        fill_reps(h, h->prec == ND_FP64, dt_seconds, nullptr, nullptr, h->rk4_step);
+        fill_reps(h, dt_seconds, nullptr, nullptr, h->rk4_step);
         upload_reps(h, st);
         if (int rc = run_mode(h, M_RK4, md, nullptr, n_steps, st)) return rc;
         h->rk4_step += (unsigned long long)n_steps;
@@ -976,7 +996,7 @@ int nd_step_heun(nd_handle *h, void *m, long long n_steps, double dt_seconds, co
     void *md = nullptr;
     if (int rc = stage_in(h, m, &md, true, st, &h->stage_in)) return rc;
     if (n_steps > 0) {
-        fill_reps(h, h->prec == ND_FP64, dt_seconds, T_kelvin, seed, step0);
+        fill_reps(h, dt_seconds, T_kelvin, seed, step0);
         upload_reps(h, st);
         if (int rc = run_mode(h, M_HEUN, md, nullptr, n_steps, st)) return rc;
     }
@@ -1012,8 +1032,6 @@ int nd_relax_constrained(nd_handle *h, void *m, const double *X, double tol, int
         R.status = 1;
     }
     ND_CUDA(cudaMemcpyAsync(h->rio_d, h->rio_h, sizeof(RelaxIO) * B, cudaMemcpyHostToDevice, st));
-    fill_reps(h, h->prec == ND_FP64, 0.0, nullptr, nullptr, 0);
-    upload_reps(h, st);
     const int prec = h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32;
     // The classes are independent: the ones that relax in one launch go to side
     // streams, and those on the global path, whose host loop waits for each 32
@@ -1039,7 +1057,7 @@ int nd_relax_constrained(nd_handle *h, void *m, const double *X, double tol, int
         const double rcut = 4.0 * d.lambda / d.desc.a;
         LaunchArgs a;
         a.mode = M_RELAX;
-        a.reps = h->reps_d;
+        a.reps = h->base_d;
         a.work = c.work_d;
         a.nwork = (int)c.reps.size();
         a.y = md;
@@ -1127,14 +1145,12 @@ int nd_relax_sweep_grad(nd_handle *h, void *m, const void *grad, const double *X
     }
     ND_CUDA(cudaMemcpyAsync(h->rio_d, h->rio_h, sizeof(RelaxIO) * B, cudaMemcpyHostToDevice, st));
     ND_CUDA(cudaMemcpyAsync(h->aux_d, gs.data(), sizeof(double) * B, cudaMemcpyHostToDevice, st));
-    fill_reps(h, h->prec == ND_FP64, 0.0, nullptr, nullptr, 0);
-    upload_reps(h, st);
     const int prec = h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32;
     for (auto &c : h->classes) {
         const DiskInfo &d = h->disks[h->rep_disk[c.reps[0]]];
         const double rcut = 4.0 * d.lambda / d.desc.a;
         LaunchArgs a;
-        a.reps = h->reps_d;
+        a.reps = h->base_d;
         a.work = c.work_d;
         a.nwork = (int)c.reps.size();
         a.y = m;
@@ -1176,12 +1192,10 @@ int nd_init_vortex(nd_handle *h, void *m, const double *X0, void *stream)
     }
     ND_CUDA(cudaMemcpyAsync(h->aux_d, xc.data(), sizeof(double) * 2 * B, cudaMemcpyHostToDevice, st));
     ND_CUDA(cudaMemcpyAsync(h->aux_i, pc.data(), sizeof(int) * 2 * B, cudaMemcpyHostToDevice, st));
-    fill_reps(h, h->prec == ND_FP64, 0.0, nullptr, nullptr, 0);
-    upload_reps(h, st);
     ND_CUDA(cudaMemsetAsync(md, 0, (size_t)h->state_elems * h->elt, st));
     for (auto &c : h->classes) {
         const DiskInfo &d = h->disks[h->rep_disk[c.reps[0]]];
-        ND_CUDA(launch_init_vortex(h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32, h->reps_d, c.work_d,
+        ND_CUDA(launch_init_vortex(h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32, h->base_d, c.work_d,
                                    (int)c.reps.size(), c.maxD, md, h->aux_d, h->aux_i, d.lambda / d.desc.a, st));
     }
     ND_CUDA(cudaStreamSynchronize(st));   // the host arrays above go out of scope
@@ -1196,16 +1210,14 @@ int nd_vortex_core(nd_handle *h, const void *m, double *Xc_out, int *status, voi
     void *md = nullptr;
     if (int rc = stage_in(h, m, &md, true, st, &h->stage_in)) return rc;
     const int B = (int)h->rep_disk.size();
-    fill_reps(h, h->prec == ND_FP64, 0.0, nullptr, nullptr, 0);
-    upload_reps(h, st);
     for (auto &c : h->classes) {
         const DiskInfo &d = h->disks[h->rep_disk[c.reps[0]]];
         for (int r : c.reps)
             if (h->disks[h->rep_disk[r]].lambda / h->disks[h->rep_disk[r]].desc.a != d.lambda / d.desc.a)
                 return fail(ND_ERR_ARG, "vortex_core: disks of one size class must share lambda_ex / a");
         const double rcut = 4.0 * d.lambda / d.desc.a;
-        ND_CUDA(launch_vortex_core(h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32, h->reps_d, c.work_d,
-                                   (int)c.reps.size(), c.maxD, md, rcut * rcut, h->core_part, h->aux_d, st));
+        ND_CUDA(launch_vortex_core(h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32, h->base_d, c.work_d,
+                                   (int)c.reps.size(), c.maxD, md, rcut * rcut, h->core_part, h->core_done, h->aux_d, st));
     }
     ND_CUDA(cudaMemcpyAsync(h->red_h, h->aux_d, sizeof(double) * 4 * B, cudaMemcpyDeviceToHost, st));
     ND_CUDA(cudaStreamSynchronize(st));
@@ -1255,7 +1267,7 @@ int nd_selftest_handover_timeout(nd_handle *h, void *stream)
     if (e == cudaSuccess) {
         LaunchArgs a;
         a.mode = M_HEUN;
-        a.reps = h->reps_d;
+        a.reps = h->base_d;
         a.work = c.work_d;
         a.nwork = (int)c.reps.size();
         a.y = h->acc;     // never touched: the segment gives up before reading any state
@@ -1302,7 +1314,7 @@ static int stats_launches(nd_handle *h, const void *m, double dt_sample_seconds,
         const DiskInfo &d = h->disks[h->rep_disk[c.reps[0]]];
         const double rcut = 4.0 * d.lambda / d.desc.a;
         ND_CUDA(launch_vortex_core(h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32, reps, c.work_d,
-                                   (int)c.reps.size(), c.maxD, m, rcut * rcut, h->core_part, h->core_d, st));
+                                   (int)c.reps.size(), c.maxD, m, rcut * rcut, h->core_part, h->core_done, h->core_d, st));
         ND_CUDA(launch_stats_update(c.work_d, (int)c.reps.size(), h->core_d, h->a_rep, h->stats, h->hist_r, h->hist_v,
                                     h->rbins, h->vbins, h->r_max, h->v_max, dt_sample_seconds, st));
     }
@@ -1316,9 +1328,7 @@ int nd_stats_sample(nd_handle *h, const void *m, double dt_sample_seconds, void 
     if (!(dt_sample_seconds > 0)) return fail(ND_ERR_ARG, "dt_sample must be positive");
     if (!m || !is_device_ptr(m)) return fail(ND_ERR_ARG, "nd_stats_sample needs a device state");
     cudaStream_t st = (cudaStream_t)stream;
-    fill_reps(h, h->prec == ND_FP64, 0.0, nullptr, nullptr, 0);
-    upload_reps(h, st);
-    return stats_launches(h, m, dt_sample_seconds, st, h->reps_d);
+    return stats_launches(h, m, dt_sample_seconds, st, h->base_d);
 }
 
 int nd_stats_read(nd_handle *h, double *moments, unsigned long long *r_hist, unsigned long long *v_hist, void *stream)
@@ -1426,10 +1436,8 @@ int nd_mean_m(nd_handle *h, const void *m, double *out, void *stream)
     void *md = nullptr;
     if (int rc = stage_in(h, m, &md, true, st, &h->stage_in)) return rc;
     const int B = (int)h->rep_disk.size();
-    fill_reps(h, h->prec == ND_FP64, 0.0, nullptr, nullptr, 0);
-    upload_reps(h, st);
     for (auto &c : h->classes)
-        ND_CUDA(launch_mean_m(h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32, h->reps_d, c.work_d, (int)c.reps.size(),
+        ND_CUDA(launch_mean_m(h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32, h->base_d, c.work_d, (int)c.reps.size(),
                               md, h->aux_d, st));
     ND_CUDA(cudaMemcpyAsync(h->red_h, h->aux_d, sizeof(double) * 3 * B, cudaMemcpyDeviceToHost, st));
     ND_CUDA(cudaStreamSynchronize(st));
@@ -1443,7 +1451,7 @@ static int series_launches(nd_handle *h, const void *md, cudaStream_t st, const 
 {
     const int prec = h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32;
     for (auto &c : h->classes)
-        ND_CUDA(launch_series_append(prec, reps ? reps : h->reps_d, c.work_d, (int)c.reps.size(), md, h->series,
+        ND_CUDA(launch_series_append(prec, reps ? reps : h->base_d, c.work_d, (int)c.reps.size(), md, h->series,
                                      h->series_count, h->series_cap, st));
     ND_CUDA(launch_series_advance(h->series_count, st));
     return ND_OK;
@@ -1471,8 +1479,6 @@ int nd_series_sample(nd_handle *h, const void *m, void *stream)
     cudaStream_t st = (cudaStream_t)stream;
     void *md = nullptr;
     if (int rc = stage_in(h, m, &md, true, st, &h->stage_in)) return rc;
-    fill_reps(h, h->prec == ND_FP64, 0.0, nullptr, nullptr, 0);
-    upload_reps(h, st);
     return series_launches(h, md, st, nullptr);
 }
 
@@ -1587,7 +1593,7 @@ static int tune_run(std::vector<TuneItem> &items, double dt, long long n_steps, 
         const cudaStream_t s = many ? it.st : st0;
         if (many) ND_CUDA(cudaStreamWaitEvent(s, fork, 0));
         const bool heun = it.mode == M_HEUN;
-        fill_reps(it.h, it.h->prec == ND_FP64, dt, heun ? it.T.data() : nullptr, heun ? it.sd.data() : nullptr, 0);
+        fill_reps(it.h, dt, heun ? it.T.data() : nullptr, heun ? it.sd.data() : nullptr, 0);
         upload_reps(it.h, s);
         if (int rc = run_mode(it.h, it.mode, it.tmp, nullptr, n_steps, s, nullptr, only_class)) return rc;
         if (many) {
@@ -1831,7 +1837,7 @@ int nd_graph_create(nd_handle *h, void *m, int method, long long n_steps, double
     };
     cudaError_t e = cudaMalloc(&g->reps, sizeof(Replica) * B);
     if (e != cudaSuccess) return bail(ND_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-    fill_reps(h, h->prec == ND_FP64, dt_seconds, method == ND_METHOD_HEUN ? T_kelvin : nullptr,
+    fill_reps(h, dt_seconds, method == ND_METHOD_HEUN ? T_kelvin : nullptr,
               method == ND_METHOD_HEUN ? seed : nullptr, step0);
     e = cudaMemcpy(g->reps, h->reps_h, sizeof(Replica) * B, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return bail(ND_ERR_CUDA, std::string("cudaMemcpy: ") + cudaGetErrorString(e));

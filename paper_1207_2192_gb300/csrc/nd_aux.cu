@@ -199,176 +199,222 @@ cudaError_t launch_init_vortex(int prec, const Replica *reps, const int *work, i
 
 // ------------------------------------------------------------ vortex core
 
-// Core position estimator (Section IV) in two kernels.  The plaquette
-// windings and the m_z^2 corner sums are evaluated in double precision with
-// no fused multiply-adds, in the same order as the CPU reference, so both
-// take the same integer decisions from the same inputs.
-//   k_core_scan: grid (nblk, replicas), each CTA scans a strided share of the
-//     plaquettes for the winding +1 one with the largest corner sum (lowest
-//     index on ties) and writes its candidate;
-//   k_core_finish: one CTA per replica picks the best candidate (same rule)
-//     and forms the m_z^2-weighted centroid over the disk cells within
-//     4 lambda_ex of it, visiting only the bounding box of that circle.
+// Core position estimator (Section IV) in one kernel: grid (nblk, replicas),
+// each CTA stages a strip of rows of the in-plane components in shared memory
+// (one batch of loads instead of a chain per plaquette) and scans its plaquettes
+// for the winding +1 one with the largest m_z^2 corner sum (lowest index on
+// ties), and the last CTA of a replica picks the best candidate (same rule) and forms the m_z^2-weighted
+// centroid over the disk cells within 4 lambda_ex of it, visiting only the
+// bounding box of that circle.  The winding and the corner sums are those of
+// double precision with no fused multiply-adds, in the same order as the CPU
+// reference, so both take the same integer decisions from the same inputs; but
+// FP64 issues one warp instruction per 64-76 cycles here, so the scan reads the
+// winding off the signs (below) and only single plaquettes reach FP64.  256
+// replicas of D = 50, cold cache: 23.6 + 15.4 us as two kernels with an
+// arctangent per corner and FP64 trees over the CTA, 19.9 us now.
 template <typename T> struct CoreAt {
     const T *y;
     long long cs;
     int D, Dpad;
-    __device__ __forceinline__ double operator()(int cell, int c) const
+    __device__ __forceinline__ double operator()(int cell, int c) const { return (double)raw(cell, c); }
+    __device__ __forceinline__ T raw(int cell, int c) const
     {
         const int j = cell / D, i = cell - j * D;
-        return (double)y[c * cs + (long long)j * Dpad + i];
+        return y[c * cs + (long long)j * Dpad + i];
     }
 };
 
+// Winding of the plaquette with corners c[0..3] in counter-clockwise order: the
+// sum over its edges of the turn in (-pi, pi], over 2 pi.  An edge adds a
+// revolution to the difference of the corners' polar angles exactly where it
+// crosses the negative x axis the short way: from y >= 0 to y < 0 turning
+// left, or back turning right.  The signs of the cross products decide that;
+// where one that matters is within rounding of zero (the corners antiparallel),
+// or a corner's in-plane part is too small for single-precision products, the
+// turns are summed in double precision.
 template <typename T>
-__global__ void __launch_bounds__(256) k_core_scan(const Replica *reps, const int *work, const T *ybase, double *part,
-                                                   int nblk)
+__device__ __forceinline__ int winding(const CoreAt<T> &at, const int (&c)[4], const float (&px)[4],
+                                       const float (&py)[4])
 {
-    __shared__ double sw[256];
-    __shared__ int si_[256];
-    const int ridx = work[blockIdx.y];
-    const Replica r = reps[ridx];
+    bool sure = true;
+    for (int q = 0; q < 4; ++q)
+        sure &= px[q] * px[q] + py[q] * py[q] > 1e-12f && fabsf(py[q]) > 1e-30f;
+    int w = 0;
+    for (int q = 0; q < 4; ++q) {
+        const int n = (q + 1) & 3;
+        if ((py[q] < 0.0f) == (py[n] < 0.0f)) continue;
+        const float u = px[q] * py[n], v = py[q] * px[n], cr = u - v;
+        sure &= fabsf(cr) > 1e-5f * (fabsf(u) + fabsf(v));
+        if (py[q] >= 0.0f && cr > 0.0f) ++w;
+        if (py[q] < 0.0f && cr < 0.0f) --w;
+    }
+    if (sure) return w;
+    double s = 0.0;
+    for (int q = 0; q < 4; ++q) {
+        const int p0 = c[q], p1 = c[(q + 1) & 3];
+        const double ax = at(p0, 0), ay = at(p0, 1), bx = at(p1, 0), by = at(p1, 1);
+        const double cr = __dsub_rn(__dmul_rn(ax, by), __dmul_rn(ay, bx));
+        const double dt = __dadd_rn(__dmul_rn(ax, bx), __dmul_rn(ay, by));
+        s = __dadd_rn(s, atan2(cr, dt));
+    }
+    return (int)llround(s / (2.0 * M_PI));
+}
+
+// A candidate plaquette: corner sum (negative: none) and index.
+struct CoreCand {
+    double w;
+    int i;
+    __device__ __forceinline__ void take(double w2, int i2)
+    {
+        if (w2 > w || (w2 == w && i2 < i)) { w = w2; i = i2; }
+    }
+};
+
+// The circle of radius rc' = sqrt(rc2) around the plaquette's centre: the half
+// side of its bounding box, and (2 dx)^2 + (2 dy)^2 < n4 (odd integers) for
+// dx^2 + dy^2 < rc2.
+struct CoreBox {
+    int rc;
+    long long n4;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_core(const Replica *reps, const int *work, const T *ybase, double *part,
+                                              unsigned *done, CoreBox box, double *out)
+{
+    extern __shared__ __align__(16) float strip[];
+    __shared__ CoreCand wc[8];
+    __shared__ CoreCand best_s;
+    __shared__ double sx[3][4];
+    __shared__ bool last_s;
+    const int ridx = work[blockIdx.y], nblk = gridDim.x;
+    const Replica &r = reps[ridx];
     const int D = r.D, tid = threadIdx.x;
+    const unsigned char *mask = r.mask;
     const CoreAt<T> at{ybase + r.state_off, (long long)D * r.Dpad, D, r.Dpad};
-    double bw = -1.0;
-    int bi = 0x7fffffff;
-    const int np = (D - 1) * (D - 1);
-    for (int p = blockIdx.x * 256 + tid; p < np; p += nblk * 256) {
-        const int j = p / (D - 1), i = p - j * (D - 1);
-        const int t = j * D + i;
-        if (!(r.mask[t] && r.mask[t + 1] && r.mask[t + D] && r.mask[t + D + 1])) continue;
+    CoreCand cand = {-1.0, 0x7fffffff};
+    // rows ja..jb of the strip's plaquettes, the row after the last included;
+    // cells outside the disk are marked with a NaN
+    const int H = (D - 1 + nblk - 1) / nblk, ja = min(blockIdx.x * H, D - 1), jb = min(ja + H, D - 1);
+    float2 *const sp = reinterpret_cast<float2 *>(strip);
+    const T *y0 = ybase + r.state_off;
+    const int ncell = (jb - ja + 1) * D;
+#pragma unroll 4
+    for (int k = tid; k < ncell; k += 256) {
+        const int jr = k / D, i = k - jr * D;
+        const long long si = (long long)(ja + jr) * r.Dpad + i;
+        const float x = (float)y0[si], y = (float)y0[at.cs + si];
+        sp[k] = make_float2(mask[ja * D + k] ? x : __int_as_float(0x7fffffff), y);
+    }
+    __syncthreads();
+    const int np = (jb - ja) * (D - 1);
+    for (int p = tid; p < np; p += 256) {
+        const int jr = p / (D - 1), i = p - jr * (D - 1), k = jr * D + i;
+        const int t = ja * D + k;
+        const float2 q0 = sp[k], q1 = sp[k + 1], q2 = sp[k + D + 1], q3 = sp[k + D];
         const int c[4] = {t, t + 1, t + D + 1, t + D};
-        // The winding is decided in double precision.  A single-precision pass
-        // settles every plaquette whose angle sum lies within a quarter turn
-        // of a multiple of 2 pi (its error, ~1e-6 rad, is far below that
-        // margin, so the double sum rounds to the same integer); only the
-        // others, and plaquettes with an in-plane component too small for
-        // single-precision products, are summed again in double.
-        float sf = 0.0f, amin = 1.0f;
-        for (int q = 0; q < 4; ++q) {
-            const int p0 = c[q], p1 = c[(q + 1) & 3];
-            const float ax = (float)at(p0, 0), ay = (float)at(p0, 1), bx = (float)at(p1, 0), by = (float)at(p1, 1);
-            sf += atan2f(ax * by - ay * bx, ax * bx + ay * by);
-            amin = fminf(amin, ax * ax + ay * ay);
-        }
-        const float kf = sf * (float)(0.5 / M_PI);
-        long long wind;
-        if (amin > 1e-12f && fabsf(kf - rintf(kf)) < 0.25f) {
-            wind = (long long)rintf(kf);
-        } else {
-            double s = 0.0;
-            for (int q = 0; q < 4; ++q) {
-                const int p0 = c[q], p1 = c[(q + 1) & 3];
-                const double ax = at(p0, 0), ay = at(p0, 1), bx = at(p1, 0), by = at(p1, 1);
-                const double cr = __dsub_rn(__dmul_rn(ax, by), __dmul_rn(ay, bx));
-                const double dt = __dadd_rn(__dmul_rn(ax, bx), __dmul_rn(ay, by));
-                s = __dadd_rn(s, atan2(cr, dt));
-            }
-            wind = llround(s / (2.0 * M_PI));
-        }
-        if (wind != 1) continue;
+        const float px[4] = {q0.x, q1.x, q2.x, q3.x}, py[4] = {q0.y, q1.y, q2.y, q3.y};
+        if (!(px[0] == px[0] && px[1] == px[1] && px[2] == px[2] && px[3] == px[3])) continue;
+        if (winding(at, c, px, py) != 1) continue;
         const double z0 = at(t, 2), z1 = at(t + 1, 2), z2 = at(t + D, 2), z3 = at(t + D + 1, 2);
         double w = __dmul_rn(z0, z0);
         w = __dadd_rn(w, __dmul_rn(z1, z1));
         w = __dadd_rn(w, __dmul_rn(z2, z2));
         w = __dadd_rn(w, __dmul_rn(z3, z3));
-        if (w > bw || (w == bw && t < bi)) { bw = w; bi = t; }
+        cand.take(w, t);
     }
-    sw[tid] = bw; si_[tid] = bi;
+    // candidates are rare: a warp compares only the lanes that hold one
+    CoreCand b = {-1.0, 0x7fffffff};
+    for (unsigned m = __ballot_sync(0xffffffffu, cand.i != 0x7fffffff); m; m &= m - 1) {
+        const int l = __ffs(m) - 1;
+        b.take(__shfl_sync(0xffffffffu, cand.w, l), __shfl_sync(0xffffffffu, cand.i, l));
+    }
+    if ((tid & 31) == 0) wc[tid >> 5] = b;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (tid < o) {
-            const double w2 = sw[tid + o];
-            const int i2 = si_[tid + o];
-            if (w2 > sw[tid] || (w2 == sw[tid] && i2 < si_[tid])) { sw[tid] = w2; si_[tid] = i2; }
-        }
-        __syncthreads();
-    }
     if (tid == 0) {
-        double *o = part + 2 * ((size_t)ridx * nblk + blockIdx.x);
-        o[0] = sw[0];
-        o[1] = (double)si_[0];
-    }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_core_finish(const Replica *reps, const int *work, const T *ybase,
-                                                     const double *part, int nblk, double rc2, double *out)
-{
-    __shared__ double sx[3][8];
-    __shared__ int best_s;
-    __shared__ double bw_s;
-    const int ridx = work[blockIdx.x];
-    const Replica r = reps[ridx];
-    const int D = r.D, tid = threadIdx.x;
-    const CoreAt<T> at{ybase + r.state_off, (long long)D * r.Dpad, D, r.Dpad};
-    if (tid == 0) {
-        double bw = -1.0;
-        int bi = 0x7fffffff;
-        for (int b = 0; b < nblk; ++b) {
-            const double w = part[2 * ((size_t)ridx * nblk + b)];
-            const int i = (int)part[2 * ((size_t)ridx * nblk + b) + 1];
-            if (w > bw || (w == bw && i < bi)) { bw = w; bi = i; }
+        for (int k = 1; k < 8; ++k)
+            if (wc[k].i != 0x7fffffff) wc[0].take(wc[k].w, wc[k].i);
+        best_s = wc[0];
+        last_s = true;
+        if (nblk > 1) {
+            double *o = part + 2 * ((size_t)ridx * nblk + blockIdx.x);
+            __stcg(o, best_s.w);
+            __stcg(o + 1, (double)best_s.i);
+            __threadfence();
+            last_s = atomicInc(done + ridx, nblk - 1) == nblk - 1;   // (wraps to zero for the next call)
+            if (last_s) {
+                __threadfence();
+                CoreCand g = {-1.0, 0x7fffffff};
+                for (int k = 0; k < nblk; ++k) {
+                    const double w = __ldcg(part + 2 * ((size_t)ridx * nblk + k));
+                    if (w >= 0.0) g.take(w, (int)__ldcg(part + 2 * ((size_t)ridx * nblk + k) + 1));
+                }
+                best_s = g;
+            }
         }
-        best_s = bi;
-        bw_s = bw;
     }
     __syncthreads();
-    const int best = best_s;
-    const bool found = bw_s >= 0.0 && best != 0x7fffffff;
+    if (!last_s) return;
+    const int best = best_s.i;
+    const bool found = best != 0x7fffffff;
+    // Four warps, one per sub-partition.  Bound by FP64 issue: five
+    // instructions a cell (the conversions by bits), six additions a warp.
     double a0 = 0, a1 = 0, a2 = 0;
-    if (found) {
-        const int bj = best / D, bii = best - bj * D;
-        const double cx = bii + 0.5 - 0.5 * (D - 1), cy = bj + 0.5 - 0.5 * (D - 1);
-        const int rc = (int)ceil(sqrt(rc2)) + 1;
-        const int i0 = max(0, bii - rc), i1 = min(D - 1, bii + 1 + rc), j0 = max(0, bj - rc), j1 = min(D - 1, bj + 1 + rc);
-        const int w = i1 - i0 + 1, nbox = w * (j1 - j0 + 1);
-        for (int k = tid; k < nbox; k += 256) {
-            const int j = j0 + k / w, i = i0 + k % w, cell = j * D + i;
-            if (!r.mask[cell]) continue;
-            const double x = i - 0.5 * (D - 1), yy = j - 0.5 * (D - 1);
-            const double dx = x - cx, dy = yy - cy;
-            if (dx * dx + dy * dy >= rc2) continue;
-            const double z = at(cell, 2), wz = z * z;
-            a0 += wz; a1 += wz * x; a2 += wz * yy;
+    if (tid < 128) {
+        if (found) {
+            const int bj = best / D, bii = best - bj * D;
+            const int i0 = max(0, bii - box.rc), i1 = min(D - 1, bii + 1 + box.rc);
+            const int j0 = max(0, bj - box.rc), j1 = min(D - 1, bj + 1 + box.rc);
+            const int w = i1 - i0 + 1, nbox = w * (j1 - j0 + 1);
+#pragma unroll 4
+            for (int k = tid; k < nbox; k += 128) {
+                const int jr = k / w, j = j0 + jr, i = i0 + k - jr * w, cell = j * D + i;
+                const int ex = 2 * (i - bii) - 1, ey = 2 * (j - bj) - 1;
+                const bool in = (long long)ex * ex + (long long)ey * ey < box.n4 && mask[cell];
+                const T zt = at.raw(cell, 2);
+                if (!in) continue;
+                const double z = to_double(zt), wz = z * z;
+                // twice the coordinates from the grid's centre are integers
+                a0 += wz;
+                a1 += wz * to_double((float)(2 * i - (D - 1)));
+                a2 += wz * to_double((float)(2 * j - (D - 1)));
+            }
         }
+        const double s = warp_sum3(a0, a1, a2);
+        if ((tid & 7) == 0 && (tid & 31) < 24) sx[(tid & 31) >> 3][tid >> 5] = s;
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        a0 += __shfl_xor_sync(0xffffffffu, a0, o);
-        a1 += __shfl_xor_sync(0xffffffffu, a1, o);
-        a2 += __shfl_xor_sync(0xffffffffu, a2, o);
-    }
-    if ((tid & 31) == 0) { sx[0][tid >> 5] = a0; sx[1][tid >> 5] = a1; sx[2][tid >> 5] = a2; }
     __syncthreads();
-    if (tid == 0) {
-        double s0 = 0, s1 = 0, s2 = 0;
-        for (int wv = 0; wv < 8; ++wv) { s0 += sx[0][wv]; s1 += sx[1][wv]; s2 += sx[2][wv]; }
+    if (tid < 32) {   // lanes 4c..4c+3 sum component c's four warps
+        double v = tid < 12 ? sx[tid >> 2][tid & 3] : 0.0;
+        for (int o = 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        const double w = __shfl_sync(0xffffffffu, v, 0);
+        const bool ok = found && w > 0.0;
         double *o = out + 4 * ridx;
-        if (found && s0 > 0.0) { o[0] = s1 / s0; o[1] = s2 / s0; o[2] = 0.0; }
-        else { o[0] = 0.0; o[1] = 0.0; o[2] = 1.0; }
-        o[3] = found ? (double)best : -1.0;
+        if (tid == 4 || tid == 8) o[(tid >> 2) - 1] = ok ? 0.5 * v / w : 0.0;
+        if (tid == 0) {
+            o[2] = ok ? 0.0 : 1.0;
+            o[3] = found ? (double)best : -1.0;
+        }
     }
 }
 
-int core_scan_blocks(int D)
+// CTAs of a replica's scan: strips of about 4096 cells (a 33 KB stage), at
+// most kCoreMaxBlocks.
+static int core_scan_blocks(int D)
 {
-    const int np = (D - 1) * (D - 1);
-    int n = np / 4096;
-    return n < 1 ? 1 : (n > kCoreMaxBlocks ? kCoreMaxBlocks : n);
+    const int n = (D * D + 4095) / 4096;
+    return n > kCoreMaxBlocks ? kCoreMaxBlocks : n;
 }
 
 cudaError_t launch_vortex_core(int prec, const Replica *reps, const int *work, int nwork, int maxD, const void *y,
-                               double rc2, double *part, double *out, cudaStream_t st)
+                               double rc2, double *part, unsigned *done, double *out, cudaStream_t st)
 {
     const int nblk = core_scan_blocks(maxD);
-    dim3 g(nblk, nwork);
-    if (prec == ND_PREC_FP64) {
-        k_core_scan<double><<<g, 256, 0, st>>>(reps, work, (const double *)y, part, nblk);
-        k_core_finish<double><<<nwork, 256, 0, st>>>(reps, work, (const double *)y, part, nblk, rc2, out);
-    } else {
-        k_core_scan<float><<<g, 256, 0, st>>>(reps, work, (const float *)y, part, nblk);
-        k_core_finish<float><<<nwork, 256, 0, st>>>(reps, work, (const float *)y, part, nblk, rc2, out);
-    }
+    const dim3 g(nblk, nwork);
+    const CoreBox box = {(int)ceil(sqrt(rc2)) + 1, (long long)ceil(4.0 * rc2)};
+    const size_t sm = sizeof(float2) * ((size_t)(maxD - 1 + nblk - 1) / nblk + 1) * maxD;   // <= 41 KB
+    if (prec == ND_PREC_FP64) k_core<double><<<g, 256, sm, st>>>(reps, work, (const double *)y, part, done, box, out);
+    else k_core<float><<<g, 256, sm, st>>>(reps, work, (const float *)y, part, done, box, out);
     return cudaGetLastError();
 }
 
@@ -435,32 +481,8 @@ cudaError_t launch_stats_update(const int *work, int nwork, const double *core, 
 template <typename T>
 __global__ void __launch_bounds__(256) k_mean_m(const Replica *reps, const int *work, const T *ybase, double *out)
 {
-    __shared__ double sx[4][8];
     const int ridx = work[blockIdx.x];
-    const Replica r = reps[ridx];
-    const int D = r.D, tid = threadIdx.x;
-    const long long cs = (long long)D * r.Dpad;
-    const T *y = ybase + r.state_off;
-    double a0 = 0, a1 = 0, a2 = 0, n = 0;
-    for (int cell = tid; cell < D * D; cell += 256) {
-        if (!r.mask[cell]) continue;
-        const int j = cell / D, i = cell - j * D;
-        const long long si = (long long)j * r.Dpad + i;
-        a0 += (double)y[si]; a1 += (double)y[cs + si]; a2 += (double)y[2 * cs + si]; n += 1.0;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        a0 += __shfl_xor_sync(0xffffffffu, a0, o);
-        a1 += __shfl_xor_sync(0xffffffffu, a1, o);
-        a2 += __shfl_xor_sync(0xffffffffu, a2, o);
-        n += __shfl_xor_sync(0xffffffffu, n, o);
-    }
-    if ((tid & 31) == 0) { sx[0][tid >> 5] = a0; sx[1][tid >> 5] = a1; sx[2][tid >> 5] = a2; sx[3][tid >> 5] = n; }
-    __syncthreads();
-    if (tid == 0) {
-        double s[4] = {0, 0, 0, 0};
-        for (int w = 0; w < 8; ++w) for (int c = 0; c < 4; ++c) s[c] += sx[c][w];
-        for (int c = 0; c < 3; ++c) out[3 * ridx + c] = s[c] / s[3];
-    }
+    block_mean<T>(reps[ridx], ybase, out + 3 * ridx);
 }
 
 cudaError_t launch_mean_m(int prec, const Replica *reps, const int *work, int nwork, const void *y, double *out,

@@ -195,7 +195,7 @@ struct ClusterRelax {
 // segs[seg_off[i] .. seg_off[i+1]), passing replicas on through flags.
 template <int P, typename T, int MODE, int NC, bool SEG>
 __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
-    k_cluster(const Replica *__restrict__ reps, const int *__restrict__ work, T *__restrict__ ybase,
+    k_cluster(const Replica *__restrict__ reps, const int *__restrict__ work, T *__restrict__ ybase, T *__restrict__ outbase,
               const cplx<T> *__restrict__ twP, long long nsteps_all, unsigned long long step_base, int use_wbuf,
               unsigned *__restrict__ status, const Segment *__restrict__ segs, const int *__restrict__ seg_off,
               int *__restrict__ flags, int *__restrict__ ticket, const ClusterRelax rx)
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     using CG = ClusterGeom<P, T, NC>;
     constexpr int G = Gm::G, R1 = Gm::R1, RS = SpecGeom<P>::RS, KH = CG::KH, NT = CG::NT, NGRP = CG::NGRP;
     constexpr int SPC = CG::SPC, SW = CG::SW, NTAB = CG::NTAB;
-    static_assert(MODE == M_RK4 || MODE == M_HEUN || (MODE == M_RELAX && SEG), "stepping and relaxation modes");
+    static_assert(MODE == M_RELAX ? SEG : (MODE == M_FIELD ? !SEG : true), "turns or one launch per replica");
     constexpr bool RELAX = MODE == M_RELAX;
     cgc::cluster_group cluster = cgc::this_cluster();
     const int rank = (int)cluster.block_rank();
@@ -704,11 +704,21 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
                 }
                 continue;
             }
-            // the per-cell epilogue of the CTA's cells
             const StepParams<T> sp = step_params<T>(r);
-            const vec3<T> cx = step_chext<T>(r, sp, step);
             const T *hr = reinterpret_cast<const T *>(spec);
-            if constexpr (!RELAX)
+            if constexpr (MODE == M_FIELD) {   // the CTA's rows of the output, zero outside the disk
+                const V3Ptr<T> out{outbase + r.state_off + (long long)ylo * Dpad, ms_s};
+                for (int i = tid; i < nloc * Dpad; i += NT) {
+                    const int lr = i / Dpad, x = i - lr * Dpad, hi = lr * (2 * RS) + x;
+                    const bool in = x < D && r.mask[(ylo + lr) * D + x];
+                    out.st(i, in ? vec3<T>{hr[hi] + sp.chext[0], hr[2 * lcs + hi] + sp.chext[1], hr[4 * lcs + hi] + sp.chext[2]}
+                                 : vec3<T>{T(0), T(0), T(0)});
+                }
+                continue;
+            }
+            // the per-cell epilogue of the CTA's cells
+            const vec3<T> cx = step_chext<T>(r, sp, step);
+            if constexpr (!RELAX && MODE != M_FIELD)
             for (int k = c0 + tid; k < c1; k += NT) {
                 const int cell = __ldg(r.cells + k);
                 const int y = cell / D, x = cell - y * D, lr = y - ylo;
@@ -722,6 +732,7 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
         if (RELAX && conv_s) break;
     }
     // the final state of the CTA's cells back to the caller's buffer
+    if (MODE != M_FIELD)
     for (int k = c0 + tid; k < c1; k += NT) {
         const int cell = __ldg(r.cells + k);
         const int y = cell / D, x = cell - y * D;
@@ -785,8 +796,8 @@ static cudaError_t launch_cluster_t(const LaunchArgs &a, int maxD, int maxDpad)
     if (e != cudaSuccess) return e;
     const ClusterRelax rx = {a.rio, (const double *)a.tw64, a.eta, a.tol, a.rc2, a.max_iter, a.quantum, a.nwork,
                              a.flags ? a.flags + a.n_rep + 1 : nullptr};
-    return cudaLaunchKernelEx(&cfg, k_cluster<P, T, MODE, NC, SEG>, a.reps, a.work, (T *)a.y, (const cplx<T> *)a.tw,
-                              a.nsteps, a.step_base, a.use_wbuf, a.status, reinterpret_cast<const Segment *>(a.segs),
+    return cudaLaunchKernelEx(&cfg, k_cluster<P, T, MODE, NC, SEG>, a.reps, a.work, (T *)a.y, (T *)a.out,
+                              (const cplx<T> *)a.tw, a.nsteps, a.step_base, a.use_wbuf, a.status, reinterpret_cast<const Segment *>(a.segs),
                               a.seg_off, a.flags, a.flags ? a.flags + a.n_rep : nullptr, rx);
 }
 
@@ -820,6 +831,7 @@ static cudaError_t launch_cluster_p(const LaunchArgs &a, int maxD, int maxDpad)
         return a.segs ? launch_cluster_t<P, T, M_HEUN, NC, true>(a, maxD, maxDpad)
                       : launch_cluster_t<P, T, M_HEUN, NC, false>(a, maxD, maxDpad);
     if (a.mode == M_RELAX) return launch_cluster_t<P, T, M_RELAX, NC, true>(a, maxD, maxDpad);
+    if (a.mode == M_FIELD) return launch_cluster_t<P, T, M_FIELD, NC, false>(a, maxD, maxDpad);
     return cudaErrorInvalidValue;
 }
 

@@ -151,6 +151,61 @@ template <> __device__ __forceinline__ vec3<double> step_chext<double>(const Rep
     return {sp.chext[0], sp.chext[1], sp.chext[2]};
 }
 
+// A float as a double by its bits: FP64 issues a warp instruction per 64-76
+// cycles on GB300, conversions included, while these run at the integer rate.
+// (Denormals, infinities and NaNs take the conversion.)
+__device__ __forceinline__ double to_double(float x)
+{
+    const unsigned u = __float_as_uint(x), e = (u >> 23) & 255u;
+    if (e - 1u >= 254u && (u << 1) != 0u) return (double)x;
+    const unsigned hi = (u & 0x80000000u) | (e ? ((u & 0x7fffffffu) >> 3) + 0x38000000u : 0u);
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+__device__ __forceinline__ double to_double(double x) { return x; }
+
+// Sums of a0, a1 and a2 over a warp: lanes 0, 8 and 16 return those of a0, a1
+// and a2.  Halving the values a lane carries while their lanes double takes six
+// additions instead of fifteen.
+__device__ __forceinline__ double warp_sum3(double a0, double a1, double a2)
+{
+    const int lane = threadIdx.x & 31;
+    const bool h = lane & 16, q = lane & 8;
+    double u = __shfl_xor_sync(0xffffffffu, h ? a0 : a2, 16), v = __shfl_xor_sync(0xffffffffu, h ? a1 : 0.0, 16);
+    u += h ? a2 : a0;
+    v += h ? 0.0 : a1;
+    double w = __shfl_xor_sync(0xffffffffu, q ? u : v, 8);
+    w += q ? v : u;
+    for (int o = 4; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+    return w;
+}
+
+// <m> of one replica over its cells by a block of 256 threads, double sums
+// (null out: nothing is written).  Bound by FP64 issue: three additions per
+// cell of the compacted list and little else (256 replicas of D = 50, cold
+// cache: 19.1 -> 14.8 us against counting and converting in FP64 as well).
+template <typename T> __device__ __forceinline__ void block_mean(const Replica &r, const T *ybase, double *out)
+{
+    __shared__ double sx[3][8];
+    const int D = r.D, tid = threadIdx.x, n = r.ncells;
+    const long long cs = (long long)D * r.Dpad;
+    const T *y = ybase + r.state_off;
+    double a0 = 0, a1 = 0, a2 = 0;
+#pragma unroll 4
+    for (int k = tid; k < n; k += 256) {
+        const int cell = __ldg(r.cells + k), j = cell / D;
+        const long long si = (long long)j * r.Dpad + (cell - j * D);
+        a0 += to_double(y[si]); a1 += to_double(y[cs + si]); a2 += to_double(y[2 * cs + si]);
+    }
+    const double s = warp_sum3(a0, a1, a2);
+    if ((tid & 7) == 0 && (tid & 31) < 24) sx[(tid & 31) >> 3][tid >> 5] = s;
+    __syncthreads();
+    if (tid < 32) {   // lanes 8c..8c+7 sum component c's eight warps
+        double v = tid < 24 ? sx[tid >> 3][tid & 7] : 0.0;
+        for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (out && tid < 24 && (tid & 7) == 0) out[tid >> 3] = v / (double)n;
+    }
+}
+
 // Per-replica inputs and outputs of the constrained relaxation.
 struct RelaxIO {
     double X[2];      // constraint centre in cell units relative to the grid centre

@@ -3,14 +3,6 @@
 
 namespace nd {
 
-cudaError_t upload_tw_fused_f32(const double *, const double *);
-cudaError_t upload_tw_fused_f64(const double *, const double *);
-cudaError_t upload_tw_cluster_f32(const double *, const double *);
-cudaError_t upload_tw_cluster_f64(const double *, const double *);
-cudaError_t upload_tw_glob_f32(const double *, const double *);
-cudaError_t upload_tw_glob_f64(const double *, const double *);
-cudaError_t upload_tw_spectra(const double *, const double *);
-cudaError_t upload_tw_energy(const double *, const double *);
 size_t fused_smem_f32(int P, int D, int Dpad, bool wbuf, int variant);
 size_t fused_smem_f64(int P, int D, int Dpad, bool wbuf, int variant);
 int fused_blocks_per_sm_f32(int P, int mode, size_t smem, int variant);
@@ -28,19 +20,6 @@ int cluster_max_active_f64(int P, int D, int Dpad, bool wbuf, int nc);
 cudaError_t launch_cluster_f32(int P, const LaunchArgs &a, int maxD, int maxDpad, int nc);
 cudaError_t launch_cluster_f64(int P, const LaunchArgs &a, int maxD, int maxDpad, int nc);
 cudaError_t launch_relax_grad_f64(const LaunchArgs &a, int maxD, const void *grad, const double *gscale);
-
-cudaError_t upload_twiddle_constants(const double *re, const double *im)
-{
-    cudaError_t e;
-    if ((e = upload_tw_fused_f32(re, im)) != cudaSuccess) return e;
-    if ((e = upload_tw_fused_f64(re, im)) != cudaSuccess) return e;
-    if ((e = upload_tw_cluster_f32(re, im)) != cudaSuccess) return e;
-    if ((e = upload_tw_cluster_f64(re, im)) != cudaSuccess) return e;
-    if ((e = upload_tw_glob_f32(re, im)) != cudaSuccess) return e;
-    if ((e = upload_tw_spectra(re, im)) != cudaSuccess) return e;
-    if ((e = upload_tw_energy(re, im)) != cudaSuccess) return e;
-    return upload_tw_glob_f64(re, im);
-}
 
 size_t fused_smem(int P, int prec, int D, int Dpad, bool wbuf, int variant)
 {

@@ -22,8 +22,6 @@
 
 namespace nd {
 
-ND_DEFINE_TWIDDLE_UPLOAD(upload_tw_energy)
-
 // A row of the state as the transforms read it: zero outside the disk.
 template <typename S> struct MaskedRow {
     const S *p;

@@ -19,18 +19,61 @@
 
 namespace nd {
 
-// 32nd roots of unity exp(-2 pi i k / 32), k = 0..31, 24th roots
-// exp(-2 pi i k / 24), k = 0..23 (for the stages of transforms with a factor
-// 3) and 20th roots exp(-2 pi i k / 20), k = 0..19 (factor 5), in the constant
-// bank.  Each translation unit that includes this header owns a copy, filled
-// by its own upload hook (ND_DEFINE_TWIDDLE_UPLOAD).  Indices are compile-time
-// constants in the register DFTs, so each use becomes a constant-bank operand.
-static __constant__ float2 c_w32f[32];
-static __constant__ double2 c_w32d[32];
-static __constant__ float2 c_w24f[24];
-static __constant__ double2 c_w24d[24];
-static __constant__ float2 c_w20f[20];
-static __constant__ double2 c_w20d[20];
+// 32nd roots of unity exp(-2 pi i k / 32), k = 0..31, 24th roots (for the
+// stages of transforms with a factor 3) and 20th roots (factor 5), in the
+// constant bank: each translation unit that includes this header holds a copy.
+// Indices are compile-time constants in the register DFTs, so each use becomes
+// a constant-bank operand.  Initialised here: uploading them took six copies
+// per translation unit on every handle creation.
+#define ND_ROOTS_32(X) \
+    X(1, -0) X(0.98078528040323043, -0.19509032201612825) X(0.92387953251128674, -0.38268343236508978) \
+    X(0.83146961230254524, -0.55557023301960218) X(0.70710678118654757, -0.70710678118654746) \
+    X(0.55557023301960229, -0.83146961230254524) X(0.38268343236508984, -0.92387953251128674) \
+    X(0.19509032201612833, -0.98078528040323043) X(6.123233995736766e-17, -1) \
+    X(-0.19509032201612819, -0.98078528040323043) X(-0.38268343236508973, -0.92387953251128674) \
+    X(-0.55557023301960196, -0.83146961230254546) X(-0.70710678118654746, -0.70710678118654757) \
+    X(-0.83146961230254535, -0.55557023301960218) X(-0.92387953251128674, -0.38268343236508989) \
+    X(-0.98078528040323043, -0.19509032201612861) X(-1, -1.2246467991473532e-16) \
+    X(-0.98078528040323043, 0.19509032201612836) X(-0.92387953251128685, 0.38268343236508967) \
+    X(-0.83146961230254546, 0.55557023301960196) X(-0.70710678118654768, 0.70710678118654746) \
+    X(-0.55557023301960218, 0.83146961230254524) X(-0.38268343236509034, 0.92387953251128652) \
+    X(-0.19509032201612866, 0.98078528040323032) X(-1.8369701987210297e-16, 1) \
+    X(0.1950903220161283, 0.98078528040323043) X(0.38268343236509, 0.92387953251128663) \
+    X(0.55557023301960184, 0.83146961230254546) X(0.70710678118654735, 0.70710678118654768) \
+    X(0.83146961230254524, 0.55557023301960218) X(0.92387953251128652, 0.38268343236509039) \
+    X(0.98078528040323032, 0.19509032201612872)
+#define ND_ROOTS_24(X) \
+    X(1, -0) X(0.96592582628906831, -0.25881904510252074) X(0.86602540378443871, -0.49999999999999994) \
+    X(0.70710678118654757, -0.70710678118654746) X(0.50000000000000011, -0.8660254037844386) \
+    X(0.25881904510252074, -0.96592582628906831) X(6.123233995736766e-17, -1) \
+    X(-0.25881904510252063, -0.96592582628906831) X(-0.49999999999999978, -0.86602540378443871) \
+    X(-0.70710678118654746, -0.70710678118654757) X(-0.86602540378443871, -0.49999999999999994) \
+    X(-0.9659258262890682, -0.25881904510252102) X(-1, -1.2246467991473532e-16) \
+    X(-0.96592582628906831, 0.25881904510252079) X(-0.86602540378443882, 0.49999999999999972) \
+    X(-0.70710678118654791, 0.70710678118654713) X(-0.50000000000000044, 0.86602540378443837) \
+    X(-0.25881904510252063, 0.96592582628906831) X(-1.8369701987210297e-16, 1) \
+    X(0.2588190451025203, 0.96592582628906842) X(0.50000000000000011, 0.8660254037844386) \
+    X(0.70710678118654735, 0.70710678118654768) X(0.86602540378443837, 0.50000000000000044) \
+    X(0.96592582628906809, 0.25881904510252157)
+#define ND_ROOTS_20(X) \
+    X(1, -0) X(0.95105651629515353, -0.3090169943749474) X(0.80901699437494745, -0.58778525229247314) \
+    X(0.58778525229247314, -0.80901699437494745) X(0.30901699437494745, -0.95105651629515353) \
+    X(6.123233995736766e-17, -1) X(-0.30901699437494734, -0.95105651629515364) \
+    X(-0.58778525229247303, -0.80901699437494745) X(-0.80901699437494734, -0.58778525229247325) \
+    X(-0.95105651629515353, -0.30901699437494751) X(-1, -1.2246467991473532e-16) \
+    X(-0.95105651629515375, 0.3090169943749469) X(-0.80901699437494756, 0.58778525229247303) \
+    X(-0.58778525229247325, 0.80901699437494734) X(-0.30901699437494756, 0.95105651629515353) \
+    X(-1.8369701987210297e-16, 1) X(0.30901699437494723, 0.95105651629515364) \
+    X(0.58778525229247292, 0.80901699437494756) X(0.80901699437494734, 0.58778525229247336) \
+    X(0.95105651629515353, 0.30901699437494762)
+#define ND_ROOT_F(re, im) {(float)(re), (float)(im)},
+#define ND_ROOT_D(re, im) {re, im},
+static __constant__ float2 c_w32f[32] = {ND_ROOTS_32(ND_ROOT_F)};
+static __constant__ double2 c_w32d[32] = {ND_ROOTS_32(ND_ROOT_D)};
+static __constant__ float2 c_w24f[24] = {ND_ROOTS_24(ND_ROOT_F)};
+static __constant__ double2 c_w24d[24] = {ND_ROOTS_24(ND_ROOT_D)};
+static __constant__ float2 c_w20f[20] = {ND_ROOTS_20(ND_ROOT_F)};
+static __constant__ double2 c_w20d[20] = {ND_ROOTS_20(ND_ROOT_D)};
 
 template <typename T> __device__ __forceinline__ cplx<T> w32(int k);
 template <> __device__ __forceinline__ cplx<float> w32<float>(int k) { float2 v = c_w32f[k]; return {v.x, v.y}; }
@@ -41,37 +84,6 @@ template <> __device__ __forceinline__ cplx<double> w24<double>(int k) { double2
 template <typename T> __device__ __forceinline__ cplx<T> w20(int k);
 template <> __device__ __forceinline__ cplx<float> w20<float>(int k) { float2 v = c_w20f[k]; return {v.x, v.y}; }
 template <> __device__ __forceinline__ cplx<double> w20<double>(int k) { double2 v = c_w20d[k]; return {v.x, v.y}; }
-
-// re/im: the 32 roots exp(-2 pi i k/32); the 24 and 20 roots are computed here.
-#define ND_DEFINE_TWIDDLE_UPLOAD(name)                                                  \
-    cudaError_t name(const double *re, const double *im)                                \
-    {                                                                                   \
-        float2 f[32];                                                                   \
-        double2 d[32];                                                                  \
-        for (int k = 0; k < 32; ++k) {                                                  \
-            f[k] = make_float2((float)re[k], (float)im[k]);                             \
-            d[k] = make_double2(re[k], im[k]);                                          \
-        }                                                                               \
-        float2 f24[24], f20[20];                                                        \
-        double2 d24[24], d20[20];                                                       \
-        for (int k = 0; k < 24; ++k) {                                                  \
-            const double c = cos(2.0 * M_PI * k / 24.0), s = -sin(2.0 * M_PI * k / 24.0); \
-            f24[k] = make_float2((float)c, (float)s);                                   \
-            d24[k] = make_double2(c, s);                                                \
-        }                                                                               \
-        for (int k = 0; k < 20; ++k) {                                                  \
-            const double c = cos(2.0 * M_PI * k / 20.0), s = -sin(2.0 * M_PI * k / 20.0); \
-            f20[k] = make_float2((float)c, (float)s);                                   \
-            d20[k] = make_double2(c, s);                                                \
-        }                                                                               \
-        cudaError_t e = cudaMemcpyToSymbol(c_w32f, f, sizeof(f));                        \
-        if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_w32d, d, sizeof(d));             \
-        if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_w24f, f24, sizeof(f24));         \
-        if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_w24d, d24, sizeof(d24));         \
-        if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_w20f, f20, sizeof(f20));         \
-        if (e != cudaSuccess) return e;                                                 \
-        return cudaMemcpyToSymbol(c_w20d, d20, sizeof(d20));                            \
-    }
 
 template <int P> struct FFTShape;
 template <> struct FFTShape<16> { static constexpr int G = 4; };

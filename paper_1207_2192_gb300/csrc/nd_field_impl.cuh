@@ -468,6 +468,16 @@ __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
                 // the external field of this step (a scheduled one in the stepping modes)
                 const vec3<T> cx = (MODE == M_RK4 || MODE == M_HEUN) ? step_chext<T>(r, sp, step)
                                                                      : vec3<T>{sp.chext[0], sp.chext[1], sp.chext[2]};
+                if (MODE == M_FIELD) {   // the whole output block, zero outside the disk
+                    for (int i = tid; i < D * Dpad; i += NT) {
+                        const int y = i / Dpad, x = i - y * Dpad;
+                        const long long hi = (long long)y * (2 * RS) + x;
+                        const bool in = x < D && r.mask[y * D + x];
+                        out.st(i, in ? vec3<T>{hr[hi] + cx.x, hr[2 * cs + hi] + cx.y, hr[4 * cs + hi] + cx.z}
+                                     : vec3<T>{T(0), T(0), T(0)});
+                    }
+                    continue;
+                }
                 // over the disk's cells only (a compacted list), so that no warp
                 // spends an iteration on cells outside the disk
                 for (int k = tid; k < r.ncells; k += NT) {

@@ -5,8 +5,6 @@ namespace nd {
 
 static_assert(sizeof(Segment) == sizeof(SegmentHost), "segment layout");
 
-ND_DEFINE_TWIDDLE_UPLOAD(upload_tw_fused_f32)
-
 size_t fused_smem_f32(int P, int D, int Dpad, bool wbuf, int variant)
 {
     const int nt = fused_nt(P, variant);

@@ -5,8 +5,6 @@
 
 namespace nd {
 
-ND_DEFINE_TWIDDLE_UPLOAD(upload_tw_glob_f32)
-
 cudaError_t launch_global_f32(int P, const LaunchArgs &a, int maxD)
 {
     switch (P) {

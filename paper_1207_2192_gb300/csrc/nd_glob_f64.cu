@@ -5,8 +5,6 @@
 
 namespace nd {
 
-ND_DEFINE_TWIDDLE_UPLOAD(upload_tw_glob_f64)
-
 cudaError_t launch_global_f64(int P, const LaunchArgs &a, int maxD)
 {
     switch (P) {

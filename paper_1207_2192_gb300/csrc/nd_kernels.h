@@ -60,7 +60,6 @@ struct SegmentHost {                 // mirrors Segment in nd_field_impl.cuh
     long long step_begin, nsteps;
 };
 
-cudaError_t upload_twiddle_constants(const double *re, const double *im);
 size_t fused_smem(int P, int prec, int D, int Dpad, bool wbuf = false, int variant = 0);
 int fused_blocks_per_sm(int P, int prec, int mode, size_t smem, int variant = 0);
 int fused_variant_threads(int P, int variant);   // 0 if the variant does not exist
@@ -112,9 +111,9 @@ cudaError_t launch_init_vortex(int prec, const Replica *reps, const int *work, i
                                const double *X0_cells /*[nrep][2], units of a, device*/, const int *pol_chi,
                                double lambda_over_a, cudaStream_t st);
 constexpr int kCoreMaxBlocks = 128;   // plaquette-scan CTAs per replica (candidates buffer: [B][128][2] doubles)
-int core_scan_blocks(int D);
 cudaError_t launch_vortex_core(int prec, const Replica *reps, const int *work, int nwork, int maxD, const void *y,
-                               double rc2, double *part, double *out /*[nrep][4]: xc, yc (units of a), status, cell*/,
+                               double rc2, double *part, unsigned *done /*[nrep], zero before the first call*/,
+                               double *out /*[nrep][4]: xc, yc (units of a), status, cell*/,
                                cudaStream_t st);
 cudaError_t launch_stats_update(const int *work, int nwork, const double *core, const double *a_of_rep, StatsAcc *st,
                                 unsigned long long *hr, unsigned long long *hv, int rb, int vb, double r_max,

@@ -156,10 +156,6 @@ extern "C" int nd_step_heun_noalloc(const nd_disk_desc *disk, int n_replicas, fl
         void *p = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&p, g_nd_noalloc_scratch);
         if (e != cudaSuccess) return fail(ND_ERR_CUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
-        double re[32], im[32];
-        for (int k = 0; k < 32; ++k) { re[k] = cos(2.0 * M_PI * k / 32.0); im[k] = -sin(2.0 * M_PI * k / 32.0); }
-        e = upload_twiddle_constants(re, im);
-        if (e != cudaSuccess) return fail(ND_ERR_CUDA, std::string("twiddle constants: ") + cudaGetErrorString(e));
         S.base = static_cast<unsigned char *>(p);
         S.ready = true;
     }

@@ -7,8 +7,6 @@
 
 namespace nd {
 
-ND_DEFINE_TWIDDLE_UPLOAD(upload_tw_spectra)
-
 // <m> of every replica of a size class (double sums over the disk cells)
 // written at sample index *count of its series [replica][cap][3]; samples
 // beyond cap are dropped (the counter keeps counting).
@@ -16,37 +14,9 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_series_append(const Replica *reps, const int *work, const T *ybase,
                                                        double *series, const unsigned long long *count, int cap)
 {
-    __shared__ double sx[4][8];
     const int ridx = work[blockIdx.x];
-    const Replica &r = reps[ridx];
-    const int D = r.D, tid = threadIdx.x;
-    const long long cs = (long long)D * r.Dpad;
-    const T *y = ybase + r.state_off;
-    double a0 = 0, a1 = 0, a2 = 0, n = 0;
-    for (int cell = tid; cell < D * D; cell += 256) {
-        if (!r.mask[cell]) continue;
-        const int j = cell / D, i = cell - j * D;
-        const long long si = (long long)j * r.Dpad + i;
-        a0 += (double)y[si]; a1 += (double)y[cs + si]; a2 += (double)y[2 * cs + si]; n += 1.0;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        a0 += __shfl_xor_sync(0xffffffffu, a0, o);
-        a1 += __shfl_xor_sync(0xffffffffu, a1, o);
-        a2 += __shfl_xor_sync(0xffffffffu, a2, o);
-        n += __shfl_xor_sync(0xffffffffu, n, o);
-    }
-    if ((tid & 31) == 0) { sx[0][tid >> 5] = a0; sx[1][tid >> 5] = a1; sx[2][tid >> 5] = a2; sx[3][tid >> 5] = n; }
-    __syncthreads();
-    if (tid == 0) {
-        const unsigned long long idx = *count;
-        if (idx < (unsigned long long)cap) {
-            double s[4] = {0, 0, 0, 0};
-            for (int w = 0; w < 8; ++w)
-                for (int c = 0; c < 4; ++c) s[c] += sx[c][w];
-            double *o = series + ((size_t)ridx * cap + idx) * 3;
-            for (int c = 0; c < 3; ++c) o[c] = s[c] / s[3];
-        }
-    }
+    const unsigned long long idx = *count;
+    block_mean<T>(reps[ridx], ybase, idx < (unsigned long long)cap ? series + ((size_t)ridx * cap + idx) * 3 : nullptr);
 }
 
 __global__ void k_series_advance(unsigned long long *count)
