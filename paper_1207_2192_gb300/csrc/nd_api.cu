@@ -518,8 +518,9 @@ static int run_mode(nd_handle *h, int mode, void *y, void *out, long long nsteps
             if (!a.ms || !a.spec) return fail(ND_ERR_ARG, "global-path buffers are not allocated");
             ND_CUDA(launch_global(c.P, prec, a, c.maxD));
         }
-        // a stepped state with a non-finite cell sets the NaN bit of the status word
-        if (mode == M_RK4 || mode == M_HEUN)
+        // a stepped state with a non-finite cell sets the NaN bit of the status
+        // word (the cluster kernel looks at its cells itself)
+        if (stepping && !cluster_nc)
             ND_CUDA(launch_check_finite(prec, a.reps, c.work_d, (int)c.reps.size(), c.maxD, y, h->status_d, st));
         if (concurrent && ci > 0) ND_CUDA(cudaEventRecord(h->join_ev[ci - 1], st));
     }

@@ -1,6 +1,6 @@
 // nd_aux.cu -- once-per-geometry spectral kernel build and the small
 // per-replica kernels: analytic vortex profile, vortex-core estimator, <m>,
-// finiteness check.
+// finiteness scan.
 #include <math.h>
 
 #include "nd_common.cuh"

@@ -732,13 +732,17 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
         if (RELAX && conv_s) break;
     }
     // the final state of the CTA's cells back to the caller's buffer
+    bool bad = false;
     if (MODE != M_FIELD)
     for (int k = c0 + tid; k < c1; k += NT) {
         const int cell = __ldg(r.cells + k);
         const int y = cell / D, x = cell - y * D;
         const long long mi = (long long)(y - ylo) * Dpad + x;
-        yg.st((long long)y * Dpad + x, RELAX ? ms.ld(mi) : ynv.ld(mi));
+        const vec3<T> v = RELAX ? ms.ld(mi) : ynv.ld(mi);
+        yg.st((long long)y * Dpad + x, v);
+        bad |= !finite3(v);
     }
+    if (MODE == M_RK4 || MODE == M_HEUN) flag_nan(bad, status);
     if (RELAX && rank == 0 && tid == 0) {
         RelaxIO *io = rx.rio + seg.rep;
         const int iters = __ldcg(&io->iters) + (int)n;

@@ -59,6 +59,20 @@ template <typename T> __device__ __forceinline__ vec3<T> heun_dm(vec3<T> m, vec3
 // the launch attribute this is a no-op.
 __device__ __forceinline__ void wait_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// A stepping call whose final state has a non-finite cell sets the NaN bit of
+// the status word.  The cluster kernel looks at the cells it writes last; the
+// others are followed by a scan of its own (k_check_finite, 5-10 us): the same
+// look took registers from k_fused's column pass (256 replicas, 50 Heun steps:
+// 3.44 -> 3.55 ms) and from the global epilogue (8 of D = 500: 5.05 -> 5.10 ms).
+template <typename T> __device__ __forceinline__ bool finite3(vec3<T> v)
+{
+    return isfinite(v.x) && isfinite(v.y) && isfinite(v.z);
+}
+__device__ __forceinline__ void flag_nan(bool bad, unsigned *status)
+{
+    if (bad && status) atomicOr(status, ND_DEV_NAN);
+}
+
 template <typename T> struct V3Ptr {
     T *p;
     long long s;  // component stride
