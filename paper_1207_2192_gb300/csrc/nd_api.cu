@@ -326,7 +326,7 @@ struct EvalTime { int P; float one, c8, c16; };
 static const EvalTime kEval32[] = {{16, 3.6f, 0, 0},        {32, 5.1f, 4.6f, 4.4f}, {64, 7.0f, 4.0f, 4.0f},
                                    {128, 20.5f, 6.1f, 5.3f}, {192, 30.f, 0, 10.2f},  {256, 28.f, 0, 11.5f}};
 static const EvalTime kEval64[] = {{16, 23.8f, 16.9f, 0}, {32, 50.f, 36.f, 33.f}, {64, 130.f, 36.f, 36.f},
-                                   {128, 282.f, 94.f, 70.f}};
+                                   {128, 140.f, 94.f, 70.f}};
 
 // The plan that the default (-1) stands for.  Few replicas leave most SMs
 // idle with one CTA each, so they take a cluster plan while its rounds, with

@@ -183,6 +183,16 @@ template <int MODE> struct ModeStages { static constexpr int n = 1; };
 template <> struct ModeStages<M_RK4> { static constexpr int n = 4; };
 template <> struct ModeStages<M_HEUN> { static constexpr int n = 2; };
 
+// Threads per CTA of the passes whose work divides by warps.  FP64 issues one
+// warp instruction per sub-partition in 64-76 cycles, so its CTAs are small: one
+// or two warps land on every sub-partition of the chip instead of eight on a few
+// SMs (FP64 relaxation of R = 30/65/100 nm, two replicas each: 194 -> 142 ms,
+// against rows of 34 us, a reduction of 19 and an update of 11 with 256 threads;
+// one FP64 disk of R = 50 nm on this path: 282 -> 137 us per evaluation).
+template <typename T> struct GlobNT { static constexpr int v = sizeof(T) == 8 ? 32 : 256; };
+template <typename T> struct CellNT { static constexpr int v = sizeof(T) == 8 ? 64 : 256; };
+template <typename T> struct RedNT { static constexpr int v = sizeof(T) == 8 ? 128 : 256; };   // partial sums
+
 // ------------------------------------------------------------ fused path
 
 template <int P, typename T>
@@ -773,7 +783,7 @@ __global__ void __launch_bounds__(ColTile<P, T>::NT, ColTile<P, T>::MINB)
 
 // Elementwise epilogue of the global path.  grid = (cell blocks, replicas).
 template <int P, typename T, int MODE>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(CellNT<T>::v)
     k_g_epi(const Replica *__restrict__ reps, const int *__restrict__ work, T *__restrict__ msbase,
             T *__restrict__ ybase, T *__restrict__ accbase, T *__restrict__ outbase,
             const cplx<T> *__restrict__ specbase, int stage, unsigned long long step)
@@ -783,7 +793,7 @@ __global__ void __launch_bounds__(256)
     const Replica r = reps[ridx];
     const int D = r.D, DD = D * D;
     const long long ms_s = (long long)D * r.Dpad, cs = (long long)D * RS;
-    const int cell = blockIdx.x * 256 + threadIdx.x;
+    const int cell = blockIdx.x * CellNT<T>::v + threadIdx.x;
     if (cell < DD && r.mask[cell]) {
         const int y = cell / D, x = cell - y * D;
         const long long si = (long long)y * r.Dpad + x;
@@ -833,7 +843,7 @@ template <> __device__ __forceinline__ void st_quad<double>(double *p, const Qua
 // aligned state buffers (rows and replica blocks are multiples of 4
 // elements; the spectrum rows start on 32-byte sectors).
 template <int P, typename T, int MODE>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(CellNT<T>::v)
     k_g_epi_quad(const Replica *__restrict__ reps, const int *__restrict__ work, T *__restrict__ msbase,
                  T *__restrict__ ybase, T *__restrict__ accbase, const cplx<T> *__restrict__ specbase, int stage,
                  unsigned long long step)
@@ -843,7 +853,7 @@ __global__ void __launch_bounds__(256)
     wait_prior_grid();
     const Replica &r = reps[work[blockIdx.y]];
     const int D = r.D, Dpad = r.Dpad, qpr = Dpad / 4;
-    const int qd = blockIdx.x * 256 + threadIdx.x;
+    const int qd = blockIdx.x * CellNT<T>::v + threadIdx.x;
     if (qd >= D * qpr) return;
     const int y = qd / qpr, x0 = 4 * (qd - y * qpr);
     const long long ms_s = (long long)D * Dpad, cs2 = 2LL * D * RS;   // component strides (state, field rows)
@@ -929,13 +939,13 @@ __global__ void k_g_load_stage(const Replica *__restrict__ reps, const int *__re
 //   k_g_relax_update  the damped alignment with the new multipliers.
 // Replicas that have converged (status 0) are left untouched.
 template <int P, typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(RedNT<T>::v)
     k_g_relax_reduce(const Replica *__restrict__ reps, const int *__restrict__ work, const T *__restrict__ msbase,
                      const cplx<T> *__restrict__ specbase, const RelaxIO *__restrict__ rio, double rc2_d,
                      double eta_d, double *__restrict__ part)
 {
     constexpr int RS = SpecGeom<P>::RS;
-    __shared__ RelaxAcc<T> racc[8];
+    __shared__ RelaxAcc<T> racc[RedNT<T>::v / 32];
     const int ridx = work[blockIdx.y], tid = threadIdx.x;
     if (rio[ridx].status == 0) return;   // CTA-uniform
     const Replica &r = reps[ridx];
@@ -947,7 +957,7 @@ __global__ void __launch_bounds__(256)
     const T eta = (T)eta_d, rc2 = (T)rc2_d;
     const StepParams<T> sp = step_params<T>(r);
     RelaxAcc<T> a = {T(0), T(0), T(0), T(0), T(0), T(0)};
-    for (int cell = blockIdx.x * 256 + tid; cell < DD; cell += kRelaxBlocks * 256) {
+    for (int cell = blockIdx.x * RedNT<T>::v + tid; cell < DD; cell += kRelaxBlocks * RedNT<T>::v) {
         if (!r.mask[cell]) continue;
         const int y = cell / D, x = cell - y * D;
         const long long si = (long long)y * r.Dpad + x, hi = (long long)y * (2 * RS) + x;
@@ -961,7 +971,7 @@ __global__ void __launch_bounds__(256)
     __syncthreads();
     if (tid == 0) {
         RelaxAcc<T> t = racc[0];
-        for (int w = 1; w < 8; ++w) {
+        for (int w = 1; w < RedNT<T>::v / 32; ++w) {
             t.C0 += racc[w].C0; t.C1 += racc[w].C1; t.J00 += racc[w].J00; t.J01 += racc[w].J01;
             t.J11 += racc[w].J11; t.res = max(t.res, racc[w].res);
         }
@@ -1004,7 +1014,7 @@ static __global__ void __launch_bounds__(128) k_g_relax_newton(const int *__rest
 }
 
 template <int P, typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(CellNT<T>::v)
     k_g_relax_update(const Replica *__restrict__ reps, const int *__restrict__ work, T *__restrict__ msbase,
                      const cplx<T> *__restrict__ specbase, const RelaxIO *__restrict__ rio, double rc2_d, double eta_d)
 {
@@ -1013,7 +1023,7 @@ __global__ void __launch_bounds__(256)
     if (rio[ridx].status == 0) return;
     const Replica &r = reps[ridx];
     const int D = r.D, DD = D * D;
-    const int cell = blockIdx.x * 256 + threadIdx.x;
+    const int cell = blockIdx.x * CellNT<T>::v + threadIdx.x;
     if (cell >= DD || !r.mask[cell]) return;
     const long long ms_s = (long long)D * r.Dpad, cs = (long long)D * RS;
     const T *hr = reinterpret_cast<const T *>(specbase + r.spec_off);
@@ -1033,12 +1043,12 @@ __global__ void __launch_bounds__(256)
 // the state layout), read in place of the spectrum rows.  Used by
 // nd_relax_sweep_grad.
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(RedNT<T>::v)
     k_relax_grad_reduce(const Replica *__restrict__ reps, const int *__restrict__ work, const T *__restrict__ mbase,
                         const T *__restrict__ gbase, const double *__restrict__ gscale,
                         const RelaxIO *__restrict__ rio, double rc2_d, double eta_d, double *__restrict__ part)
 {
-    __shared__ RelaxAcc<T> racc[8];
+    __shared__ RelaxAcc<T> racc[RedNT<T>::v / 32];
     const int ridx = work[blockIdx.y], tid = threadIdx.x;
     if (rio[ridx].status == 0) return;   // CTA-uniform
     const Replica &r = reps[ridx];
@@ -1048,7 +1058,7 @@ __global__ void __launch_bounds__(256)
     const T relX = (T)rio[ridx].X[0], relY = (T)rio[ridx].X[1], l0 = (T)rio[ridx].lam[0], l1 = (T)rio[ridx].lam[1];
     const T eta = (T)eta_d, rc2 = (T)rc2_d, sc = (T)gscale[ridx];
     RelaxAcc<T> a = {T(0), T(0), T(0), T(0), T(0), T(0)};
-    for (int cell = blockIdx.x * 256 + tid; cell < DD; cell += kRelaxBlocks * 256) {
+    for (int cell = blockIdx.x * RedNT<T>::v + tid; cell < DD; cell += kRelaxBlocks * RedNT<T>::v) {
         if (!r.mask[cell]) continue;
         const int y = cell / D, x = cell - y * D;
         const long long si = (long long)y * r.Dpad + x;
@@ -1062,7 +1072,7 @@ __global__ void __launch_bounds__(256)
     __syncthreads();
     if (tid == 0) {
         RelaxAcc<T> t = racc[0];
-        for (int w = 1; w < 8; ++w) {
+        for (int w = 1; w < RedNT<T>::v / 32; ++w) {
             t.C0 += racc[w].C0; t.C1 += racc[w].C1; t.J00 += racc[w].J00; t.J01 += racc[w].J01;
             t.J11 += racc[w].J11; t.res = max(t.res, racc[w].res);
         }
@@ -1072,7 +1082,7 @@ __global__ void __launch_bounds__(256)
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(CellNT<T>::v)
     k_relax_grad_update(const Replica *__restrict__ reps, const int *__restrict__ work, T *__restrict__ mbase,
                         const T *__restrict__ gbase, const double *__restrict__ gscale,
                         const RelaxIO *__restrict__ rio, double rc2_d, double eta_d)
@@ -1081,7 +1091,7 @@ __global__ void __launch_bounds__(256)
     if (rio[ridx].status == 0) return;
     const Replica &r = reps[ridx];
     const int D = r.D, DD = D * D;
-    const int cell = blockIdx.x * 256 + threadIdx.x;
+    const int cell = blockIdx.x * CellNT<T>::v + threadIdx.x;
     if (cell >= DD || !r.mask[cell]) return;
     const long long ms_s = (long long)D * r.Dpad;
     V3Ptr<T> ms{mbase + r.state_off, ms_s};
@@ -1100,11 +1110,12 @@ __global__ void __launch_bounds__(256)
 template <typename T>
 static cudaError_t launch_relax_grad_t(const LaunchArgs &a, int maxD, const void *grad, const double *gscale)
 {
-    const dim3 gp(kRelaxBlocks, a.nwork), gu((maxD * maxD + 255) / 256, a.nwork);
-    k_relax_grad_reduce<T><<<gp, 256, 0, a.stream>>>(a.reps, a.work, (const T *)a.y, (const T *)grad, gscale, a.rio,
+    constexpr int NC = CellNT<T>::v, NR = RedNT<T>::v;
+    const dim3 gp(kRelaxBlocks, a.nwork), gu((maxD * maxD + NC - 1) / NC, a.nwork);
+    k_relax_grad_reduce<T><<<gp, NR, 0, a.stream>>>(a.reps, a.work, (const T *)a.y, (const T *)grad, gscale, a.rio,
                                                      a.rc2, a.eta, a.part);
     k_g_relax_newton<<<(a.nwork + 3) / 4, 128, 0, a.stream>>>(a.work, a.nwork, a.rio, a.part, a.tol, 0);
-    k_relax_grad_update<T><<<gu, 256, 0, a.stream>>>(a.reps, a.work, (T *)a.y, (const T *)grad, gscale, a.rio, a.rc2,
+    k_relax_grad_update<T><<<gu, NC, 0, a.stream>>>(a.reps, a.work, (T *)a.y, (const T *)grad, gscale, a.rio, a.rc2,
                                                      a.eta);
     return cudaGetLastError();
 }
@@ -1138,7 +1149,6 @@ inline int fused_nt(int P, int variant)
     default: return 0;
     }
 }
-template <int P> struct GlobNT { static constexpr int v = 256; };
 // The tiled column pass runs above P = 128 (rows of the global spectrum start
 // on 32-byte sectors there).
 template <int P> struct GlobTiled { static constexpr bool v = P > 128; };
@@ -1250,7 +1260,7 @@ static cudaError_t launch_fused_p(const LaunchArgs &a)
 template <int P, typename T, int MODE>
 static void launch_g_epi(const LaunchArgs &a, dim3 ge, int stage, unsigned long long step)
 {
-    k_g_epi<P, T, MODE><<<ge, 256, 0, a.stream>>>(a.reps, a.work, (T *)a.ms, (T *)a.y, (T *)a.acc, (T *)a.out,
+    k_g_epi<P, T, MODE><<<ge, CellNT<T>::v, 0, a.stream>>>(a.reps, a.work, (T *)a.ms, (T *)a.y, (T *)a.acc, (T *)a.out,
                                                    (const cplx<T> *)a.spec, stage, step);
 }
 
@@ -1280,10 +1290,11 @@ static void launch_g_epi_step(const LaunchArgs &a, int maxD, int stage, unsigned
                         reinterpret_cast<uintptr_t>(a.acc)) & 15) == 0;
     if (quad) {
         const int maxq = maxD * ((maxD + 3) / 4);
-        launch_pdl(k_g_epi_quad<P, T, MODE>, dim3((maxq + 255) / 256, a.nwork), dim3(256), 0, a.stream, a.reps,
+        constexpr int NC = CellNT<T>::v;
+        launch_pdl(k_g_epi_quad<P, T, MODE>, dim3((maxq + NC - 1) / NC, a.nwork), dim3(NC), 0, a.stream, a.reps,
                    a.work, (T *)a.ms, (T *)a.y, (T *)a.acc, (const cplx<T> *)a.spec, stage, step);
     } else {
-        launch_g_epi<P, T, MODE>(a, dim3((maxD * maxD + 255) / 256, a.nwork), stage, step);
+        launch_g_epi<P, T, MODE>(a, dim3((maxD * maxD + CellNT<T>::v - 1) / CellNT<T>::v, a.nwork), stage, step);
     }
 }
 
@@ -1293,7 +1304,7 @@ static void launch_g_epi_step(const LaunchArgs &a, int maxD, int stage, unsigned
 template <int P, typename T>
 static void glob_rows(const LaunchArgs &a, int maxD, int inverse)
 {
-    constexpr int NT = GlobNT<P>::v, NGRP = groups_per_block<P, NT>();
+    constexpr int NT = GlobNT<T>::v, NGRP = groups_per_block<P, NT>();
     const int nrow = row_pass_tasks<P>(maxD);
     dim3 gr((nrow + NGRP - 1) / NGRP, a.nwork);
     launch_pdl(k_g_rows<P, T, NT>, gr, dim3(NT), glob_smem_bytes<P, T, NT>(), a.stream, a.reps, a.work,
@@ -1303,7 +1314,7 @@ static void glob_rows(const LaunchArgs &a, int maxD, int inverse)
 template <int P, typename T>
 static void glob_cols(const LaunchArgs &a, int maxD)
 {
-    constexpr int NT = GlobNT<P>::v, NGRP = groups_per_block<P, NT>();
+    constexpr int NT = GlobNT<T>::v, NGRP = groups_per_block<P, NT>();
     if constexpr (GlobTiled<P>::v) {
         using CT = ColTile<P, T>;
         const int ntask = a.nwork * (CT::NXY + CT::NZ);
@@ -1330,7 +1341,7 @@ template <int P, typename T>
 static cudaError_t glob_eval(const LaunchArgs &a, int maxD, int stage, int mode, unsigned long long step)
 {
     glob_field_passes<P, T>(a, maxD);
-    dim3 ge((maxD * maxD + 255) / 256, a.nwork);
+    dim3 ge((maxD * maxD + CellNT<T>::v - 1) / CellNT<T>::v, a.nwork);
     switch (mode) {
     case M_FIELD: launch_g_epi<P, T, M_FIELD>(a, ge, stage, step); break;
     case M_RK4: launch_g_epi_step<P, T, M_RK4>(a, maxD, stage, step); break;
@@ -1343,7 +1354,7 @@ static cudaError_t glob_eval(const LaunchArgs &a, int maxD, int stage, int mode,
 template <int P, typename T>
 static cudaError_t launch_global_p(const LaunchArgs &a, int maxD)
 {
-    constexpr int NT = GlobNT<P>::v;
+    constexpr int NT = GlobNT<T>::v;
     const int sm = (int)glob_smem_bytes<P, T, NT>();
     cudaError_t e0 = cudaFuncSetAttribute(k_g_rows<P, T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if constexpr (!GlobTiled<P>::v) {
@@ -1362,14 +1373,15 @@ static cudaError_t launch_global_p(const LaunchArgs &a, int maxD)
     if (e != cudaSuccess) return e;
     if (a.mode == M_RELAX) {
         if (!a.rio || !a.part || !a.rio_host || !a.work_host) return cudaErrorInvalidValue;
-        const dim3 gp(kRelaxBlocks, a.nwork), gu((maxD * maxD + 255) / 256, a.nwork);
+        constexpr int NC = CellNT<T>::v;
+        const dim3 gp(kRelaxBlocks, a.nwork), gu((maxD * maxD + NC - 1) / NC, a.nwork);
         constexpr int kCheck = 32;   // iterations between host checks for convergence of every replica
         for (int it = 0; it < a.max_iter; ++it) {
             glob_field_passes<P, T>(a, maxD);
-            k_g_relax_reduce<P, T><<<gp, 256, 0, a.stream>>>(a.reps, a.work, (const T *)a.ms, (const cplx<T> *)a.spec,
+            k_g_relax_reduce<P, T><<<gp, RedNT<T>::v, 0, a.stream>>>(a.reps, a.work, (const T *)a.ms, (const cplx<T> *)a.spec,
                                                              a.rio, a.rc2, a.eta, a.part);
             k_g_relax_newton<<<(a.nwork + 3) / 4, 128, 0, a.stream>>>(a.work, a.nwork, a.rio, a.part, a.tol, it);
-            k_g_relax_update<P, T><<<gu, 256, 0, a.stream>>>(a.reps, a.work, (T *)a.ms, (const cplx<T> *)a.spec, a.rio,
+            k_g_relax_update<P, T><<<gu, NC, 0, a.stream>>>(a.reps, a.work, (T *)a.ms, (const cplx<T> *)a.spec, a.rio,
                                                              a.rc2, a.eta);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             if ((it + 1) % kCheck == 0 || it + 1 == a.max_iter) {
