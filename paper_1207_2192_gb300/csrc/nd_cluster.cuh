@@ -78,6 +78,7 @@ __host__ __device__ __forceinline__ size_t cluster_smem_bytes(int D, int Dpad, b
 // component after the forward transform of c0 + i c_{P/2}: separation with
 // the mirror element, the diagonal kernel entries s0 (kx = 0) and s1
 // (kx = P/2) from shared memory, and re-packing for the inverse transform.
+// (The entries come halved: they hold the separation's factor 1/2.)
 template <int P, typename T>
 __device__ __forceinline__ void cluster_packed_scale(cplx<T> *v, const T *s0t, const T *s1t, int t, cplx<T> *scr,
                                                      unsigned gmask)
@@ -91,9 +92,8 @@ __device__ __forceinline__ void cluster_packed_scale(cplx<T> *v, const T *s0t, c
         const int ky = t + G * o;
         const int kyr = ky <= P / 2 ? ky : P - ky;
         const cplx<T> w = mirror_get<P>(scr, ky);
-        const T h = T(0.5);
-        cplx<T> F0 = {h * (v[o].x + w.x), h * (v[o].y - w.y)};
-        cplx<T> F1 = {h * (v[o].y + w.y), -h * (v[o].x - w.x)};
+        const cplx<T> F0 = {v[o].x + w.x, v[o].y - w.y};
+        const cplx<T> F1 = {v[o].y + w.y, w.x - v[o].x};
         const T s0 = s0t[kyr], s1 = s1t[kyr];
         v[o] = {fm(F0.x, s0, -(F1.y * s1)), fm(F0.y, s0, F1.x * s1)};   // s0 F0 + i s1 F1
     }
@@ -316,12 +316,16 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
         for (int i = tid; i < 4 * NTAB * KH; i += NT) {
             const int c = i / (NTAB * KH), rem = i - c * (NTAB * KH), j = rem / KH, ky = rem - j * KH;
             const int kx = j < SPC ? rank * SPC + j : P / 2;
+            // with the factors 1/2 of the separations of row pairs and of the
+            // packed columns: powers of two, so the rounding is that of the
+            // other kernels, which apply them where they separate
+            const T half = (HalfRows<P>::on ? T(1) : T(0.5)) * (kx == 0 || kx == P / 2 ? T(0.5) : T(1));
             if constexpr (RELAX) {   // without the exchange
                 const double g = __ldg(r.Ghat64 + (long long)(4 + c) * KK + kx * KH + ky);
                 const double ex = c == 2 ? 0.0 : 2.0 * (__ldg(rx.twP64 + 2 * kx) + __ldg(rx.twP64 + 2 * ky));
-                gtab[i] = (T)fm(-ex, 1.0 / ((double)P * P), g);
+                gtab[i] = half * (T)fm(-ex, 1.0 / ((double)P * P), g);
             } else {
-                gtab[i] = __ldg(Gc + (long long)c * KK + kx * KH + ky);
+                gtab[i] = half * __ldg(Gc + (long long)c * KK + kx * KH + ky);
             }
         }
     }
@@ -444,9 +448,9 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
                         const int k = gid.t + G * o;
                         if (k <= P / 2) {
                             const cplx<T> w = mirror_get<P>(scr, k);
-                            const T h = T(0.5);
-                            const cplx<T> A = {h * (v[o].x + w.x), h * (v[o].y - w.y)};
-                            const cplx<T> B = {h * (v[o].y + w.y), -h * (v[o].x - w.x)};
+                            // twice the spectra (the kernel's entries are halved)
+                            const cplx<T> A = {v[o].x + w.x, v[o].y - w.y};
+                            const cplx<T> B = {v[o].y + w.y, w.x - v[o].x};
                             if (k == 0) {
                                 rA0 = A.x;
                                 rB0 = B.x;
