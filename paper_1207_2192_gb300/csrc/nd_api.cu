@@ -79,6 +79,8 @@ struct SizeClass {
     int *seg_off_d = nullptr;
     int seg_mode = -1, seg_ncta = 0;
     long long seg_nsteps = -1;
+    bool seg_captured = false;            // a graph replays with the cached schedule
+    std::vector<void *> seg_kept;         // schedules of graphs, kept until the handle goes
     int *cflags_d = nullptr;   // cluster schedules: hand-over flags of the replicas, the ticket counter, the count of finished ones
     // resident clusters per (RK4 / Heun, 8 / 16 CTAs) and the plan the default
     // stands for per method: -1 not yet looked up
@@ -328,6 +330,13 @@ static const EvalTime kEval32[] = {{16, 3.6f, 0, 0},        {32, 5.1f, 4.6f, 4.4
 static const EvalTime kEval64[] = {{16, 23.8f, 16.9f, 0}, {32, 50.f, 36.f, 33.f}, {64, 130.f, 36.f, 36.f},
                                    {128, 140.f, 94.f, 70.f}};
 
+static const EvalTime *eval_time(int prec, int P)
+{
+    if (prec == ND_PREC_FP64) { for (const auto &t : kEval64) if (t.P == P) return &t; }
+    else                      { for (const auto &t : kEval32) if (t.P == P) return &t; }
+    return nullptr;
+}
+
 // The plan that the default (-1) stands for.  Few replicas leave most SMs
 // idle with one CTA each, so they take a cluster plan while its rounds, with
 // the replicas time-sliced over the clusters the GPU holds (about 15 of 8
@@ -347,9 +356,7 @@ static int default_plan(const nd_handle *h, const SizeClass &c0, int mode)
     int sms = 0;
     for (const auto &c : h->classes) {
         const int plain = c.fused_main ? 0 : kPlanGlobal, B = (int)c.reps.size();
-        const EvalTime *e = nullptr;
-        if (prec == ND_PREC_FP64) { for (const auto &t : kEval64) if (t.P == c.P) e = &t; }
-        else                      { for (const auto &t : kEval32) if (t.P == c.P) e = &t; }
+        const EvalTime *e = eval_time(prec, c.P);
         int best = plain, best_nc = 0;
         float t = e ? e->one : 0.f;
         for (int nc : {8, 16}) {
@@ -386,19 +393,40 @@ static int relax_cluster_nc(const nd_handle *h, const SizeClass &c)
     return plan_cluster_nc(c.alone_plan[1]);
 }
 
-// The time-sliced schedule of a class's replicas over nslots CTAs or clusters,
-// cached per (mode, n_steps, slots).
-static int class_segments(SizeClass &c, int mode, long long nsteps, int nslots)
+static bool capturing(cudaStream_t st)
 {
-    if (c.seg_mode == mode && c.seg_nsteps == nsteps && c.seg_ncta == nslots) return ND_OK;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
+}
+
+// The time-sliced schedule of a class's replicas over nslots CTAs or clusters,
+// cached per (mode, n_steps, slots).  One that a graph was captured with stays
+// allocated for its replays when another takes its place.
+static bool segments_cached(const SizeClass &c, int mode, long long nsteps, int nslots)
+{
+    return c.seg_mode == mode && c.seg_nsteps == nsteps && c.seg_ncta == nslots;
+}
+static int class_segments(SizeClass &c, int mode, long long nsteps, int nslots, cudaStream_t st)
+{
+    if (segments_cached(c, mode, nsteps, nslots)) {
+        c.seg_captured |= capturing(st);
+        return ND_OK;
+    }
     std::vector<SegmentHost> segs;
     std::vector<int> off;
     build_segments((int)c.reps.size(), nsteps, nslots, segs, off);
     for (auto &g : segs) g.rep = c.reps[g.rep];   // segments refer to positions in c.reps
-    cudaFree(c.segs_d);
-    cudaFree(c.seg_off_d);
+    if (c.seg_captured) {
+        c.seg_kept.push_back(c.segs_d);
+        c.seg_kept.push_back(c.seg_off_d);
+    } else {
+        cudaFree(c.segs_d);
+        cudaFree(c.seg_off_d);
+    }
     c.segs_d = nullptr;
     c.seg_off_d = nullptr;
+    c.seg_mode = -1;
+    c.seg_captured = false;
     ND_CUDA(cudaMalloc(&c.segs_d, sizeof(SegmentHost) * segs.size()));
     ND_CUDA(cudaMalloc(&c.seg_off_d, sizeof(int) * off.size()));
     ND_CUDA(cudaMemcpy(c.segs_d, segs.data(), sizeof(SegmentHost) * segs.size(), cudaMemcpyHostToDevice));
@@ -409,14 +437,17 @@ static int class_segments(SizeClass &c, int mode, long long nsteps, int nslots)
     return ND_OK;
 }
 
-// CTAs per replica of a field call: clusters where all replicas of the class
-// hold one at once.
+// CTAs per replica of a field call: clusters where their waves (whole replicas,
+// one evaluation each) take less than one evaluation of the one-CTA kernel.
 static int field_cluster_nc(const nd_handle *h, const SizeClass &c)
 {
     default_plan(h, c, M_RK4);
     const int nc = plan_cluster_nc(c.alone_plan[0]);
     const int prec = h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32;
-    return nc && (int)c.reps.size() <= cluster_slots(h, c, prec, false, nc) ? nc : 0;
+    if (!nc) return 0;
+    const EvalTime *e = eval_time(prec, c.P);
+    const int slots = cluster_slots(h, c, prec, false, nc), waves = ((int)c.reps.size() + slots - 1) / slots;
+    return waves * (nc == 8 ? e->c8 : e->c16) < e->one ? nc : 0;
 }
 
 // Run one mode over all replicas in the handle's precision.
@@ -473,10 +504,13 @@ static int run_mode(nd_handle *h, int mode, void *y, void *out, long long nsteps
             a.status = h->status_d;
             const int slots = cluster_slots(h, c, prec, mode == M_HEUN, cluster_nc);
             const int Bc = (int)c.reps.size(), B = (int)h->rep_disk.size();
-            if (Bc > slots && nsteps >= 2) {
+            if (Bc > slots && nsteps >= 2 &&
+                ((segments_cached(c, mode, nsteps, slots) && c.cflags_d) || !capturing(st))) {
                 // more replicas than resident clusters: every cluster steps for
-                // the same time instead of in waves of whole replicas
-                if (int rc = class_segments(c, mode, nsteps, slots)) return rc;
+                // the same time instead of in waves of whole replicas (which
+                // they do, bit for bit the same, where a capture forbids the
+                // allocation of a schedule)
+                if (int rc = class_segments(c, mode, nsteps, slots, st)) return rc;
                 if (int rc = ensure_alloc((void **)&c.cflags_d, sizeof(int) * (B + 2))) return rc;
                 ND_CUDA(cudaMemsetAsync(c.cflags_d, 0, sizeof(int) * (B + 2), st));
                 a.segs = c.segs_d;
@@ -503,7 +537,7 @@ static int run_mode(nd_handle *h, int mode, void *y, void *out, long long nsteps
                 const int ncta = per_sm * h->n_sm;
                 const int Bc = (int)c.reps.size();
                 if (per_sm > 0 && Bc > ncta) {
-                    if (int rc = class_segments(c, mode, nsteps, ncta)) return rc;
+                    if (int rc = class_segments(c, mode, nsteps, ncta, st)) return rc;
                     ND_CUDA(cudaMemsetAsync(h->flags_d, 0, sizeof(int) * h->rep_disk.size(), st));
                     a.segs = c.segs_d;
                     a.seg_off = c.seg_off_d;
@@ -756,7 +790,7 @@ void nd_destroy(nd_handle *h)
     for (auto st2 : h->side) { cudaStreamSynchronize(st2); cudaStreamDestroy(st2); }
     for (auto e2 : h->join_ev) cudaEventDestroy(e2);
     if (h->fork_ev) cudaEventDestroy(h->fork_ev);
-    for (auto &c : h->classes) { cudaFree(c.work_d); cudaFree(c.segs_d); cudaFree(c.seg_off_d); cudaFree(c.cflags_d); }
+    for (auto &c : h->classes) { cudaFree(c.work_d); cudaFree(c.segs_d); cudaFree(c.seg_off_d); cudaFree(c.cflags_d); for (void *p : c.seg_kept) cudaFree(p); }
     cudaFree(h->flags_d);
     cudaFree(h->status_d);
     for (auto &kv : h->tw64) cudaFree(kv.second);

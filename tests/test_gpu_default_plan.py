@@ -73,3 +73,26 @@ def test_replicas_relaxing_in_turns_end_where_they_do_alone(prec, tol, max_iter)
     assert torch.equal(m, torch.cat([p[0] for p in parts]))
     assert np.array_equal(lam, np.concatenate([p[2] for p in parts]))
     assert np.array_equal(it, np.concatenate([p[3] for p in parts]))
+
+
+def test_graph_of_time_sliced_clusters_outlives_other_schedules():
+    """A graph keeps the schedule it was captured with when direct calls of
+    other lengths replace the handle's cached one."""
+    disk = Disk(40e-9, 8e-9, alpha=0.02)
+    B = 20                                                   # more than the resident clusters
+    T, seeds, dt = np.full(B, 300.0), np.arange(B, dtype=np.uint64), 1e-14
+    a, b = Nanodisk([disk], [B]), Nanodisk([disk], [B])
+    ma, mb, mc = a.empty_device(), b.empty_device(), a.empty_device()
+    for h, m in ((a, ma), (b, mb), (a, mc)):
+        h.init_vortex(m, np.zeros((B, 2)))
+    g = nd.nd_graph_create(a.h, ma, nd.ND_METHOD_HEUN, 6, dt, T, seeds, step0=0)
+    try:
+        for k in range(3):
+            nd.nd_graph_launch(g)
+            a.heun(mc, 3 + k, dt, T, seeds)                  # another schedule each time
+            b.heun(mb, 6, dt, T, seeds, step0=6 * k)
+        torch.cuda.synchronize()
+        assert torch.equal(ma, mb)
+    finally:
+        nd.nd_graph_destroy(g)
+    assert nd.nd_check_status(a.h) == nd.ND_OK
