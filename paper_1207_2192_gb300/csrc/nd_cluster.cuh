@@ -1,5 +1,5 @@
-// nd_cluster.cuh -- one replica's time steps on a thread-block cluster of NC
-// CTAs (one per SM): for the sizes P <= 128 when a class has too few replicas
+// nd_cluster.cuh -- one replica's time steps, constrained relaxation or field
+// on a thread-block cluster of NC CTAs (one per SM): for the sizes P <= 128 when a class has too few replicas
 // to fill the GPU with one CTA each, and for P = 192 and 256, whose spectra
 // fit in the shared memory of 16 CTAs but not of one.
 //
@@ -30,6 +30,12 @@
 // read once at the start and written once at the end.  The waits on the
 // transaction barriers give up after about two seconds, set ND_DEV_TIMEOUT in
 // the status word and skip the remaining waits, so a launch always ends.
+//
+// What bounds it: the chain of one evaluation (rows, exchange, columns,
+// exchange, rows, cells), 4.9 us at P = 128 with FP32 and 16 CTAs; in FP64 the
+// issue of one warp instruction per 64-76 cycles and sub-partition.  One disk of
+// R = 50 nm, 50 Heun steps: 497 us; 16 of R = 60 nm, 50 RK4 steps, time-sliced
+// over 15 clusters of 8: 1.25 ms against 4.42 on one CTA each.
 #pragma once
 #include <cooperative_groups.h>
 
