@@ -12,9 +12,9 @@
 //   k_energy_cols  three groups per column slot (x, y, z), each transforms its
 //                  column and sums its part of both forms; the last CTA of a
 //                  replica adds the partial sums in a fixed order.
-// Sixteen replicas of R = 60 nm (P = 128), energies with dE/dL: the former two
-// field evaluations (rows, columns there and back, epilogue) took 2 x 240 us;
-// this takes about 35 us.
+// Sixteen replicas of R = 60 nm (P = 128), energies with dE/dL, cold cache: the
+// former two field evaluations (rows, columns there and back, epilogue) took
+// 2 x 240 us; the rows here take 18 us (21 in CTAs of four warps), the columns 47.
 #include <math.h>
 
 #include "nd_phases.cuh"
@@ -29,7 +29,7 @@ template <typename S> struct MaskedRow {
     __device__ __forceinline__ double operator[](int x) const { return mask[x] ? (double)p[x] : 0.0; }
 };
 
-constexpr int kRowThreads = 128;
+constexpr int kRowThreads = 32;   // one warp: the row tasks spread over every sub-partition
 
 template <int P, typename S>
 __global__ void __launch_bounds__(kRowThreads)
