@@ -245,8 +245,9 @@ int nd_relax_sweep_grad(nd_handle *h, void *m, const void *grad, const double *X
 /* Synchronise `stream` and read (then clear) the handle's device status
  * word.  Returns ND_ERR_TIMEOUT if a bounded device-side wait expired since
  * the last check (the time-sliced stepping schedule hands replicas between
- * CTAs through flags and gives up rather than hang), ND_ERR_NAN if a kernel
- * flagged non-finite values, else ND_OK.  The paper has no counterpart. */
+ * CTAs through flags and gives up rather than hang), ND_ERR_ARG if stepping
+ * calls of this handle were found to overlap (they must be ordered),
+ * ND_ERR_NAN if a kernel flagged non-finite values, else ND_OK.  The paper has no counterpart. */
 int nd_check_status(nd_handle *h, void *stream);
 
 /* Failure-path self-test of the time-sliced schedule: launches the stepping
@@ -402,7 +403,9 @@ int nd_plan_info(const nd_handle *h, int cls, int *P, int *n_replicas, int *plan
  * nd_graph_join makes one graph of n_parts graphs (for example the RK4 graph
  * of a handle of T = 0 replicas and the Heun graph of a handle of the others)
  * as independent branches: one nd_graph_launch replays all parts side by
- * side, each advancing its own step counter as its own launch would.  The
+ * side, each advancing its own step counter as its own launch would.  Parts
+ * that step the same handle share its working memory, so they follow one
+ * another in the order given (parts of joined graphs included).  The
  * parts must outlive the joined graph (it uses their device buffers); destroy
  * it with nd_graph_destroy.  ND_ERR_ARG for no parts or a null part. */
 typedef struct nd_graph nd_graph;

@@ -1277,6 +1277,7 @@ int nd_check_status(nd_handle *h, void *stream)
     unsigned v = 0;
     ND_CUDA(cudaMemcpy(&v, h->status_d, sizeof(v), cudaMemcpyDeviceToHost));
     ND_CUDA(cudaMemset(h->status_d, 0, sizeof(v)));
+    if (v & ND_DEV_ORDER) return fail(ND_ERR_ARG, "calls on one handle overlapped: their states are not valid");
     if (v & ND_DEV_TIMEOUT) return fail(ND_ERR_TIMEOUT, "a bounded device-side wait expired (replica hand-over)");
     if (v & ND_DEV_NAN) return fail(ND_ERR_NAN, "non-finite values in the state");
     return ND_OK;
@@ -1838,6 +1839,7 @@ struct nd_graph {
     cudaStream_t cap = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
+    std::vector<nd_handle *> handles; // the handles it steps (those of all parts of a joined graph)
 };
 
 void nd_graph_destroy(nd_graph *g)
@@ -1866,6 +1868,7 @@ int nd_graph_create(nd_handle *h, void *m, int method, long long n_steps, double
     const int mode = method == ND_METHOD_RK4 ? M_RK4 : M_HEUN;
     nd_graph *g = new nd_graph();
     g->h = h;
+    g->handles.push_back(h);
     auto bail = [&](int code, const std::string &msg) {
         nd_graph_destroy(g);
         return fail(code, msg);
@@ -1921,9 +1924,18 @@ int nd_graph_join(nd_graph *const *parts, int n_parts, nd_graph **out)
         if (!parts[k] || !parts[k]->graph) return fail(ND_ERR_ARG, "null graph among the parts");
     nd_graph *g = new nd_graph();
     cudaError_t e = cudaGraphCreate(&g->graph, 0);
+    std::vector<cudaGraphNode_t> nodes(n_parts);
     for (int k = 0; k < n_parts && e == cudaSuccess; ++k) {
-        cudaGraphNode_t node;
-        e = cudaGraphAddChildGraphNode(&node, g->graph, nullptr, 0, parts[k]->graph);   // no edges: side by side
+        // side by side, but a part follows the earlier parts that step a handle
+        // of its own: they share its accumulators, hand-over flags and tickets
+        const std::vector<nd_handle *> &hk = parts[k]->handles;
+        std::vector<cudaGraphNode_t> after;
+        for (int j = 0; j < k; ++j) {
+            const std::vector<nd_handle *> &hj = parts[j]->handles;
+            if (std::find_first_of(hk.begin(), hk.end(), hj.begin(), hj.end()) != hk.end()) after.push_back(nodes[j]);
+        }
+        e = cudaGraphAddChildGraphNode(&nodes[k], g->graph, after.data(), after.size(), parts[k]->graph);
+        g->handles.insert(g->handles.end(), hk.begin(), hk.end());
     }
     if (e == cudaSuccess) e = cudaGraphInstantiate(&g->exec, g->graph, 0);
     if (e != cudaSuccess) {

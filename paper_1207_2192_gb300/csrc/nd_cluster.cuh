@@ -239,8 +239,12 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     const int slot = SEG && !RELAX ? *cluster.map_shared_rank(&bcast, 0) : 0;
     uint32_t phase = 0, hphase = 0;
     bool bailed = false;   // this thread's wait ran out once: it skips every later wait
-    const int sg_begin = SEG && !RELAX ? seg_off[slot] : 0;
-    const int sg_end = RELAX ? 0x7fffffff : SEG ? seg_off[slot + 1] : 1;
+    // Only launches that share the counter (calls of one handle that overlap) draw
+    // a ticket beyond the schedule: such a cluster has nothing to run.
+    const bool beyond = SEG && !RELAX && slot >= (int)(gridDim.x / NC);
+    if (beyond && rank == 0 && tid == 0) atomicOr(status, ND_DEV_ORDER);
+    const int sg_begin = SEG && !RELAX && !beyond ? seg_off[slot] : 0;
+    const int sg_end = RELAX ? 0x7fffffff : beyond ? 0 : SEG ? seg_off[slot + 1] : 1;
     for (int sg = sg_begin; sg < sg_end; ++sg) {
     Segment seg;
     if constexpr (RELAX) {

@@ -225,6 +225,6 @@ struct StatsAcc {
 };
 
 // Status word written by kernels (bit flags), read by the host after a sync.
-enum : unsigned { ND_DEV_NAN = 1u, ND_DEV_TIMEOUT = 2u };
+enum : unsigned { ND_DEV_NAN = 1u, ND_DEV_TIMEOUT = 2u, ND_DEV_ORDER = 4u };
 
 }  // namespace nd
