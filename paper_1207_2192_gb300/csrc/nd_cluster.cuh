@@ -217,12 +217,17 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     extern __shared__ __align__(16) unsigned char smem[];
     const int tid = threadIdx.x;
     GroupId<P> gid(tid);
-    unsigned long long *mbars = reinterpret_cast<unsigned long long *>(smem);   // [0] columns, [1] rows, [2] sums, [3] halos
-    const uint32_t mb_col = smem_addr(mbars), mb_row = smem_addr(mbars + 1), mb_red = smem_addr(mbars + 2);
-    const uint32_t mb_halo = smem_addr(mbars + 3);
+    unsigned long long *mbars = reinterpret_cast<unsigned long long *>(smem);   // [0] columns, [1] rows, [2] [3] sums
+    const uint32_t mb_col = smem_addr(mbars), mb_row = smem_addr(mbars + 1), mb_sum = smem_addr(mbars + 2);
+    __shared__ unsigned long long halo_bar;
+    const uint32_t mb_halo = smem_addr(&halo_bar);
     cplx<T> *tw = reinterpret_cast<cplx<T> *>(smem + 32);
     __shared__ RelaxAcc<T> racc[RELAX ? NT / 32 : 1];   // per warp
-    __shared__ T rpart[RELAX ? NC : 1][6];              // per CTA of the cluster
+    // Per CTA of the cluster, for even and odd sweeps: a CTA without rows waits
+    // for no field of the others, so its sums of the next sweep may reach another
+    // such CTA before a third one's of this sweep.  It cannot be two sweeps ahead
+    // (it needs everyone's sums to go on).
+    __shared__ T rpart[2][RELAX ? NC : 1][6];
     __shared__ T lam_s[2];
     __shared__ int conv_s;
     __shared__ int bcast;   // rank 0's: the cluster's ticket, then whether a hand-over arrived
@@ -230,14 +235,15 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     if (tid == 0) {
         mbar_init(mb_col, 1);
         mbar_init(mb_row, 1);
-        mbar_init(mb_red, 1);
+        mbar_init(mb_sum, 1);
+        mbar_init(mb_sum + 8, 1);
         mbar_init(mb_halo, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (SEG && !RELAX && rank == 0) bcast = atomicAdd(ticket, 1);
     }
     cluster.sync();   // every CTA runs, with its barriers initialised, before the first remote store
     const int slot = SEG && !RELAX ? *cluster.map_shared_rank(&bcast, 0) : 0;
-    uint32_t phase = 0, hphase = 0;
+    uint32_t phase = 0, hphase = 0, sweep = 0;   // sweep: of the launch, over all its turns
     bool bailed = false;   // this thread's wait ran out once: it skips every later wait
     // Only launches that share the counter (calls of one handle that overlap) draw
     // a ticket beyond the schedule: such a cluster has nothing to run.
@@ -399,7 +405,7 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
             if (tid == 0) {
                 mbar_expect(mb_col, bytes_col);
                 mbar_expect(mb_row, bytes_row);
-                if (RELAX) mbar_expect(mb_red, (uint32_t)((NC - 1) * 6 * sizeof(T)));
+                if (RELAX) mbar_expect(mb_sum + 8 * (sweep & 1), (uint32_t)((NC - 1) * 6 * sizeof(T)));
             }
             // 1. forward rows of the CTA's own rows, sent to the column owners
             if constexpr (HR) {
@@ -654,6 +660,8 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
                 a.J01 = warp_sum_t(a.J01); a.J11 = warp_sum_t(a.J11); a.res = warp_max_t(a.res);
                 if ((tid & 31) == 0) racc[tid >> 5] = a;
                 __syncthreads();
+                T(*const rp)[6] = rpart[sweep & 1];
+                const uint32_t mb_red = mb_sum + 8 * (sweep & 1);
                 if (tid < 6 * NC) {   // value v of this CTA to CTA q
                     const int q = tid / 6, v = tid - 6 * q;
                     T t = (&racc[0].C0)[v];
@@ -661,18 +669,18 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
                         const T u = (&racc[w].C0)[v];
                         t = v == 5 ? max(t, u) : t + u;
                     }
-                    if (q == rank) rpart[q][v] = t;
-                    else st_async(cluster_addr(smem_addr(&rpart[rank][v]), q), t, cluster_addr(mb_red, q));
+                    if (q == rank) rp[q][v] = t;
+                    else st_async(cluster_addr(smem_addr(&rp[rank][v]), q), t, cluster_addr(mb_red, q));
                 }
                 __syncthreads();
                 if (tid < 32) {
-                    if (!bailed && !mbar_wait(mb_red, (phase - 1) & 1)) {
+                    if (!bailed && !mbar_wait(mb_red, (sweep >> 1) & 1)) {
                         bailed = true;
                         atomicOr(status, ND_DEV_TIMEOUT);
                     }
                     const int v = min(tid, 5);
-                    T t = rpart[0][v];
-                    for (int q = 1; q < NC; ++q) t = v == 5 ? max(t, rpart[q][v]) : t + rpart[q][v];
+                    T t = rp[0][v];
+                    for (int q = 1; q < NC; ++q) t = v == 5 ? max(t, rp[q][v]) : t + rp[q][v];
                     const T C0 = __shfl_sync(0xffffffffu, t, 0), C1 = __shfl_sync(0xffffffffu, t, 1);
                     const T J00 = __shfl_sync(0xffffffffu, t, 2), J01 = __shfl_sync(0xffffffffu, t, 3);
                     const T J11 = __shfl_sync(0xffffffffu, t, 4), res = __shfl_sync(0xffffffffu, t, 5);
@@ -690,6 +698,7 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
                     }
                 }
                 __syncthreads();
+                ++sweep;
                 if (conv_s) break;   // leaves the stage loop; the sweep loop stops below
                 const T m0 = lam_s[0], m1 = lam_s[1];
                 for (int k = c0 + tid; k < c1; k += NT) {
