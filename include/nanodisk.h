@@ -245,20 +245,32 @@ int nd_relax_sweep_grad(nd_handle *h, void *m, const void *grad, const double *X
 /* Synchronise `stream` and read (then clear) the handle's device status
  * word.  Returns ND_ERR_TIMEOUT if a bounded device-side wait expired since
  * the last check (the time-sliced stepping schedule hands replicas between
- * CTAs through flags and gives up rather than hang), ND_ERR_ARG if stepping
+ * CTAs through flags, and gives up rather than hang when the other side has
+ * made no progress for about two seconds), ND_ERR_ARG if stepping
  * calls of this handle were found to overlap (they must be ordered),
  * ND_ERR_NAN if a kernel flagged non-finite values, else ND_OK.  The paper has no counterpart. */
 int nd_check_status(nd_handle *h, void *stream);
 
 /* Failure-path self-test of the time-sliced schedule: launches the stepping
  * kernel as one CTA with one segment that waits for a replica hand-over flag
- * that no segment ever sets.  The wait is bounded (about one second of
+ * that no segment ever sets.  The wait is bounded (about two seconds of
  * polling); when it expires the kernel sets ND_DEV_TIMEOUT in the handle's
  * status word and returns without reading or writing any state, so the
  * context stays usable and the next nd_check_status returns ND_ERR_TIMEOUT.
  * Synchronises `stream`.  Needs an ND_FP32 handle whose first size class is
  * held on chip (P <= 128), else ND_ERR_ARG.  The paper has no counterpart. */
 int nd_selftest_handover_timeout(nd_handle *h, void *stream);
+
+/* Self-test of a long hand-over: n_steps RK4 steps of the first replica of
+ * the first size class, cut in halves for two CTAs (plan 0) or two clusters
+ * (plan 200 or 201).  The second waits for the whole first half, with a limit
+ * of about 17 ms instead of two seconds: the wait outlasts it when the first
+ * half does, since the limit counts from the last progress of the other side.
+ * The state m (device) ends as after nd_step_rk4, other replicas untouched;
+ * nd_check_status returns ND_OK.  Synchronises `stream`.  Needs a handle as
+ * nd_selftest_handover_timeout does, else ND_ERR_ARG.  The paper has no
+ * counterpart. */
+int nd_selftest_handover_progress(nd_handle *h, void *m, long long n_steps, double dt_seconds, int plan, void *stream);
 
 /* Analytic q = +1 vortex centred at X0[r] = (x0, y0) metres (host array
  * [B][2]) for every replica (Sec. IV profile): in-plane angle atan2(y - y0,

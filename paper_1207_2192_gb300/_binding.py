@@ -67,6 +67,7 @@ SIGNATURES = {
     "nd_stats_reset": (_I, [_P, _D, _I, _D, _I]),
     "nd_check_status": (_I, [_P, _P]),
     "nd_selftest_handover_timeout": (_I, [_P, _P]),
+    "nd_selftest_handover_progress": (_I, [_P, _P, _LL, _D, _I, _P]),
     "nd_graph_create": (_I, [_P, _P, _I, _LL, _D, _P, _P, _ULL, _I, _P]),
     "nd_autotune": (_I, [_P, _I, _D, _LL, _P]),
     "nd_autotune_group": (_I, [_P, _P, _I, _D, _LL, _P]),
@@ -355,6 +356,11 @@ def nd_check_status(h, stream=None):
 def nd_selftest_handover_timeout(h, stream=None):
     """Run the bounded-wait failure path once (see include/nanodisk.h)."""
     _check(lib().nd_selftest_handover_timeout(h, _stream(stream)))
+
+
+def nd_selftest_handover_progress(h, m, n_steps, dt_seconds, plan, stream=None):
+    """RK4 steps of the first replica passed on once between two CTAs or clusters (see include/nanodisk.h)."""
+    _check(lib().nd_selftest_handover_progress(h, _ptr(m), int(n_steps), float(dt_seconds), int(plan), _stream(stream)))
 
 
 ND_GRAPH_STATS = 1

@@ -1327,6 +1327,58 @@ int nd_selftest_handover_timeout(nd_handle *h, void *stream)
     return ND_OK;
 }
 
+int nd_selftest_handover_progress(nd_handle *h, void *m, long long n_steps, double dt_seconds, int plan, void *stream)
+{
+    if (int rc = check_handle(h)) return rc;
+    auto &c = h->classes[0];
+    const int nc = plan_cluster_nc(plan), prec = ND_PREC_FP32;
+    if (!c.fused_main || h->prec == ND_FP64 || (plan != 0 && !nc) || (nc && !cluster_plan_fits(h, c, prec, false, nc)))
+        return fail(ND_ERR_ARG, "the hand-over self-test needs an on-chip FP32 size class first in the handle and plan 0, 200 or 201");
+    if (!m || !is_device_ptr(m) || n_steps < 2 || !(dt_seconds > 0))
+        return fail(ND_ERR_ARG, "the hand-over self-test needs a device state, n_steps >= 2 and dt > 0");
+    cudaStream_t st = (cudaStream_t)stream;
+    const int B = (int)h->rep_disk.size();
+    std::vector<SegmentHost> segs;
+    std::vector<int> off;
+    build_segments(1, n_steps, 2, segs, off);
+    for (auto &g : segs) g.rep = c.reps[0];
+    void *segs_d = nullptr, *off_d = nullptr;
+    ND_CUDA(cudaMalloc(&segs_d, sizeof(SegmentHost) * segs.size()));
+    cudaError_t e = cudaMalloc(&off_d, sizeof(int) * off.size());
+    if (e == cudaSuccess) e = cudaMemcpy(segs_d, segs.data(), sizeof(SegmentHost) * segs.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(off_d, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && !c.cflags_d) e = cudaMalloc((void **)&c.cflags_d, sizeof(int) * (B + 2));
+    if (e == cudaSuccess) e = cudaMemsetAsync(c.cflags_d, 0, sizeof(int) * (B + 2), st);
+    if (e == cudaSuccess) {
+        fill_reps(h, dt_seconds, nullptr, nullptr, 0);
+        upload_reps(h, st);
+        LaunchArgs a;
+        a.mode = M_RK4;
+        a.reps = h->reps_d;
+        a.work = c.work_d;
+        a.nwork = 1;
+        a.y = m;
+        a.acc = h->acc;
+        a.tw = h->tw32[c.P];
+        a.nsteps = n_steps;
+        a.smem = c.smem_main;
+        a.stream = st;
+        a.status = h->status_d;
+        a.segs = segs_d;
+        a.seg_off = (const int *)off_d;
+        a.flags = c.cflags_d;
+        a.n_rep = B;
+        a.ncta = 2;
+        a.wait_polls = 1 << 15;
+        e = nc ? launch_cluster(c.P, prec, a, c.maxD, c.maxDpad, nc) : launch_fused(c.P, prec, a);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    cudaFree(segs_d);
+    cudaFree(off_d);
+    if (e != cudaSuccess) return fail(ND_ERR_CUDA, std::string("hand-over self-test: ") + cudaGetErrorString(e));
+    return ND_OK;
+}
+
 int nd_stats_reset(nd_handle *h, double r_max, int r_bins, double v_max, int v_bins)
 {
     if (int rc = check_handle(h)) return rc;

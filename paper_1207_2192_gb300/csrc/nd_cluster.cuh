@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     k_cluster(const Replica *__restrict__ reps, const int *__restrict__ work, T *__restrict__ ybase, T *__restrict__ outbase,
               const cplx<T> *__restrict__ twP, long long nsteps_all, unsigned long long step_base, int use_wbuf,
               unsigned *__restrict__ status, const Segment *__restrict__ segs, const int *__restrict__ seg_off,
-              int *__restrict__ flags, int *__restrict__ ticket, const ClusterRelax rx)
+              int *__restrict__ flags, int *__restrict__ ticket, int wait_polls, const ClusterRelax rx)
 {
     using Gm = FFTGeom<P>;
     using CG = ClusterGeom<P, T, NC>;
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     if (SEG && !RELAX) {   // (the same for every CTA of the cluster)
         cluster.sync();   // the ticket is read; the previous segment's rows and columns are no longer used
         if (rank == 0 && tid == 0) {
-            bcast = seg.wait ? (int)wait_flag(flags + seg.rep) : 1;
+            bcast = seg.wait ? (int)wait_flag(flags + seg.rep, wait_polls) : 1;
             if (!bcast) atomicOr(status, ND_DEV_TIMEOUT);
         }
         cluster.sync();
@@ -752,6 +752,7 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
             }
             __syncthreads();
         }
+        if (SEG && !RELAX && rank == 0 && tid == 0 && seg.signal) post_progress(flags + seg.rep, n);
         if (RELAX && conv_s) break;
     }
     // the final state of the CTA's cells back to the caller's buffer
@@ -782,7 +783,7 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
         if (rank == 0 && tid == 0) {
             __threadfence();
             if (RELAX) atomicAdd(flags + seg.rep, 1);
-            else atomicExch(flags + seg.rep, 1);
+            else atomicExch(flags + seg.rep, kHandedOver);
         }
     }
     }
@@ -825,7 +826,7 @@ static cudaError_t launch_cluster_t(const LaunchArgs &a, int maxD, int maxDpad)
                              a.flags ? a.flags + a.n_rep + 1 : nullptr};
     return cudaLaunchKernelEx(&cfg, k_cluster<P, T, MODE, NC, SEG>, a.reps, a.work, (T *)a.y, (T *)a.out,
                               (const cplx<T> *)a.tw, a.nsteps, a.step_base, a.use_wbuf, a.status, reinterpret_cast<const Segment *>(a.segs),
-                              a.seg_off, a.flags, a.flags ? a.flags + a.n_rep : nullptr, rx);
+                              a.seg_off, a.flags, a.flags ? a.flags + a.n_rep : nullptr, a.wait_polls, rx);
 }
 
 // Clusters of the size class that can be resident at once (0: the cluster

@@ -210,21 +210,39 @@ __host__ __device__ __forceinline__ size_t fused_smem_bytes(int D, int Dpad, int
 // A piece of one replica's trajectory run by one CTA (time-sliced schedule).
 struct Segment {
     int rep;                 // replica index
-    int wait;                // wait until flags[rep] is set before starting
-    int signal;              // set flags[rep] when done
+    int wait;                // wait until flags[rep] is kHandedOver before starting
+    int signal;              // set flags[rep] to kHandedOver when done
     int pad;
     long long step_begin;    // first time step (relative to the call's step0)
     long long nsteps;
 };
 
-// Bounded wait of thread 0 on a flag set by another CTA of the same
-// (cooperative) launch; returns false after about 2^22 polls.
-__device__ __forceinline__ bool wait_flag(int *flag)
+// The hand-over word of a replica: 0, then a count that the signalling segment
+// posts every 64 steps, at last kHandedOver.
+constexpr int kHandedOver = -1;
+__device__ __forceinline__ void post_progress(int *flag, long long n)
 {
-    for (long long it = 0; it < (1LL << 22); ++it) {
-        if (atomicAdd(flag, 0) != 0) {
+    if ((n & 63) == 63) atomicExch(flag, (int)((n >> 6) & 0x3fffffff) + 1);
+}
+
+// Wait of one thread until another CTA (cluster) of the same launch, one that
+// runs already, hands a replica over.  The wait lasts as long as the other
+// side works, which grows with the steps of the call and with the difference
+// of the replicas' costs: it gives up, and returns false, after `polls` polls
+// in which the word has not moved (2^22, about two seconds, against 64 steps of
+// at most a few hundred us each).
+__device__ __forceinline__ bool wait_flag(int *flag, int polls)
+{
+    int seen = 0;
+    for (int it = 0; it < polls; ++it) {
+        const int v = atomicAdd(flag, 0);
+        if (v == kHandedOver) {
             __threadfence();
             return true;
+        }
+        if (v != seen) {
+            seen = v;
+            it = 0;
         }
         __nanosleep(256);
     }
@@ -309,7 +327,7 @@ __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
             T *__restrict__ accbase, T *__restrict__ outbase, const cplx<T> *__restrict__ twP, long long nsteps, unsigned long long step_base,
             RelaxIO *__restrict__ rio, double eta_d, double tol_d, double rc2_d, int max_iter,
             const Segment *__restrict__ segs, const int *__restrict__ seg_off, int *__restrict__ flags,
-            unsigned *__restrict__ status, int use_wbuf)
+            int wait_polls, unsigned *__restrict__ status, int use_wbuf)
 {
     using Gm = FFTGeom<P>;
     constexpr int G = Gm::G, R1 = Gm::R1, RS = SpecGeom<P>::RS, GPW = Gm::GROUPS_PER_WARP;
@@ -317,7 +335,7 @@ __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ Replica r_sh;   // the descriptor stays in shared memory, not in registers
     __shared__ T lam_s[2];
-    __shared__ int conv_s, ok_s;
+    __shared__ int conv_s, ok_s, signal_s;
     __shared__ RelaxAcc<T> racc[NW];
     const int tid = threadIdx.x, warp = tid >> 5;
     GroupId<P> gid(tid);
@@ -338,8 +356,9 @@ __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
             ridx = work[blockIdx.x];
         }
         if (tid == 0) {
-            ok_s = wait ? (int)wait_flag(flags + ridx) : 1;
+            ok_s = wait ? (int)wait_flag(flags + ridx, wait_polls) : 1;
             if (!ok_s) atomicOr(status, ND_DEV_TIMEOUT);
+            signal_s = signal;
             r_sh = reps[ridx];
         }
         __syncthreads();
@@ -514,6 +533,7 @@ __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
                 }
                 __syncthreads();
             }
+            if ((MODE == M_RK4 || MODE == M_HEUN) && tid == 0 && signal_s) post_progress(flags + ridx, n);
             if (MODE == M_RELAX && conv_s) break;
         }
         if (MODE == M_RELAX) {
@@ -533,9 +553,9 @@ __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
             }
         }
         __syncthreads();   // every write of this segment is done before the flag and the next segment
-        if (signal && tid == 0) {
+        if (tid == 0 && signal_s) {
             __threadfence();
-            atomicExch(flags + ridx, 1);
+            atomicExch(flags + ridx, kHandedOver);
         }
     }
 }
@@ -1171,7 +1191,8 @@ static cudaError_t launch_fused_t(const LaunchArgs &a)
     if (!segs) {
         kern<<<a.nwork, NT, a.smem, a.stream>>>(a.reps, a.work, (T *)a.y, (T *)a.acc, (T *)a.out,
                                                 (const cplx<T> *)a.tw, a.nsteps, a.step_base, a.rio, a.eta, a.tol,
-                                                a.rc2, a.max_iter, nullptr, nullptr, nullptr, a.status, a.use_wbuf);
+                                                a.rc2, a.max_iter, nullptr, nullptr, nullptr, a.wait_polls, a.status,
+                                                a.use_wbuf);
         return cudaGetLastError();
     }
     // time-sliced schedule: the CTAs wait on one another, so they must all be
@@ -1184,14 +1205,14 @@ static cudaError_t launch_fused_t(const LaunchArgs &a)
     unsigned long long step_base = a.step_base;
     RelaxIO *rio = a.rio;
     double eta = a.eta, tol = a.tol, rc2 = a.rc2;
-    int max_iter = a.max_iter, use_wbuf = a.use_wbuf;
+    int max_iter = a.max_iter, use_wbuf = a.use_wbuf, wait_polls = a.wait_polls;
     const int *seg_off = a.seg_off;
     int *flags = a.flags;
     unsigned *status = a.status;
     void *args[] = {(void *)&reps, (void *)&work, (void *)&y, (void *)&acc, (void *)&out, (void *)&tw,
                     (void *)&nsteps, (void *)&step_base, (void *)&rio, (void *)&eta, (void *)&tol, (void *)&rc2,
-                    (void *)&max_iter, (void *)&segs, (void *)&seg_off, (void *)&flags, (void *)&status,
-                    (void *)&use_wbuf};
+                    (void *)&max_iter, (void *)&segs, (void *)&seg_off, (void *)&flags, (void *)&wait_polls,
+                    (void *)&status, (void *)&use_wbuf};
     // cudaLaunchKernelEx with the cooperative attribute is also legal inside a
     // stream capture (graph kernel node)
     cudaLaunchConfig_t cfg = {};

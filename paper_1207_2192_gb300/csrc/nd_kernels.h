@@ -46,6 +46,7 @@ struct LaunchArgs {
     int *flags = nullptr;            // cluster plans: n_rep flags, then the ticket counter
     int n_rep = 0;
     int ncta = 0;                    // CTAs (cluster plans: clusters) of the schedule
+    int wait_polls = 1 << 22;        // polls without progress after which a hand-over wait gives up
     unsigned *status = nullptr;      // device status word (ND_DEV_* bits)
     int use_wbuf = 0;                // keep the Heun predictor's normals in shared memory
     int smem_optin = 0;              // per-block shared-memory limit of the device
