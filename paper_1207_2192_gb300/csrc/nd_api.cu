@@ -450,6 +450,35 @@ static int field_cluster_nc(const nd_handle *h, const SizeClass &c)
     return waves * (nc == 8 ? e->c8 : e->c16) < e->one ? nc : 0;
 }
 
+// Size classes side by side: side stream k, forked from the caller's stream,
+// is joined back to it on every way out, errors included, so that whatever
+// follows on the caller's stream comes after the classes that were launched.
+struct SideBySide {
+    nd_handle *h;
+    cudaStream_t st;
+    size_t used = 0;   // side streams 0..used-1
+    SideBySide(nd_handle *h_, cudaStream_t st_) : h(h_), st(st_) {}
+    ~SideBySide() { join(); }
+    cudaError_t fork() { return cudaEventRecord(h->fork_ev, st); }
+    cudaError_t next(cudaStream_t *s)
+    {
+        *s = h->side[used];
+        const cudaError_t e = cudaStreamWaitEvent(*s, h->fork_ev, 0);
+        if (e == cudaSuccess) ++used;
+        return e;
+    }
+    cudaError_t join()
+    {
+        cudaError_t first = cudaSuccess;
+        for (; used > 0; --used) {
+            cudaError_t e = cudaEventRecord(h->join_ev[used - 1], h->side[used - 1]);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(st, h->join_ev[used - 1], 0);
+            if (first == cudaSuccess) first = e;
+        }
+        return first;
+    }
+};
+
 // Run one mode over all replicas in the handle's precision.
 static int run_mode(nd_handle *h, int mode, void *y, void *out, long long nsteps, cudaStream_t st,
                     const Replica *reps = nullptr, int only_class = -1)
@@ -464,16 +493,14 @@ static int run_mode(nd_handle *h, int mode, void *y, void *out, long long nsteps
                       h->side.size() + 1 == h->classes.size();
     for (const auto &c : h->classes)
         if ((int)c.reps.size() > h->n_sm) concurrent = false;
-    if (concurrent) ND_CUDA(cudaEventRecord(h->fork_ev, st));
+    SideBySide sides(h, st);
+    if (concurrent) ND_CUDA(sides.fork());
     const cudaStream_t st0 = st;
     for (int ci = 0; ci < (int)h->classes.size(); ++ci) {
         if (only_class >= 0 && ci != only_class) continue;
         auto &c = h->classes[ci];
         cudaStream_t st = st0;
-        if (concurrent && ci > 0) {
-            st = h->side[ci - 1];
-            ND_CUDA(cudaStreamWaitEvent(st, h->fork_ev, 0));
-        }
+        if (concurrent && ci > 0) ND_CUDA(sides.next(&st));
         LaunchArgs a;
         a.mode = mode;
         a.reps = reps ? reps : h->reps_d;
@@ -556,10 +583,8 @@ static int run_mode(nd_handle *h, int mode, void *y, void *out, long long nsteps
         // word (the cluster kernel looks at its cells itself)
         if (stepping && !cluster_nc)
             ND_CUDA(launch_check_finite(prec, a.reps, c.work_d, (int)c.reps.size(), c.maxD, y, h->status_d, st));
-        if (concurrent && ci > 0) ND_CUDA(cudaEventRecord(h->join_ev[ci - 1], st));
     }
-    if (concurrent)
-        for (size_t k = 0; k < h->side.size(); ++k) ND_CUDA(cudaStreamWaitEvent(st0, h->join_ev[k], 0));
+    ND_CUDA(sides.join());
     return ND_OK;
 }
 
@@ -1072,22 +1097,18 @@ int nd_relax_constrained(nd_handle *h, void *m, const double *X, double tol, int
     // streams, and those on the global path, whose host loop waits for each 32
     // sweeps, follow one by one on the caller's.
     const bool side = h->side.size() + 1 == h->classes.size() && !h->side.empty();
-    if (side) ND_CUDA(cudaEventRecord(h->fork_ev, st));
+    SideBySide sides(h, st);
+    if (side) ND_CUDA(sides.fork());
     auto on_chip = [&](const SizeClass &c) { return c.fused_main || relax_cluster_nc(h, c); };
     std::vector<int> order;
     for (int pass = 0; pass < 2; ++pass)
         for (int ci = 0; ci < (int)h->classes.size(); ++ci)
             if (on_chip(h->classes[ci]) == (pass == 0)) order.push_back(ci);
-    size_t nside = 0;
-    std::vector<cudaEvent_t> joined;
     const cudaStream_t st0 = st;
     for (int ci : order) {
         auto &c = h->classes[ci];
         cudaStream_t st = st0;
-        if (side && nside < h->side.size() && on_chip(c)) {
-            st = h->side[nside++];
-            ND_CUDA(cudaStreamWaitEvent(st, h->fork_ev, 0));
-        }
+        if (side && sides.used < h->side.size() && on_chip(c)) ND_CUDA(sides.next(&st));
         const DiskInfo &d = h->disks[h->rep_disk[c.reps[0]]];
         const double rcut = 4.0 * d.lambda / d.desc.a;
         LaunchArgs a;
@@ -1131,12 +1152,8 @@ int nd_relax_constrained(nd_handle *h, void *m, const double *X, double tol, int
             a.n_sm = h->n_sm;
             ND_CUDA(launch_global(c.P, prec, a, c.maxD));
         }
-        if (st != st0) {
-            ND_CUDA(cudaEventRecord(h->join_ev[nside - 1], st));
-            joined.push_back(h->join_ev[nside - 1]);
-        }
     }
-    for (cudaEvent_t e : joined) ND_CUDA(cudaStreamWaitEvent(st0, e, 0));
+    ND_CUDA(sides.join());
     ND_CUDA(cudaMemcpyAsync(h->rio_h, h->rio_d, sizeof(RelaxIO) * B, cudaMemcpyDeviceToHost, st));
     ND_CUDA(cudaStreamSynchronize(st));
     int rc = ND_OK;
