@@ -220,7 +220,9 @@ int nd_step_heun(nd_handle *h, void *m, long long n_steps, double dt_seconds, co
  * sweep is summed from neighbour differences instead of through the FFT, so
  * with few replicas an ND_FP32 relaxation stops closer to where FP64
  * arithmetic does; the two forms agree to rounding.  Returns ND_ERR_NOT_CONVERGED if
- * a replica reached max_iter.  Synchronises `stream`. */
+ * a replica reached max_iter, ND_ERR_TIMEOUT if a bounded device-side wait
+ * expired (the states are then not valid; nd_check_status reports it once
+ * more).  Synchronises `stream`. */
 int nd_relax_constrained(nd_handle *h, void *m, const double *X, double tol, int max_iter, double *U_out,
                          double *lambda_out, int *iters_out, void *stream);
 
@@ -268,8 +270,15 @@ int nd_selftest_handover_timeout(nd_handle *h, void *stream);
  * half does, since the limit counts from the last progress of the other side.
  * The state m (device) ends as after nd_step_rk4, other replicas untouched;
  * nd_check_status returns ND_OK.  Synchronises `stream`.  Needs a handle as
- * nd_selftest_handover_timeout does, else ND_ERR_ARG.  The paper has no
+ * nd_selftest_handover_timeout does, else ND_ERR_ARG.
+ *
+ * nd_selftest_relax_timeout: a relaxation (arguments as nd_relax_constrained)
+ * whose replicas' turns on the clusters wait for turns that nobody takes, for
+ * some milliseconds each.  Returns ND_ERR_TIMEOUT, as a relaxation in which a
+ * wait expires does, and leaves the states of the first size class alone;
+ * ND_ERR_ARG if that class does not relax on clusters.  The paper has no
  * counterpart. */
+int nd_selftest_relax_timeout(nd_handle *h, void *m, const double *X, void *stream);
 int nd_selftest_handover_progress(nd_handle *h, void *m, long long n_steps, double dt_seconds, int plan, void *stream);
 
 /* Analytic q = +1 vortex centred at X0[r] = (x0, y0) metres (host array

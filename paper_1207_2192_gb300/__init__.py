@@ -14,7 +14,7 @@ import numpy as np
 from . import _binding as _b
 from ._binding import (ND_METHOD_HEUN, ND_METHOD_RK4, nd_autotune, nd_autotune_group, nd_plan_info, nd_set_plan, nd_graph_create, nd_graph_destroy, nd_graph_launch,
                        nd_graph_join,
-                       nd_graph_nodes, nd_check_status, nd_selftest_handover_timeout, nd_selftest_handover_progress, nd_series_reset,
+                       nd_graph_nodes, nd_check_status, nd_selftest_handover_timeout, nd_selftest_handover_progress, nd_selftest_relax_timeout, nd_series_reset,
                        nd_series_sample, nd_series_read, nd_power_spectrum, ND_GRAPH_STATS, ND_GRAPH_SERIES, ND_ERR_ARG, ND_ERR_CUDA, ND_ERR_NAN, ND_ERR_NO_VORTEX, ND_ERR_NOT_CONVERGED, ND_ERR_TIMEOUT,
                        ND_FP32, ND_FP64, ND_GRID_3X, ND_OK, NDError, nd_create_disk, nd_destroy, nd_disk_desc, nd_disk_mask,
                        nd_effective_field, nd_energy, nd_get_info, nd_init_vortex, nd_last_error, nd_mean_m,
@@ -27,7 +27,7 @@ __all__ = ["Disk", "Nanodisk", "NDError", "ND_FP32", "ND_FP64", "ND_GRID_3X", "n
            "nd_energy", "nd_step_rk4", "nd_step_heun", "nd_init_vortex", "nd_vortex_core", "nd_mean_m",
            "nd_set_green_tensor", "nd_set_damping", "nd_set_mask", "nd_set_field_schedule", "nd_units", "nd_replica_layout", "nd_get_info",
            "nd_disk_mask", "nd_last_error", "nd_relax_constrained",
-           "nd_stats_reset", "nd_stats_sample", "nd_stats_read", "nd_stats_save", "nd_stats_load", "nd_check_status", "nd_selftest_handover_timeout", "nd_selftest_handover_progress",
+           "nd_stats_reset", "nd_stats_sample", "nd_stats_read", "nd_stats_save", "nd_stats_load", "nd_check_status", "nd_selftest_handover_timeout", "nd_selftest_handover_progress", "nd_selftest_relax_timeout",
            "nd_series_reset", "nd_series_sample", "nd_series_read", "nd_power_spectrum", "ND_GRAPH_STATS", "ND_GRAPH_SERIES",
            "nd_graph_create", "nd_graph_launch", "nd_graph_join", "nd_graph_nodes", "nd_graph_destroy",
            "nd_autotune", "nd_autotune_group", "nd_plan_info", "nd_set_plan"]

@@ -68,6 +68,7 @@ SIGNATURES = {
     "nd_check_status": (_I, [_P, _P]),
     "nd_selftest_handover_timeout": (_I, [_P, _P]),
     "nd_selftest_handover_progress": (_I, [_P, _P, _LL, _D, _I, _P]),
+    "nd_selftest_relax_timeout": (_I, [_P, _P, _P, _P]),
     "nd_graph_create": (_I, [_P, _P, _I, _LL, _D, _P, _P, _ULL, _I, _P]),
     "nd_autotune": (_I, [_P, _I, _D, _LL, _P]),
     "nd_autotune_group": (_I, [_P, _P, _I, _D, _LL, _P]),
@@ -356,6 +357,12 @@ def nd_check_status(h, stream=None):
 def nd_selftest_handover_timeout(h, stream=None):
     """Run the bounded-wait failure path once (see include/nanodisk.h)."""
     _check(lib().nd_selftest_handover_timeout(h, _stream(stream)))
+
+
+def nd_selftest_relax_timeout(h, m, X, stream=None):
+    """A relaxation whose turns on the clusters never come (see include/nanodisk.h); returns the status code."""
+    X = np.ascontiguousarray(X, dtype=np.float64)
+    return lib().nd_selftest_relax_timeout(h, _ptr(m), _ptr(X), _stream(stream))
 
 
 def nd_selftest_handover_progress(h, m, n_steps, dt_seconds, plan, stream=None):

@@ -192,6 +192,8 @@ struct nd_handle {
     cudaEvent_t fork_ev = nullptr;
     int *flags_d = nullptr;               // [B] replica hand-over flags of the time-sliced schedule
     unsigned *status_d = nullptr;         // device status word (ND_DEV_* bits)
+    unsigned *relax_status = nullptr;     // the same of one relaxation (behind status_d and core_done)
+    unsigned status_seen = 0;             // bits of relaxations, for nd_check_status
     unsigned long long rk4_step = 0;      // step index of the next nd_step_rk4 step (field schedules)
 };
 
@@ -768,9 +770,10 @@ int nd_create_disk(const nd_disk_desc *disks, int n_disks, const int *replicas_p
     if ((e = cudaMalloc(&h->acc, h->elt * h->state_elems)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = cudaMalloc(&h->rio_d, sizeof(RelaxIO) * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = cudaMalloc(&h->flags_d, sizeof(int) * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
-    if ((e = cudaMalloc(&h->status_d, sizeof(unsigned) * (1 + B))) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
-    if ((e = cudaMemset(h->status_d, 0, sizeof(unsigned) * (1 + B))) != cudaSuccess) return cuda_fail(e, "cudaMemset");
+    if ((e = cudaMalloc(&h->status_d, sizeof(unsigned) * (2 + B))) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
+    if ((e = cudaMemset(h->status_d, 0, sizeof(unsigned) * (2 + B))) != cudaSuccess) return cuda_fail(e, "cudaMemset");
     h->core_done = h->status_d + 1;
+    h->relax_status = h->core_done + B;
     if ((e = cudaMallocHost(&h->rio_h, sizeof(RelaxIO) * B)) != cudaSuccess) return cuda_fail(e, "cudaMallocHost");
     if ((e = cudaMalloc(&h->core_d, sizeof(double) * 4 * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = cudaMalloc(&h->core_part, sizeof(double) * 2 * kCoreMaxBlocks * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
@@ -1063,8 +1066,12 @@ int nd_step_heun(nd_handle *h, void *m, long long n_steps, double dt_seconds, co
     return stage_out(h, m, md, st);
 }
 
-int nd_relax_constrained(nd_handle *h, void *m, const double *X, double tol, int max_iter, double *U_out,
-                         double *lambda_out, int *iters_out, void *stream)
+}  // extern "C"
+
+// nd_relax_constrained.  starve (self-test): the clusters' turns begin with the
+// second one of every replica, whose first nobody takes, and wait for a few ms.
+static int relax_constrained(nd_handle *h, void *m, const double *X, double tol, int max_iter, double *U_out,
+                             double *lambda_out, int *iters_out, void *stream, bool starve)
 {
     if (int rc = check_handle(h)) return rc;
     if (!X) return fail(ND_ERR_ARG, "null X");
@@ -1092,6 +1099,7 @@ int nd_relax_constrained(nd_handle *h, void *m, const double *X, double tol, int
         R.status = 1;
     }
     ND_CUDA(cudaMemcpyAsync(h->rio_d, h->rio_h, sizeof(RelaxIO) * B, cudaMemcpyHostToDevice, st));
+    ND_CUDA(cudaMemsetAsync(h->relax_status, 0, sizeof(unsigned), st));
     const int prec = h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32;
     // The classes are independent: the ones that relax in one launch go to side
     // streams, and those on the global path, whose host loop waits for each 32
@@ -1132,13 +1140,17 @@ int nd_relax_constrained(nd_handle *h, void *m, const double *X, double tol, int
             const int slots = cluster_slots(h, c, prec, true, nc), Bc = a.nwork;
             if (int rc = ensure_alloc((void **)&c.cflags_d, sizeof(int) * (B + 2))) return rc;
             ND_CUDA(cudaMemsetAsync(c.cflags_d, 0, sizeof(int) * (B + 2), st));
-            a.status = h->status_d;
+            if (starve) {
+                ND_CUDA(cudaMemcpyAsync(c.cflags_d + B, &a.nwork, sizeof(int), cudaMemcpyHostToDevice, st));
+                a.wait_polls = 1 << 14;
+            }
+            a.status = h->relax_status;
             a.flags = c.cflags_d;
             a.n_rep = B;
             a.ncta = std::min(Bc, slots);
             a.tw64 = h->tw64[c.P];
             a.use_wbuf = 1;   // (the halos take the normals' place)
-            a.quantum = Bc > slots ? kRelaxTurn : std::max(max_iter, 1);
+            a.quantum = starve ? 1 : Bc > slots ? kRelaxTurn : std::max(max_iter, 1);
             ND_CUDA(launch_cluster(c.P, prec, a, c.maxD, c.maxDpad, nc));
         } else if (c.fused_main) {
             ND_CUDA(launch_fused(c.P, prec, a));
@@ -1154,8 +1166,11 @@ int nd_relax_constrained(nd_handle *h, void *m, const double *X, double tol, int
         }
     }
     ND_CUDA(sides.join());
+    unsigned status = 0;
     ND_CUDA(cudaMemcpyAsync(h->rio_h, h->rio_d, sizeof(RelaxIO) * B, cudaMemcpyDeviceToHost, st));
+    ND_CUDA(cudaMemcpyAsync(&status, h->relax_status, sizeof(status), cudaMemcpyDeviceToHost, st));
     ND_CUDA(cudaStreamSynchronize(st));
+    h->status_seen |= status;
     int rc = ND_OK;
     for (int r = 0; r < B; ++r) {
         if (lambda_out) { lambda_out[2 * r] = h->rio_h[r].lam[0]; lambda_out[2 * r + 1] = h->rio_h[r].lam[1]; }
@@ -1167,8 +1182,25 @@ int nd_relax_constrained(nd_handle *h, void *m, const double *X, double tol, int
         if (e) return e;
     }
     if (int e = stage_out(h, m, md, st)) return e;
+    if (status & ND_DEV_TIMEOUT)
+        return fail(ND_ERR_TIMEOUT, "a bounded device-side wait expired in the relaxation: its states are not valid");
     if (rc) g_err = "relaxation did not converge within max_iter in at least one replica";
     return rc;
+}
+
+extern "C" {
+
+int nd_relax_constrained(nd_handle *h, void *m, const double *X, double tol, int max_iter, double *U_out,
+                         double *lambda_out, int *iters_out, void *stream)
+{
+    return relax_constrained(h, m, X, tol, max_iter, U_out, lambda_out, iters_out, stream, false);
+}
+
+int nd_selftest_relax_timeout(nd_handle *h, void *m, const double *X, void *stream)
+{
+    if (int rc = check_handle(h)) return rc;
+    if (!relax_cluster_nc(h, h->classes[0])) return fail(ND_ERR_ARG, "the first size class does not relax on clusters");
+    return relax_constrained(h, m, X, 1e-6, 4, nullptr, nullptr, nullptr, stream, true);
 }
 
 int nd_relax_sweep_grad(nd_handle *h, void *m, const void *grad, const double *X, double *lambda, double tol,
@@ -1294,8 +1326,10 @@ int nd_check_status(nd_handle *h, void *stream)
     unsigned v = 0;
     ND_CUDA(cudaMemcpy(&v, h->status_d, sizeof(v), cudaMemcpyDeviceToHost));
     ND_CUDA(cudaMemset(h->status_d, 0, sizeof(v)));
+    v |= h->status_seen;
+    h->status_seen = 0;
     if (v & ND_DEV_ORDER) return fail(ND_ERR_ARG, "calls on one handle overlapped: their states are not valid");
-    if (v & ND_DEV_TIMEOUT) return fail(ND_ERR_TIMEOUT, "a bounded device-side wait expired (replica hand-over)");
+    if (v & ND_DEV_TIMEOUT) return fail(ND_ERR_TIMEOUT, "a bounded device-side wait expired (replica hand-over or exchange in a cluster)");
     if (v & ND_DEV_NAN) return fail(ND_ERR_NAN, "non-finite values in the state");
     return ND_OK;
 }

@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
                 const int k = atomicAdd(ticket, 1), rep = work[k % rx.nwork], turn = k / rx.nwork;
                 if ((long long)turn * rx.quantum >= rx.max_iter) break;
                 bool ok = false;
-                for (int it = 0; it < (1 << 22) && !ok; ++it) {
+                for (int it = 0; it < wait_polls && !ok; ++it) {
                     ok = atomicAdd(flags + rep, 0) >= turn;
                     if (!ok) __nanosleep(256);
                 }

@@ -39,3 +39,21 @@ def test_error_in_a_later_class_leaves_the_stream_ordered():
     ref = start.clone()
     one.relax(ref, X[:1], tol=1e-300, max_iter=5000)
     assert torch.equal(at_end, ref)
+
+
+@pytest.mark.parametrize("R,prec,B", [(30e-9, nd.ND_FP32, 3), (30e-9, nd.ND_FP32, 20), (60e-9, nd.ND_FP32, 2), (30e-9, nd.ND_FP64, 2)])
+def test_expired_wait_of_a_relaxation_is_reported_as_one(R, prec, B):
+    """Turns that never come: the call says so, nd_check_status once more, no
+    state is touched, and the same handle relaxes normally afterwards."""
+    h = Nanodisk([Disk(R, 0.2 * R)], [B], prec)
+    m, X = h.empty_device(), np.zeros((B, 2))
+    h.init_vortex(m, np.full((B, 2), 1e-9))
+    before = m.clone()
+    assert nd.nd_check_status(h.h) == nd.ND_OK
+    assert nd.nd_selftest_relax_timeout(h.h, m, X) == nd.ND_ERR_TIMEOUT
+    assert torch.equal(m, before)
+    assert nd.nd_check_status(h.h) == nd.ND_ERR_TIMEOUT
+    assert nd.nd_check_status(h.h) == nd.ND_OK
+    rc, U, lam, it = h.relax(m, X, tol=1e-300, max_iter=3)
+    assert rc == nd.ND_ERR_NOT_CONVERGED and np.all(it == 3) and not torch.equal(m, before)
+    assert nd.nd_check_status(h.h) == nd.ND_OK
