@@ -185,6 +185,17 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity)
 // exchange folded into the FFT, whose rounding is relative to |b| ~ 4, the
 // residual of an FP32 sweep carried noise of ~5e-7 and replicas stopped up to
 // ten sweeps from where FP64 arithmetic stops.
+//
+// Above P = 128 in FP32 (WIDE) more replicas relax in grid-wide passes, which add
+// their CTAs' sums, take the Newton step and hold the multipliers in FP64.  Here
+// the warps' sums are added in pairs, at most ten FP32 additions deep (there
+// twelve), and the rest is computed and held in pairs of floats (Two, some 46
+// bits): FP64 issues a warp instruction in 64-76 cycles, and this is a chain that
+// every CTA waits for.  All of it in FP64 cost 0.5-0.8 us of a sweep of 13.8
+// (R = 100 nm), this 0.3 (0.15 of 11.8 at 70 nm, 0.2 of 14.5 at 128 nm).
+// Multipliers of R = 70, 100 and 128 nm after 400 sweeps, against FP64: 2.7e-8,
+// 3.5e-8 and 2.9e-8 off, as with FP64 in this place; grid-wide 1.4e-7, 2.3e-7,
+// 1.6e-7; with FP32 in this place 1.2e-7, 4.8e-8, 3.2e-8.
 struct ClusterRelax {
     RelaxIO *rio;
     const double *twP64;   // exp(-2 pi i k / P), FP64
@@ -211,7 +222,7 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     constexpr int G = Gm::G, R1 = Gm::R1, RS = SpecGeom<P>::RS, KH = CG::KH, NT = CG::NT, NGRP = CG::NGRP;
     constexpr int SPC = CG::SPC, SW = CG::SW, NTAB = CG::NTAB;
     static_assert(MODE == M_RELAX ? SEG : (MODE == M_FIELD ? !SEG : true), "turns or one launch per replica");
-    constexpr bool RELAX = MODE == M_RELAX;
+    constexpr bool RELAX = MODE == M_RELAX, WIDE = RELAX && sizeof(T) == 4 && P > 128;
     cgc::cluster_group cluster = cgc::this_cluster();
     const int rank = (int)cluster.block_rank();
     extern __shared__ __align__(16) unsigned char smem[];
@@ -383,6 +394,7 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     const uint32_t bytes_col = (uint32_t)(3 * (D - nloc) * SPC * sizeof(cplx<T>));
     const uint32_t bytes_row = (uint32_t)(3 * nloc * (P / 2 + 1 - SPC - (rank == 0 ? 1 : 0)) * sizeof(cplx<T>));
     T relX = T(0), relY = T(0);
+    Two lam2 = {0.0f, 0.0f};   // WIDE: multiplier tid of threads 0 and 1
     if constexpr (RELAX) {
         const RelaxIO *io = rx.rio + seg.rep;
         relX = (T)io->X[0];
@@ -391,6 +403,11 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
             lam_s[0] = (T)__ldcg(&io->lam[0]);
             lam_s[1] = (T)__ldcg(&io->lam[1]);
             conv_s = 0;
+        }
+        if (WIDE && tid < 2) {
+            const double l = __ldcg(&io->lam[tid]);
+            lam2.hi = (float)l;
+            lam2.lo = (float)(l - (double)lam2.hi);
         }
     }
     __syncthreads();   // the state, the kernel's entries and the cell range are in place
@@ -665,9 +682,20 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
                 if (tid < 6 * NC) {   // value v of this CTA to CTA q
                     const int q = tid / 6, v = tid - 6 * q;
                     T t = (&racc[0].C0)[v];
-                    for (int w = 1; w < NT / 32; ++w) {
-                        const T u = (&racc[w].C0)[v];
-                        t = v == 5 ? max(t, u) : t + u;
+                    if constexpr (WIDE) {
+                        T u[NT / 32];
+#pragma unroll
+                        for (int w = 0; w < NT / 32; ++w) u[w] = (&racc[w].C0)[v];
+#pragma unroll
+                        for (int o = 1; o < NT / 32; o *= 2)
+#pragma unroll
+                            for (int w = 0; w < NT / 32; w += 2 * o) u[w] = v == 5 ? max(u[w], u[w + o]) : u[w] + u[w + o];
+                        t = u[0];
+                    } else {
+                        for (int w = 1; w < NT / 32; ++w) {
+                            const T u = (&racc[w].C0)[v];
+                            t = v == 5 ? max(t, u) : t + u;
+                        }
                     }
                     if (q == rank) rp[q][v] = t;
                     else st_async(cluster_addr(smem_addr(&rp[rank][v]), q), t, cluster_addr(mb_red, q));
@@ -678,6 +706,45 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
                         bailed = true;
                         atomicOr(status, ND_DEV_TIMEOUT);
                     }
+                    if constexpr (WIDE) {
+                        // lanes 4v..4v+3 add value v's partial sums
+                        const int v = min(tid >> 2, 5), q0 = tid & 3;
+                        Two t = {rp[q0][v], 0.0f};
+                        T res = rp[q0][5];
+#pragma unroll
+                        for (int q = q0 + 4; q < q0 + NC; q += 4) {
+                            t.lo += two_sum(t.hi, rp[q][v]);
+                            res = max(res, rp[q][5]);
+                        }
+#pragma unroll
+                        for (int o = 1; o < 4; o *= 2) {
+                            const float h = __shfl_xor_sync(0xffffffffu, t.hi, o), l = __shfl_xor_sync(0xffffffffu, t.lo, o);
+                            t.lo += l + two_sum(t.hi, h);
+                            res = max(res, __shfl_xor_sync(0xffffffffu, res, o));
+                        }
+                        auto sum = [&](int k) {
+                            return Two{__shfl_sync(0xffffffffu, t.hi, 4 * k), __shfl_sync(0xffffffffu, t.lo, 4 * k)};
+                        };
+                        const Two C0 = sum(0), C1 = sum(1), J00 = sum(2), J01 = sum(3), J11 = sum(4);
+                        // lanes 0 and 1 a numerator each, lane 2 the determinant
+                        const Two n = two_det(tid == 0 ? J11 : J00, tid == 0 ? C0 : tid == 1 ? C1 : J11, J01,
+                                              tid == 0 ? C1 : tid == 1 ? C0 : J01);
+                        const float dh = __shfl_sync(0xffffffffu, n.hi, 2), dl = __shfl_sync(0xffffffffu, n.lo, 2);
+                        if (tid < 2) {   // a multiplier each
+                            res_last = res;
+                            if (res < (T)rx.tol) {
+                                conv_s = 1;
+                            } else {
+                                const float rd = 1.0f / dh, q = n.hi * rd;
+                                const float q2 = (fm(-q, dh, n.hi) + fm(-q, dl, n.lo)) * rd;
+                                if (dh != 0.0f && isfinite(dh)) {   // lam -= q + q2
+                                    lam2.lo += two_sum(lam2.hi, -q) - q2;
+                                    lam2.lo = two_sum(lam2.hi, lam2.lo);
+                                }
+                                lam_s[tid] = lam2.hi;
+                            }
+                        }
+                    } else {
                     const int v = min(tid, 5);
                     T t = rp[0][v];
                     for (int q = 1; q < NC; ++q) t = v == 5 ? max(t, rp[q][v]) : t + rp[q][v];
@@ -695,6 +762,7 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
                                 lam_s[1] += -fm(J00, C1, -(J01 * C0)) / det;
                             }
                         }
+                    }
                     }
                 }
                 __syncthreads();
@@ -767,11 +835,14 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
         bad |= !finite3(v);
     }
     if (MODE == M_RK4 || MODE == M_HEUN) flag_nan(bad, status);
+    if (WIDE && rank == 0 && tid < 2) __stcg(&rx.rio[seg.rep].lam[tid], (double)lam2.hi + (double)lam2.lo);
     if (RELAX && rank == 0 && tid == 0) {
         RelaxIO *io = rx.rio + seg.rep;
         const int iters = __ldcg(&io->iters) + (int)n;
-        __stcg(&io->lam[0], (double)lam_s[0]);
-        __stcg(&io->lam[1], (double)lam_s[1]);
+        if (!WIDE) {
+            __stcg(&io->lam[0], (double)lam_s[0]);
+            __stcg(&io->lam[1], (double)lam_s[1]);
+        }
         __stcg(&io->resid, (double)res_last);
         __stcg(&io->iters, iters);
         if (conv_s) __stcg(&io->status, 0);

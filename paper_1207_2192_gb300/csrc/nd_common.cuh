@@ -163,6 +163,29 @@ __device__ __forceinline__ double to_double(float x)
 }
 __device__ __forceinline__ double to_double(double x) { return x; }
 
+// a += b; returns the rounding error of that sum, which is a float (Knuth's
+// two-sum; only where the compiler contracts nothing).
+__device__ __forceinline__ float two_sum(float &a, float b)
+{
+    const float s = a + b, z = s - a, e = (a - (s - z)) + (b - z);
+    a = s;
+    return e;
+}
+
+// An unevaluated sum of two floats, and a x - b y of four of them, each product
+// with its rounding error (the fused multiply-add's) and the low parts' share.
+struct Two { float hi, lo; };
+__device__ __forceinline__ Two two_det(Two a, Two x, Two b, Two y)
+{
+    const float p = a.hi * x.hi, q = b.hi * y.hi;
+    const float pl = fm(a.hi, x.lo, fm(a.lo, x.hi, fm(a.hi, x.hi, -p)));
+    const float ql = fm(b.hi, y.lo, fm(b.lo, y.hi, fm(b.hi, y.hi, -q)));
+    Two r = {p, 0.0f};
+    r.lo = two_sum(r.hi, -q) + (pl - ql);
+    r.lo = two_sum(r.hi, r.lo);
+    return r;
+}
+
 // Sums of a0, a1 and a2 over a warp: lanes 0, 8 and 16 return those of a0, a1
 // and a2.  Halving the values a lane carries while their lanes double takes six
 // additions instead of fifteen.

@@ -67,3 +67,22 @@ def test_cluster_sweeps_with_ctas_that_own_no_rows(O, R, prec, B):
     assert nd.nd_check_status(h.h) == nd.ND_OK
     for mm, lam in ends[1:]:
         assert np.array_equal(mm, ends[0][0]) and np.array_equal(lam, ends[0][1])
+
+
+@pytest.mark.parametrize("R,grid3x", [(70e-9, False), (90e-9, True), (120e-9, False)])
+def test_multipliers_above_128_are_held_in_more_than_fp32(O, R, grid3x):
+    """FP32 sweeps above P = 128 hold the multipliers in more bits in every form:
+    on clusters (2 replicas) and in grid-wide passes (24) they are no widened
+    floats and follow the oracle's."""
+    disk, model = Disk(R, 0.1 * R), O.Model(R, 0.1 * R)
+    X = np.array([2.5e-9, 1.0e-9])
+    for B in (2, 24):
+        h = Nanodisk([disk], [B], nd.ND_FP32, grid3x=grid3x)
+        m = h.empty_device()
+        h.init_vortex(m, np.zeros((B, 2)))
+        mm, lm = h.unpack(m)[0], np.zeros(2)
+        rc, U, lam, it = h.relax(m, np.tile(X, (B, 1)), tol=1e-300, max_iter=4)
+        for _ in range(4):
+            mm, lm, _ = model.relax_sweep(mm, X, lm)
+        assert np.all(lam != lam.astype(np.float32))
+        assert np.allclose(lam[0], lm, rtol=100 * TOL[nd.ND_FP32], atol=100 * TOL[nd.ND_FP32] * np.abs(lm).max())
