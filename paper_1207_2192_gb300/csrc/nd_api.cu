@@ -161,6 +161,8 @@ struct nd_handle {
     void *spec = nullptr;                 // spectrum scratch (global path), sized for FP64
     void *stage_in = nullptr, *stage_out = nullptr;   // staging of host buffers
     double *red_d = nullptr;              // [B][2] energies and their thickness derivatives
+    void *energy_spec = nullptr;          // FP64 spectra of a turn of the energies, for handles without spec
+    size_t energy_spec_words = 0;         // its complex words
     double *energy_part = nullptr;        // [B][P/2][2] partial sums of the energies (largest P)
     unsigned *energy_done = nullptr;      // [B] counters of finished partial sums
     double *red_h = nullptr;              // pinned [B * 4]
@@ -848,6 +850,7 @@ void nd_destroy(nd_handle *h)
     cudaFree(h->spec);
     cudaFree(h->stage_in);
     cudaFree(h->stage_out);
+    cudaFree(h->energy_spec);
     cudaFree(h->energy_part);
     cudaFree(h->energy_done);
     delete h;
@@ -994,7 +997,20 @@ int nd_energy(nd_handle *h, const void *m, double *E_out, double *dEdL_out, void
     void *md = nullptr;
     if (int rc = stage_in(h, m, &md, true, st, &h->stage_in)) return rc;
     const int B = (int)h->rep_disk.size();
-    if (int rc = ensure_alloc(&h->spec, sizeof(double) * 2 * h->spec_words)) return rc;
+    // A class takes its turns of as many replicas as a grid has rows and, in a
+    // handle without global-path spectra, as fit in 256 MB (1280 of D = 64: many
+    // waves of small CTAs, so nothing is lost between two turns).
+    if (!h->spec && !h->energy_spec) {
+        size_t words = 0, one = 0;
+        for (auto &c : h->classes) {
+            const size_t w = spec_words(c.P, c.maxD);
+            words = std::max(words, w * c.reps.size());
+            one = std::max(one, w);
+        }
+        words = std::max(one, std::min(words, (size_t)1 << 24));
+        if (int rc = ensure_alloc(&h->energy_spec, sizeof(double) * 2 * words)) return rc;
+        h->energy_spec_words = words;
+    }
     if (!h->energy_part) {
         int maxP = 0;
         for (auto &c : h->classes) maxP = std::max(maxP, c.P);
@@ -1005,18 +1021,23 @@ int nd_energy(nd_handle *h, const void *m, double *E_out, double *dEdL_out, void
     for (auto &c : h->classes) {
         EnergyArgs a;
         a.reps = h->base_d;
-        a.work = c.work_d;
-        a.nwork = (int)c.reps.size();
         a.maxD = c.maxD;
         a.with_dl = dEdL_out ? 1 : 0;
         a.m = md;
-        a.spec = h->spec;
+        a.spec = h->spec ? h->spec : h->energy_spec;
+        a.spec_stride = h->spec ? 0 : (long long)spec_words(c.P, c.maxD);
         a.tw = h->tw64[c.P];
         a.part = h->energy_part;
         a.done = h->energy_done;
         a.out = h->red_d;
         a.stream = st;
-        ND_CUDA(launch_energy(c.P, h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32, a));
+        const int Bc = (int)c.reps.size();
+        const int turn = a.spec_stride ? (int)std::min<size_t>(65535, h->energy_spec_words / a.spec_stride) : 65535;
+        for (int k = 0; k < Bc; k += turn) {
+            a.work = c.work_d + k;
+            a.nwork = std::min(turn, Bc - k);
+            ND_CUDA(launch_energy(c.P, h->prec == ND_FP64 ? ND_PREC_FP64 : ND_PREC_FP32, a));
+        }
     }
     ND_CUDA(cudaMemcpyAsync(h->red_h, h->red_d, sizeof(double) * 2 * B, cudaMemcpyDeviceToHost, st));
     ND_CUDA(cudaStreamSynchronize(st));

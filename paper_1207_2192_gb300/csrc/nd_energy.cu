@@ -34,7 +34,7 @@ constexpr int kRowThreads = 32;   // one warp: the row tasks spread over every s
 template <int P, typename S>
 __global__ void __launch_bounds__(kRowThreads)
     k_energy_rows(const Replica *__restrict__ reps, const int *__restrict__ work, const S *__restrict__ mbase,
-                  cplx<double> *__restrict__ specbase, const cplx<double> *__restrict__ twP)
+                  cplx<double> *__restrict__ specbase, long long spec_stride, const cplx<double> *__restrict__ twP)
 {
     using Gm = FFTGeom<P>;
     constexpr int G = Gm::G, R1 = Gm::R1, RS = SpecGeom<P>::RS, NGRP = groups_per_block<P, kRowThreads>();
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(kRowThreads)
     const int q = blockIdx.x * NGRP + gid.group;
     const bool act = q < nrow;
     const long long cs = (long long)D * RS, ms = (long long)D * r.Dpad;
-    cplx<double> *spec = specbase + r.spec_off, *scr = scratch + gid.group * Gm::SCRATCH;
+    cplx<double> *spec = specbase + (spec_stride ? blockIdx.y * spec_stride : r.spec_off), *scr = scratch + gid.group * Gm::SCRATCH;
     auto row = [&](int c, int y) {
         return MaskedRow<S>{mbase + r.state_off + c * ms + (long long)y * r.Dpad, r.mask + (long long)y * D};
     };
@@ -85,7 +85,7 @@ template <int P> struct EnergyCols {
 template <int P>
 __global__ void __launch_bounds__(96)
     k_energy_cols(const Replica *__restrict__ reps, const int *__restrict__ work, const cplx<double> *__restrict__ specbase,
-                  const cplx<double> *__restrict__ twP, double *__restrict__ part, unsigned *__restrict__ done,
+                  long long spec_stride, const cplx<double> *__restrict__ twP, double *__restrict__ part, unsigned *__restrict__ done,
                   double *__restrict__ out, int with_dl)
 {
     using Gm = FFTGeom<P>;
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(96)
     double e = 0.0, el = 0.0;
     cplx<double> v[R1];
     if (gid.valid) {
-        const cplx<double> *col = specbase + r.spec_off + c * (long long)D * RS;
+        const cplx<double> *col = specbase + (spec_stride ? blockIdx.y * spec_stride : r.spec_off) + c * (long long)D * RS;
         col_load_kind<P, double>(v, const_cast<cplx<double> *>(col), packed, act ? q : 1, D, gid.t, act);
         fft_group<P, -1, FFT_HALF_IN>(v, gid.t, scr, tw, gid.gmask);
         mirror_put<P>(v, scr, gid.t);   // natural order: the packed pair's mirror, the x groups' y spectra
@@ -192,9 +192,9 @@ static cudaError_t launch_p(const EnergyArgs &a)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_energy_cols<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc);
     if (e != cudaSuccess) return e;
     k_energy_rows<P, S><<<dim3((row_pass_tasks<P>(a.maxD) + NGRP - 1) / NGRP, a.nwork), kRowThreads, sr, a.stream>>>(
-        a.reps, a.work, (const S *)a.m, (cplx<double> *)a.spec, (const cplx<double> *)a.tw);
+        a.reps, a.work, (const S *)a.m, (cplx<double> *)a.spec, a.spec_stride, (const cplx<double> *)a.tw);
     k_energy_cols<P><<<dim3(EnergyCols<P>::NBLK, a.nwork), EnergyCols<P>::NT, sc, a.stream>>>(
-        a.reps, a.work, (const cplx<double> *)a.spec, (const cplx<double> *)a.tw, a.part, a.done, a.out, a.with_dl);
+        a.reps, a.work, (const cplx<double> *)a.spec, a.spec_stride, (const cplx<double> *)a.tw, a.part, a.done, a.out, a.with_dl);
     return cudaGetLastError();
 }
 

@@ -72,14 +72,15 @@ size_t cluster_smem(int P, int prec, int D, int Dpad, bool wbuf, int nc);   // (
 int cluster_max_active(int P, int prec, int D, int Dpad, bool wbuf, int nc);  // 0: does not fit
 cudaError_t launch_cluster(int P, int prec, const LaunchArgs &a, int maxD, int maxDpad, int nc);
 cudaError_t launch_global(int P, int prec, const LaunchArgs &a, int maxD);
-// Energies E/J (and, with_dl, d(E/J)/dl) of a class's replicas in FP64 from the
+// Energies E/J (and, with_dl, d(E/J)/dl) of up to 65535 replicas of a class in FP64 from the
 // state m of the given precision (nd_energy.cu): out [replicas][2].
 struct EnergyArgs {
     const Replica *reps = nullptr;
     const int *work = nullptr;
     int nwork = 0, maxD = 0, with_dl = 0;
     const void *m = nullptr;
-    void *spec = nullptr;            // FP64 spectrum scratch (Replica::spec_off)
+    void *spec = nullptr;            // FP64 spectrum scratch
+    long long spec_stride = 0;       // its words from one replica of work to the next (0: at Replica::spec_off)
     const void *tw = nullptr;        // length-P FP64 twiddle table
     double *part = nullptr;          // [replicas][column blocks <= P/2][2] of the class's P
     unsigned *done = nullptr;        // [replicas], zero before the first call
