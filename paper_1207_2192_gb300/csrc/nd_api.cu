@@ -14,6 +14,7 @@
 #include "../../include/nanodisk.h"
 #include "nd_common.cuh"
 #include "nd_kernels.h"
+#include "nd_schedule.h"
 
 using namespace nd;
 
@@ -74,14 +75,11 @@ struct SizeClass {
     size_t smem_main = 0;
     size_t smem_wbuf = 0;      // fused Heun with the normals kept in shared memory (0: does not fit)
     int plan[2] = {-1, -1};    // stepping plan for RK4 / Heun: -1 default (default_plan), 0..2 fused variant, kPlanGlobal, kPlanCluster
-    // time-sliced schedule, cached per (mode, n_steps)
-    SegmentHost *segs_d = nullptr;
-    int *seg_off_d = nullptr;
-    int seg_mode = -1, seg_ncta = 0;
-    long long seg_nsteps = -1;
-    bool seg_captured = false;            // a graph replays with the cached schedule
-    std::vector<void *> seg_kept;         // schedules of graphs, kept until the handle goes
-    int *cflags_d = nullptr;   // cluster schedules: hand-over flags of the replicas, the ticket counter, the count of finished ones
+    // time-sliced schedule of the running call: its segments and the slots' ranges
+    // of them, the hand-over words of the handle's replicas, the clusters' ticket
+    // counter and the count of finished replicas
+    Segment *segs_d = nullptr;
+    int *seg_off_d = nullptr, *flags_d = nullptr;
     // resident clusters per (RK4 / Heun, 8 / 16 CTAs) and the plan the default
     // stands for per method: -1 not yet looked up
     mutable int max_clusters[2][2] = {{-1, -1}, {-1, -1}};
@@ -192,7 +190,7 @@ struct nd_handle {
     std::vector<cudaStream_t> side;
     std::vector<cudaEvent_t> join_ev;
     cudaEvent_t fork_ev = nullptr;
-    int *flags_d = nullptr;               // [B] replica hand-over flags of the time-sliced schedule
+    void *sched_d = nullptr;              // the classes' schedules: segs_d, seg_off_d, flags_d
     unsigned *status_d = nullptr;         // device status word (ND_DEV_* bits)
     unsigned *relax_status = nullptr;     // the same of one relaxation (behind status_d and core_done)
     unsigned status_seen = 0;             // bits of relaxations, for nd_check_status
@@ -269,34 +267,6 @@ static void fill_reps(nd_handle *h, double dt_seconds, const double *Tk, const u
         R.dsched = d.sched64;
         R.nsched = d.nsched;
     }
-}
-
-// Time-sliced schedule for more replicas than resident CTAs: the class's
-// replica-steps (B_c x n) are cut into ncta equal, contiguous ranges; CTA i
-// runs the start of the replica it shares with CTA i+1 first (and flags it),
-// then its whole replicas, then the end of the replica it shares with CTA i-1
-// after waiting for that flag.  Every CTA does the same number of steps.
-static void build_segments(int Bc, long long n, int ncta, std::vector<SegmentHost> &segs, std::vector<int> &off)
-{
-    const long long W = (long long)Bc * n, s = (W + ncta - 1) / ncta;
-    segs.clear();
-    off.assign(ncta + 1, 0);
-    for (int i = 0; i < ncta; ++i) {
-        off[i] = (int)segs.size();
-        const long long start = (long long)i * s, end = std::min(W, start + s);
-        if (start >= end) continue;
-        const int r0 = (int)(start / n), r1 = (int)((end - 1) / n);
-        const long long o0 = start % n, o1 = (end - 1) % n + 1;
-        if (r0 == r1) {
-            segs.push_back({r0, o0 > 0 ? 1 : 0, o1 < n ? 1 : 0, 0, o0, o1 - o0});
-            continue;
-        }
-        if (o1 < n) segs.push_back({r1, 0, 1, 0, 0, o1});             // start of the replica continued by CTA i+1
-        for (int r = (o0 > 0 ? r0 + 1 : r0); r < r1; ++r) segs.push_back({r, 0, 0, 0, 0, n});
-        if (o1 == n) segs.push_back({r1, 0, 0, 0, 0, n});
-        if (o0 > 0) segs.push_back({r0, 1, 0, 0, o0, n - o0});          // end of the replica started by CTA i-1
-    }
-    off[ncta] = (int)segs.size();
 }
 
 static int ensure_alloc(void **p, size_t bytes)
@@ -397,48 +367,19 @@ static int relax_cluster_nc(const nd_handle *h, const SizeClass &c)
     return plan_cluster_nc(c.alone_plan[1]);
 }
 
-static bool capturing(cudaStream_t st)
+// Sizes of a class's schedule: a call is time-sliced over fewer slots than
+// replicas (the hand-over self-test: one replica over two).
+static size_t seg_words(const SizeClass &c) { return 3 * c.reps.size() + 6; }    // >= nslots * slot_room
+static size_t off_words(const SizeClass &c) { return 2 * c.reps.size() + 4; }    // >= 2 nslots
+static cudaError_t slice(nd_handle *h, const SizeClass &c, int nwork, long long nsteps, int nslots, LaunchArgs &a)
 {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
-}
-
-// The time-sliced schedule of a class's replicas over nslots CTAs or clusters,
-// cached per (mode, n_steps, slots).  One that a graph was captured with stays
-// allocated for its replays when another takes its place.
-static bool segments_cached(const SizeClass &c, int mode, long long nsteps, int nslots)
-{
-    return c.seg_mode == mode && c.seg_nsteps == nsteps && c.seg_ncta == nslots;
-}
-static int class_segments(SizeClass &c, int mode, long long nsteps, int nslots, cudaStream_t st)
-{
-    if (segments_cached(c, mode, nsteps, nslots)) {
-        c.seg_captured |= capturing(st);
-        return ND_OK;
-    }
-    std::vector<SegmentHost> segs;
-    std::vector<int> off;
-    build_segments((int)c.reps.size(), nsteps, nslots, segs, off);
-    for (auto &g : segs) g.rep = c.reps[g.rep];   // segments refer to positions in c.reps
-    if (c.seg_captured) {
-        c.seg_kept.push_back(c.segs_d);
-        c.seg_kept.push_back(c.seg_off_d);
-    } else {
-        cudaFree(c.segs_d);
-        cudaFree(c.seg_off_d);
-    }
-    c.segs_d = nullptr;
-    c.seg_off_d = nullptr;
-    c.seg_mode = -1;
-    c.seg_captured = false;
-    ND_CUDA(cudaMalloc(&c.segs_d, sizeof(SegmentHost) * segs.size()));
-    ND_CUDA(cudaMalloc(&c.seg_off_d, sizeof(int) * off.size()));
-    ND_CUDA(cudaMemcpy(c.segs_d, segs.data(), sizeof(SegmentHost) * segs.size(), cudaMemcpyHostToDevice));
-    ND_CUDA(cudaMemcpy(c.seg_off_d, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice));
-    c.seg_mode = mode;
-    c.seg_nsteps = nsteps;
-    c.seg_ncta = nslots;
-    return ND_OK;
+    const int B = (int)h->rep_disk.size();
+    a.segs = c.segs_d;
+    a.seg_off = c.seg_off_d;
+    a.flags = c.flags_d;
+    a.n_rep = B;
+    a.ncta = nslots;
+    return launch_schedule(c.work_d, nwork, nsteps, nslots, c.segs_d, c.seg_off_d, c.flags_d, B + 2, a.stream);
 }
 
 // CTAs per replica of a field call: clusters where their waves (whole replicas,
@@ -534,21 +475,10 @@ static int run_mode(nd_handle *h, int mode, void *y, void *out, long long nsteps
             a.use_wbuf = mode == M_HEUN ? 1 : 0;
             a.status = h->status_d;
             const int slots = cluster_slots(h, c, prec, mode == M_HEUN, cluster_nc);
-            const int Bc = (int)c.reps.size(), B = (int)h->rep_disk.size();
-            if (Bc > slots && nsteps >= 2 &&
-                ((segments_cached(c, mode, nsteps, slots) && c.cflags_d) || !capturing(st))) {
-                // more replicas than resident clusters: every cluster steps for
-                // the same time instead of in waves of whole replicas (which
-                // they do, bit for bit the same, where a capture forbids the
-                // allocation of a schedule)
-                if (int rc = class_segments(c, mode, nsteps, slots, st)) return rc;
-                if (int rc = ensure_alloc((void **)&c.cflags_d, sizeof(int) * (B + 2))) return rc;
-                ND_CUDA(cudaMemsetAsync(c.cflags_d, 0, sizeof(int) * (B + 2), st));
-                a.segs = c.segs_d;
-                a.seg_off = c.seg_off_d;
-                a.flags = c.cflags_d;
-                a.n_rep = B;
-                a.ncta = slots;
+            if (a.nwork > slots && nsteps >= 2) {
+                // more replicas than resident clusters: every cluster makes the
+                // same number of steps instead of waves of whole replicas
+                ND_CUDA(slice(h, c, a.nwork, nsteps, slots, a));
             }
             ND_CUDA(launch_cluster(c.P, prec, a, c.maxD, c.maxDpad, cluster_nc));
         } else if (fused) {
@@ -566,15 +496,7 @@ static int run_mode(nd_handle *h, int mode, void *y, void *out, long long nsteps
             if (stepping && nsteps >= 2) {
                 const int per_sm = fused_blocks_per_sm(c.P, prec, mode, a.smem, variant);
                 const int ncta = per_sm * h->n_sm;
-                const int Bc = (int)c.reps.size();
-                if (per_sm > 0 && Bc > ncta) {
-                    if (int rc = class_segments(c, mode, nsteps, ncta, st)) return rc;
-                    ND_CUDA(cudaMemsetAsync(h->flags_d, 0, sizeof(int) * h->rep_disk.size(), st));
-                    a.segs = c.segs_d;
-                    a.seg_off = c.seg_off_d;
-                    a.flags = h->flags_d;
-                    a.ncta = ncta;
-                }
+                if (per_sm > 0 && a.nwork > ncta) ND_CUDA(slice(h, c, a.nwork, nsteps, ncta, a));
             }
             ND_CUDA(launch_fused(c.P, prec, a));
         } else {
@@ -771,7 +693,21 @@ int nd_create_disk(const nd_disk_desc *disks, int n_disks, const int *replicas_p
     if ((e = cudaMalloc(&h->aux_i, sizeof(int) * 2 * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = cudaMalloc(&h->acc, h->elt * h->state_elems)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = cudaMalloc(&h->rio_d, sizeof(RelaxIO) * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
-    if ((e = cudaMalloc(&h->flags_d, sizeof(int) * B)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
+    {
+        size_t segs = 0, words = 0;
+        for (auto &c : h->classes) { segs += seg_words(c); words += off_words(c) + B + 2; }
+        if ((e = cudaMalloc(&h->sched_d, sizeof(Segment) * segs + sizeof(int) * words)) != cudaSuccess)
+            return cuda_fail(e, "cudaMalloc");
+        Segment *sp = (Segment *)h->sched_d;
+        int *p = (int *)(sp + segs);
+        for (auto &c : h->classes) {
+            c.segs_d = sp;
+            sp += seg_words(c);
+            c.seg_off_d = p;
+            c.flags_d = p + off_words(c);
+            p = c.flags_d + B + 2;
+        }
+    }
     if ((e = cudaMalloc(&h->status_d, sizeof(unsigned) * (2 + B))) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = cudaMemset(h->status_d, 0, sizeof(unsigned) * (2 + B))) != cudaSuccess) return cuda_fail(e, "cudaMemset");
     h->core_done = h->status_d + 1;
@@ -820,8 +756,8 @@ void nd_destroy(nd_handle *h)
     for (auto st2 : h->side) { cudaStreamSynchronize(st2); cudaStreamDestroy(st2); }
     for (auto e2 : h->join_ev) cudaEventDestroy(e2);
     if (h->fork_ev) cudaEventDestroy(h->fork_ev);
-    for (auto &c : h->classes) { cudaFree(c.work_d); cudaFree(c.segs_d); cudaFree(c.seg_off_d); cudaFree(c.cflags_d); for (void *p : c.seg_kept) cudaFree(p); }
-    cudaFree(h->flags_d);
+    for (auto &c : h->classes) cudaFree(c.work_d);
+    cudaFree(h->sched_d);
     cudaFree(h->status_d);
     for (auto &kv : h->tw64) cudaFree(kv.second);
     for (auto &kv : h->tw32) cudaFree(kv.second);
@@ -1159,14 +1095,13 @@ static int relax_constrained(nd_handle *h, void *m, const double *X, double tol,
         const int nc = relax_cluster_nc(h, c);
         if (nc) {
             const int slots = cluster_slots(h, c, prec, true, nc), Bc = a.nwork;
-            if (int rc = ensure_alloc((void **)&c.cflags_d, sizeof(int) * (B + 2))) return rc;
-            ND_CUDA(cudaMemsetAsync(c.cflags_d, 0, sizeof(int) * (B + 2), st));
+            ND_CUDA(cudaMemsetAsync(c.flags_d, 0, sizeof(int) * (B + 2), st));
             if (starve) {
-                ND_CUDA(cudaMemcpyAsync(c.cflags_d + B, &a.nwork, sizeof(int), cudaMemcpyHostToDevice, st));
+                ND_CUDA(cudaMemcpyAsync(c.flags_d + B, &a.nwork, sizeof(int), cudaMemcpyHostToDevice, st));
                 a.wait_polls = 1 << 14;
             }
             a.status = h->relax_status;
-            a.flags = c.cflags_d;
+            a.flags = c.flags_d;
             a.n_rep = B;
             a.ncta = std::min(Bc, slots);
             a.tw64 = h->tw64[c.P];
@@ -1362,39 +1297,29 @@ int nd_selftest_handover_timeout(nd_handle *h, void *stream)
     if (!c.fused_main || h->prec == ND_FP64)
         return fail(ND_ERR_ARG, "the hand-over self-test needs an on-chip FP32 size class first in the handle");
     cudaStream_t st = (cudaStream_t)stream;
-    // one CTA, one segment of one step that waits for replica c.reps[0]'s flag,
-    // which no segment signals
-    const SegmentHost seg = {c.reps[0], 1, 0, 0, 0, 1};
-    const int off[2] = {0, 1};
-    void *segs_d = nullptr, *off_d = nullptr;
-    ND_CUDA(cudaMalloc(&segs_d, sizeof(seg)));
-    cudaError_t e = cudaMalloc(&off_d, sizeof(off));
-    if (e == cudaSuccess) e = cudaMemcpy(segs_d, &seg, sizeof(seg), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(off_d, off, sizeof(off), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->flags_d, 0, sizeof(int) * h->rep_disk.size(), st);
-    if (e == cudaSuccess) {
+    // one CTA, the second of two slots of one replica's two steps: its segment
+    // waits for the first, which no CTA runs
+    cudaError_t e;
+    {
         LaunchArgs a;
         a.mode = M_HEUN;
         a.reps = h->base_d;
         a.work = c.work_d;
-        a.nwork = (int)c.reps.size();
+        a.nwork = 1;
         a.y = h->acc;     // never touched: the segment gives up before reading any state
         a.acc = h->acc;
         a.tw = h->tw32[c.P];
-        a.nsteps = 1;
+        a.nsteps = 2;
         a.smem = c.smem_main;
         a.stream = st;
         a.status = h->status_d;
-        a.segs = segs_d;
-        a.seg_off = (const int *)off_d;
-        a.flags = h->flags_d;
+        e = slice(h, c, 1, 2, 2, a);
+        a.seg_off += 2;
         a.ncta = 1;
         a.n_sm = h->n_sm;
-        e = launch_fused(c.P, ND_PREC_FP32, a);
+        if (e == cudaSuccess) e = launch_fused(c.P, ND_PREC_FP32, a);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(segs_d);
-    cudaFree(off_d);
     if (e != cudaSuccess) return fail(ND_ERR_CUDA, std::string("hand-over self-test: ") + cudaGetErrorString(e));
     return ND_OK;
 }
@@ -1409,19 +1334,9 @@ int nd_selftest_handover_progress(nd_handle *h, void *m, long long n_steps, doub
     if (!m || !is_device_ptr(m) || n_steps < 2 || !(dt_seconds > 0))
         return fail(ND_ERR_ARG, "the hand-over self-test needs a device state, n_steps >= 2 and dt > 0");
     cudaStream_t st = (cudaStream_t)stream;
-    const int B = (int)h->rep_disk.size();
-    std::vector<SegmentHost> segs;
-    std::vector<int> off;
-    build_segments(1, n_steps, 2, segs, off);
-    for (auto &g : segs) g.rep = c.reps[0];
-    void *segs_d = nullptr, *off_d = nullptr;
-    ND_CUDA(cudaMalloc(&segs_d, sizeof(SegmentHost) * segs.size()));
-    cudaError_t e = cudaMalloc(&off_d, sizeof(int) * off.size());
-    if (e == cudaSuccess) e = cudaMemcpy(segs_d, segs.data(), sizeof(SegmentHost) * segs.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(off_d, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && !c.cflags_d) e = cudaMalloc((void **)&c.cflags_d, sizeof(int) * (B + 2));
-    if (e == cudaSuccess) e = cudaMemsetAsync(c.cflags_d, 0, sizeof(int) * (B + 2), st);
-    if (e == cudaSuccess) {
+    // two slots of one replica, each on a CTA (cluster) of its own
+    cudaError_t e;
+    {
         fill_reps(h, dt_seconds, nullptr, nullptr, 0);
         upload_reps(h, st);
         LaunchArgs a;
@@ -1436,17 +1351,11 @@ int nd_selftest_handover_progress(nd_handle *h, void *m, long long n_steps, doub
         a.smem = c.smem_main;
         a.stream = st;
         a.status = h->status_d;
-        a.segs = segs_d;
-        a.seg_off = (const int *)off_d;
-        a.flags = c.cflags_d;
-        a.n_rep = B;
-        a.ncta = 2;
         a.wait_polls = 1 << 15;
-        e = nc ? launch_cluster(c.P, prec, a, c.maxD, c.maxDpad, nc) : launch_fused(c.P, prec, a);
+        e = slice(h, c, 1, n_steps, 2, a);
+        if (e == cudaSuccess) e = nc ? launch_cluster(c.P, prec, a, c.maxD, c.maxDpad, nc) : launch_fused(c.P, prec, a);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(segs_d);
-    cudaFree(off_d);
     if (e != cudaSuccess) return fail(ND_ERR_CUDA, std::string("hand-over self-test: ") + cudaGetErrorString(e));
     return ND_OK;
 }
@@ -2003,9 +1912,9 @@ int nd_graph_create(nd_handle *h, void *m, int method, long long n_steps, double
               method == ND_METHOD_HEUN ? seed : nullptr, step0);
     e = cudaMemcpy(g->reps, h->reps_h, sizeof(Replica) * B, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return bail(ND_ERR_CUDA, std::string("cudaMemcpy: ") + cudaGetErrorString(e));
-    // one plain run of the launch sequence prepares the cached schedules
-    // (allocations are not allowed inside a capture); it works on a scratch
-    // copy so the caller's state is untouched
+    // one plain run of the launch sequence loads the kernels and looks up the
+    // plans outside the capture; it works on a scratch copy so the caller's
+    // state is untouched
     {
         void *tmp = nullptr;
         if ((e = cudaMalloc(&tmp, h->elt * h->state_elems)) != cudaSuccess)

@@ -5,6 +5,7 @@
 
 #include "nd_common.cuh"
 #include "nd_kernels.h"
+#include "nd_schedule.h"
 
 namespace nd {
 
@@ -490,6 +491,43 @@ cudaError_t launch_mean_m(int prec, const Replica *reps, const int *work, int nw
 {
     if (prec == ND_PREC_FP64) k_mean_m<double><<<nwork, 256, 0, st>>>(reps, work, (const double *)y, out);
     else k_mean_m<float><<<nwork, 256, 0, st>>>(reps, work, (const float *)y, out);
+    return cudaGetLastError();
+}
+
+// -------------------------------------------------------------- schedule
+
+// The time-sliced schedule of a call, written by the GPU in the place of the
+// memset of the hand-over words: a call needs no upload and keeps nothing,
+// whatever its method and length.  (As tables built by the host and cached per
+// class, a change of either cost two allocations, two frees and two blocking
+// copies: RK4 and Heun of two steps in turn, 16 x R = 60 nm, 208 -> 167 us a pair,
+// 10 x R = 100 nm 298 -> 258; the first Heun call of a new handle 117 -> 93 and
+// 149 -> 123.  With the closed form in the stepping kernel itself its registers
+// spill: 256 x R = 50 nm, 50 RK4 steps 6.48 -> 6.63 ms.)
+__global__ void __launch_bounds__(256) k_schedule(const int *work, int nwork, long long n, int nslots, long long share,
+                                                  int room, Segment *segs, int *seg_off, int *flags, int nflags)
+{
+    const int i = blockIdx.x * 256 + threadIdx.x, slot = i / room, k = i - slot * room;
+    for (int f = i; f < nflags; f += gridDim.x * 256) flags[f] = 0;
+    if (slot >= nslots) return;
+    Segment g;
+    const int count = slot_segment(nwork, n, share, slot, k, g);
+    if (k < count) {
+        g.rep = work[g.pos];
+        segs[i] = g;
+    }
+    if (k == 0) {
+        seg_off[2 * slot] = i;
+        seg_off[2 * slot + 1] = i + count;
+    }
+}
+
+cudaError_t launch_schedule(const int *work, int nwork, long long n, int nslots, Segment *segs, int *seg_off, int *flags,
+                            int nflags, cudaStream_t st)
+{
+    const int room = slot_room(nwork, nslots);
+    k_schedule<<<(nslots * room + 255) / 256, 256, 0, st>>>(work, nwork, n, nslots, slot_share(nwork, n, nslots), room,
+                                                          segs, seg_off, flags, nflags);
     return cudaGetLastError();
 }
 

@@ -209,7 +209,7 @@ struct ClusterRelax {
 // (more replicas than clusters fit on the GPU), a time-sliced schedule: the cluster
 // with ticket i (tickets count the clusters in the order they start, so every
 // cluster that another one waits for is already running) runs the segments
-// segs[seg_off[i] .. seg_off[i+1]), passing replicas on through flags.
+// segs[seg_off[2i] .. seg_off[2i+1]), passing replicas on through flags.
 template <int P, typename T, int MODE, int NC, bool SEG>
 __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     k_cluster(const Replica *__restrict__ reps, const int *__restrict__ work, T *__restrict__ ybase, T *__restrict__ outbase,
@@ -260,8 +260,8 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
     // a ticket beyond the schedule: such a cluster has nothing to run.
     const bool beyond = SEG && !RELAX && slot >= (int)(gridDim.x / NC);
     if (beyond && rank == 0 && tid == 0) atomicOr(status, ND_DEV_ORDER);
-    const int sg_begin = SEG && !RELAX && !beyond ? seg_off[slot] : 0;
-    const int sg_end = RELAX ? 0x7fffffff : beyond ? 0 : SEG ? seg_off[slot + 1] : 1;
+    const int sg_begin = SEG && !RELAX && !beyond ? seg_off[2 * slot] : 0;
+    const int sg_end = RELAX ? 0x7fffffff : beyond ? 0 : SEG ? seg_off[2 * slot + 1] : 1;
     for (int sg = sg_begin; sg < sg_end; ++sg) {
     Segment seg;
     if constexpr (RELAX) {
@@ -896,7 +896,7 @@ static cudaError_t launch_cluster_t(const LaunchArgs &a, int maxD, int maxDpad)
     const ClusterRelax rx = {a.rio, (const double *)a.tw64, a.eta, a.tol, a.rc2, a.max_iter, a.quantum, a.nwork,
                              a.flags ? a.flags + a.n_rep + 1 : nullptr};
     return cudaLaunchKernelEx(&cfg, k_cluster<P, T, MODE, NC, SEG>, a.reps, a.work, (T *)a.y, (T *)a.out,
-                              (const cplx<T> *)a.tw, a.nsteps, a.step_base, a.use_wbuf, a.status, reinterpret_cast<const Segment *>(a.segs),
+                              (const cplx<T> *)a.tw, a.nsteps, a.step_base, a.use_wbuf, a.status, a.segs,
                               a.seg_off, a.flags, a.flags ? a.flags + a.n_rep : nullptr, a.wait_polls, rx);
 }
 

@@ -3,8 +3,6 @@
 
 namespace nd {
 
-static_assert(sizeof(Segment) == sizeof(SegmentHost), "segment layout");
-
 // Cluster plans: NC = 8 CTAs for every on-chip size, NC = 16 for P >= 32
 // (where the P/2 column slots split over 16 CTAs).
 #define ND_CLUSTER_CASES(X)      \

@@ -16,6 +16,7 @@
 #pragma once
 #include "nd_kernels.h"
 #include "nd_phases.cuh"
+#include "nd_schedule.h"
 
 namespace nd {
 
@@ -207,16 +208,6 @@ __host__ __device__ __forceinline__ size_t fused_smem_bytes(int D, int Dpad, int
     return tw + spec + scr + ms + w;
 }
 
-// A piece of one replica's trajectory run by one CTA (time-sliced schedule).
-struct Segment {
-    int rep;                 // replica index
-    int wait;                // wait until flags[rep] is kHandedOver before starting
-    int signal;              // set flags[rep] to kHandedOver when done
-    int pad;
-    long long step_begin;    // first time step (relative to the call's step0)
-    long long nsteps;
-};
-
 // The hand-over word of a replica: 0, then a count that the signalling segment
 // posts every 64 steps, at last kHandedOver.
 constexpr int kHandedOver = -1;
@@ -345,7 +336,7 @@ __global__ void __launch_bounds__(NT, (FusedMinBlocks<P, NT>::v))
     cplx<T> *tw = reinterpret_cast<cplx<T> *>(smem);
     load_twiddles<P>(tw, twP, tid, NT);
 
-    const int s_begin = segs ? seg_off[blockIdx.x] : 0, s_end = segs ? seg_off[blockIdx.x + 1] : 1;
+    const int s_begin = segs ? seg_off[2 * blockIdx.x] : 0, s_end = segs ? seg_off[2 * blockIdx.x + 1] : 1;
     for (int sg = s_begin; sg < s_end; ++sg) {
         int ridx, wait = 0, signal = 0;
         long long sbeg = 0, nseg = nsteps;
@@ -1187,7 +1178,7 @@ static cudaError_t launch_fused_t(const LaunchArgs &a)
     auto kern = k_fused<P, T, MODE, NT>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.smem);
     if (e != cudaSuccess) return e;
-    const Segment *segs = reinterpret_cast<const Segment *>(a.segs);
+    const Segment *segs = a.segs;
     if (!segs) {
         kern<<<a.nwork, NT, a.smem, a.stream>>>(a.reps, a.work, (T *)a.y, (T *)a.acc, (T *)a.out,
                                                 (const cplx<T> *)a.tw, a.nsteps, a.step_base, a.rio, a.eta, a.tol,

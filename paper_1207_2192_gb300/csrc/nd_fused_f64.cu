@@ -3,8 +3,6 @@
 
 namespace nd {
 
-static_assert(sizeof(Segment) == sizeof(SegmentHost), "segment layout");
-
 size_t fused_smem_f64(int P, int D, int Dpad, bool wbuf, int variant)
 {
     const int nt = fused_nt(P, variant);

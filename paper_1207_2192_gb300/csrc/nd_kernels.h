@@ -12,6 +12,7 @@ enum { M_FIELD = 0, M_RK4 = 1, M_HEUN = 2, M_RELAX = 4 };
 
 struct Replica;
 struct RelaxIO;
+struct Segment;
 struct StatsAcc;
 
 struct LaunchArgs {
@@ -39,11 +40,12 @@ struct LaunchArgs {
     double eta = 0.5, tol = 1e-6, rc2 = 0.0;
     int max_iter = 0;
     int quantum = 0;                 // cluster plans: sweeps of one turn of a replica
-    // time-sliced schedule (fused steppers): ncta CTAs run the segments
-    // segs[seg_off[b] .. seg_off[b+1]) and hand replicas over through flags
-    const void *segs = nullptr;
+    // time-sliced schedule (launch_schedule): CTA or cluster b of ncta runs the
+    // segments segs[seg_off[2b] .. seg_off[2b+1]) and hands replicas over through flags
+    const Segment *segs = nullptr;
     const int *seg_off = nullptr;
-    int *flags = nullptr;            // cluster plans: n_rep flags, then the ticket counter
+    int *flags = nullptr;            // n_rep hand-over words; cluster plans: then the ticket counter and the
+                                     // count of finished replicas
     int n_rep = 0;
     int ncta = 0;                    // CTAs (cluster plans: clusters) of the schedule
     int wait_polls = 1 << 22;        // polls without progress after which a hand-over wait gives up
@@ -56,11 +58,6 @@ struct LaunchArgs {
 
 constexpr int kRelaxBlocks = 64;    // global-path relaxation: partial-sum blocks per replica
 
-struct SegmentHost {                 // mirrors Segment in nd_field_impl.cuh
-    int rep, wait, signal, pad;
-    long long step_begin, nsteps;
-};
-
 size_t fused_smem(int P, int prec, int D, int Dpad, bool wbuf = false, int variant = 0);
 int fused_blocks_per_sm(int P, int prec, int mode, size_t smem, int variant = 0);
 int fused_variant_threads(int P, int variant);   // 0 if the variant does not exist
@@ -72,6 +69,10 @@ size_t cluster_smem(int P, int prec, int D, int Dpad, bool wbuf, int nc);   // (
 int cluster_max_active(int P, int prec, int D, int Dpad, bool wbuf, int nc);  // 0: does not fit
 cudaError_t launch_cluster(int P, int prec, const LaunchArgs &a, int maxD, int maxDpad, int nc);
 cudaError_t launch_global(int P, int prec, const LaunchArgs &a, int maxD);
+// The schedule (nd_schedule.h) of nwork replicas, n steps each, over nslots CTAs or
+// clusters: segs [nslots][slot_room], seg_off [nslots][2]; flags[0 .. nflags) zeroed.
+cudaError_t launch_schedule(const int *work, int nwork, long long n, int nslots, Segment *segs, int *seg_off, int *flags,
+                            int nflags, cudaStream_t st);
 // Energies E/J (and, with_dl, d(E/J)/dl) of up to 65535 replicas of a class in FP64 from the
 // state m of the given precision (nd_energy.cu): out [replicas][2].
 struct EnergyArgs {
