@@ -1,7 +1,7 @@
 """Every form of the relaxation sweep against the oracle, sweep by sweep: the
 thread-block cluster (few replicas), the one-CTA kernel and the grid-wide passes
-(more replicas), in both precisions, with disks and with masks that are not
-disks."""
+(more replicas), in both precisions, with disks and (FP64) with masks that are
+not disks."""
 import numpy as np
 import pytest
 
@@ -86,3 +86,28 @@ def test_multipliers_above_128_are_held_in_more_than_fp32(O, R, grid3x):
             mm, lm, _ = model.relax_sweep(mm, X, lm)
         assert np.all(lam != lam.astype(np.float32))
         assert np.allclose(lam[0], lm, rtol=100 * TOL[nd.ND_FP32], atol=100 * TOL[nd.ND_FP32] * np.abs(lm).max())
+
+
+FORMS = [
+    # one CTA per replica (its threads), grid-wide passes (0), clusters of 8 and 16 CTAs
+    (7e-9, nd.ND_FP32, 3, 128), (15e-9, nd.ND_FP32, 65, 256), (30e-9, nd.ND_FP32, 65, 384), (61e-9, nd.ND_FP32, 65, 512),
+    (15e-9, nd.ND_FP64, 65, 256), (30e-9, nd.ND_FP64, 65, 384),
+    (70e-9, nd.ND_FP32, 65, 0), (37e-9, nd.ND_FP64, 65, 0), (66e-9, nd.ND_FP64, 3, 0),
+    (15e-9, nd.ND_FP32, 3, 16 * 256), (30e-9, nd.ND_FP32, 3, 8 * 256), (61e-9, nd.ND_FP32, 3, 16 * 256),
+    (61e-9, nd.ND_FP32, 17, 8 * 256), (70e-9, nd.ND_FP32, 3, 16 * 512), (7e-9, nd.ND_FP64, 3, 8 * 256),
+    (30e-9, nd.ND_FP64, 17, 8 * 256), (37e-9, nd.ND_FP64, 3, 16 * 256)]
+
+
+@pytest.mark.parametrize("R,prec,B,threads", FORMS)
+def test_every_form_of_the_sweep_matches_the_oracle(O, R, prec, B, threads):
+    h, m, X = sweeps_against_oracle(O, R, prec, B, False, 3)
+    assert nd.nd_plan_info(h.h, 0)["threads_heun"] == threads   # the form that ran
+
+
+@pytest.mark.parametrize("R,prec,B,threads", [f for f in FORMS if f[1] == nd.ND_FP64])
+def test_every_form_of_the_sweep_follows_masks_that_are_not_disks(O, R, prec, B, threads):
+    """In FP64: a cell without neighbours inside the mask has a field of a
+    hundredth of the others', whose direction FP32 transforms do not fix to the
+    tolerance (their error is relative to the largest field)."""
+    h, m, X = sweeps_against_oracle(O, R, prec, B, True, 3)
+    assert nd.nd_plan_info(h.h, 0)["threads_heun"] == threads
