@@ -35,7 +35,7 @@
 // exchange, rows, cells), 4.9 us at P = 128 with FP32 and 16 CTAs; in FP64 the
 // issue of one warp instruction per 64-76 cycles and sub-partition.  One disk of
 // R = 50 nm, 50 Heun steps: 497 us; 16 of R = 60 nm, 50 RK4 steps, time-sliced
-// over 15 clusters of 8: 1.25 ms against 4.42 on one CTA each.
+// over 15 clusters of 8: 1.24 ms against 4.42 on one CTA each.
 #pragma once
 #include <cooperative_groups.h>
 
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(ClusterGeom<P, T, NC>::NT, 1)
         mbar_init(mb_row, 1);
         mbar_init(mb_sum, 1);
         mbar_init(mb_sum + 8, 1);
-        mbar_init(mb_halo, 1);
+        if (RELAX) mbar_init(mb_halo, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (SEG && !RELAX && rank == 0) bcast = atomicAdd(ticket, 1);
     }
