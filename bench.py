@@ -78,8 +78,8 @@ def device_sms(device=0):
 # declarations and is left out).
 KERNEL_SOURCES = {
     "batched_heun": ["nd_fused_f32.cu", "nd_cluster_f32.cu", "nd_cluster.cuh", "nd_field_impl.cuh", "nd_phases.cuh", "nd_fft.cuh",
-                     "nd_common.cuh"],
-    "large_disk": ["nd_glob_f32.cu", "nd_field_impl.cuh", "nd_phases.cuh", "nd_fft.cuh", "nd_common.cuh"],
+                     "nd_common.cuh", "nd_schedule.h"],
+    "large_disk": ["nd_glob_f32.cu", "nd_field_impl.cuh", "nd_phases.cuh", "nd_fft.cuh", "nd_common.cuh", "nd_schedule.h"],
 }
 KERNEL_SOURCES["plain"] = KERNEL_SOURCES["batched_heun"]
 

@@ -298,6 +298,12 @@ static bool cluster_plan_fits(const nd_handle *h, const SizeClass &c, int prec, 
 // per CTA or cluster): the one-CTA kernel (P >= 192, and FP64 above 64: the
 // global path with up to 16 replicas), a cluster of 8 and of 16 CTAs.
 // Measured at D = 7, 14, 30, 50 (FP64 the same), 81 and 100; 0: no such plan.
+// The global path's at P = 192 and 256 are from before its column pass took one
+// launch; now it takes 22.0 and 18.9 with 12 replicas, where sliced clusters take
+// 19.2 and 20.2.  So with 11 to 15 replicas at P = 256, and 15 or 16 at 192, the
+// clusters that the table picks step slower, by up to 13%; their relaxations,
+// which follow the same line, are faster (a sweep with 15 replicas 31.5 us, in
+// grid-wide passes with 16 42.4; at P = 192 with 18 35.4, with 20 41.0).
 struct EvalTime { int P; float one, c8, c16; };
 static const EvalTime kEval32[] = {{16, 3.6f, 0, 0},        {32, 5.1f, 4.6f, 4.4f}, {64, 7.0f, 4.0f, 4.0f},
                                    {128, 20.5f, 6.1f, 5.3f}, {192, 30.f, 0, 10.2f},  {256, 28.f, 0, 11.5f}};
@@ -316,11 +322,15 @@ static const EvalTime *eval_time(int prec, int P)
 // the replicas time-sliced over the clusters the GPU holds (about 15 of 8
 // CTAs, 7 of 16; 8% for the hand-overs), cost less than one round of the
 // one-CTA kernel: up to 7 replicas 16 CTAs at P = 128 (5.3 against 20.5 us
-// per evaluation), up to 47 eight (6.1 us per 15 replicas); at P = 64 up to
-// 24 (4.0 against 7.0 us).  Every plan of a size rounds alike (at P = 128 all
-// but the global path), so the choice changes no trajectory.  The classes of
-// one handle step side by side: they take clusters only if all of them fit
-// on the GPU together.
+// per evaluation), up to 46 eight (6.1 us per 15 replicas); at P = 64 up to
+// 24 (4.0 against 7.0 us).  Every plan of a size rounds alike, so the choice
+// changes no trajectory.  The classes of one handle step side by side: they take
+// clusters only if the SMs of all of them add up to no more than the GPU's.
+// Clusters of 8 and of 16 CTAs do not pack that well (15 of the ones, 7 of the
+// others), so one class may wait for another's SMs, but no mix that the sum
+// admits was measured slower than one CTA each (Heun, us per evaluation): 15 of
+// P = 64 with 2 of P = 32 4.7 against 6.5, 8 with 5 4.6 / 6.3, 10 of P = 128
+// with 4 of P = 256 16.3 / 24.1.
 static int default_plan(const nd_handle *h, const SizeClass &c0, int mode)
 {
     const int slot = mode == M_RK4 ? 0 : 1;
