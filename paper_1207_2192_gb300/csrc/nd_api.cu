@@ -1718,7 +1718,7 @@ static int tune_items(std::vector<TuneItem> &items, double dt, long long n_steps
             for (int cand : cands) {
                 c.plan[it.slot] = cand;
                 const int only = whole ? -1 : ci;
-                rc = tune_run(items, dt, n_steps, st0, fork, joins, only);   // warm-up, builds schedules
+                rc = tune_run(items, dt, n_steps, st0, fork, joins, only);   // warm-up
                 if (rc) break;
                 float ms = 1e30f;
                 for (int rep = 0; rep < 3 && rc == ND_OK; ++rep) {
